@@ -17,8 +17,9 @@ constexpr uint32_t kErrBadTree = 2u;         // the hierarchy failed a consisten
 constexpr uint32_t kErrBadHitList = 4u;      // a saved hit list held an index outside the scene
 
 // Traversal stack depth. Karras trees over 30-bit keys with index tie-breaks
-// are at most 30 + 31 levels deep; the stack holds deferred siblings only.
-constexpr int kStackSize = 64;
+// are at most 30 + 31 levels deep; the stack holds deferred siblings only (64
+// of them, and room for the up to three a node adds at once).
+constexpr int kStackSize = 67;
 
 // Child id encoding in a node: >= 0 internal node, < 0 leaf (~m, m = Morton
 // index of the surfel), kNoChild = absent.

@@ -37,7 +37,7 @@ constexpr int kPrefH = IRGS_RELIGHT_PREF_H, kPrefW = IRGS_RELIGHT_PREF_W;
 constexpr int kLutN = IRGS_RELIGHT_LUT_N;
 constexpr int kLutSamples = 1024;
 constexpr int kReduceThreads = 256;
-constexpr int kRelightThreads = 128;
+constexpr int kRelightThreads = kTraceThreads;
 
 // Centre direction of texel (row, col) of an h x w equirect map.
 __device__ __forceinline__ f3 texel_dir(int h, int w, int row, int col) {
@@ -331,7 +331,6 @@ __device__ __forceinline__ bool relight_dir(const EnvMaps& M, int64_t p, int s, 
 
 // One warp per point; lanes take samples s = lane, lane + 32, ...; the traced
 // channels are [albedo (3), roughness, normal (3)].
-template <int K>
 __global__ void __launch_bounds__(kRelightThreads) k_relight(SceneView S, EnvMaps M, const float* __restrict__ xg,
                                                              const float* __restrict__ ng,
                                                              const float* __restrict__ ag,
@@ -339,19 +338,19 @@ __global__ void __launch_bounds__(kRelightThreads) k_relight(SceneView S, EnvMap
                                                              const float* __restrict__ wog, int64_t Pn, int Sn,
                                                              uint64_t seed, TraceParams TP, float* __restrict__ rgb,
                                                              float* __restrict__ vis, float* __restrict__ ind) {
-    static_assert(kRelightThreads == trace_threads<K>(), "k-buffer slots are laid out per block thread");
     const int lane = threadIdx.x & 31;
     const int64_t p = blockIdx.x * (int64_t)(kRelightThreads / 32) + (threadIdx.x >> 5);
     if (p >= Pn) return;
     const f3 x = ld3r(xg, p), a = ld3r(ag, p);
     const ShadeFrame F = shade_frame(ld3r(ng, p), ld3r(wog, p), rg[p]);
     float acc[7] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};   // rgb, V, L_ind
-    for (int s = lane; s < Sn; s += 32) {
-        f3 w;
-        float pdf;
-        if (!relight_dir(M, p, s, Sn, seed, w, pdf)) continue;
-        MarchState<K, 7> st;
-        const bool ok = march_forward<K, 7, false>(S, make_ray(x, w), TP, st, nullptr, 0, true);
+    for (int s0 = 0; s0 < Sn; s0 += 32) {
+        f3 w = mk3(0.f, 0.f, 1.f);
+        float pdf = 0.f;
+        const bool live = s0 + lane < Sn && relight_dir(M, p, s0 + lane, Sn, seed, w, pdf);
+        MarchState<7> st;
+        const bool ok = march_forward<7, false>(S, make_ray(x, w), TP, st, nullptr, 0, live, warp_scratch<false>());
+        if (!live) continue;
         if (!ok) atomicOr(S.status, kErrStackOverflow);
         relight_sample(M, F, a, w, pdf, st.C, st.T, acc);
     }
@@ -376,21 +375,21 @@ __global__ void k_relight_gen(EnvMaps M, const float* __restrict__ xg, int64_t p
     val[i] = (int32_t)i;
 }
 
-template <int K>
 __global__ void __launch_bounds__(kRelightThreads, 6) k_relight_trace(SceneView S, TraceParams P,
                                                                       const float* __restrict__ xg, int64_t p0,
                                                                       int Sn, const float4* __restrict__ dir,
                                                                       const int32_t* __restrict__ order,
                                                                       int64_t rays, float4* __restrict__ res) {
-    static_assert(kRelightThreads == trace_threads<K>(), "k-buffer slots are laid out per block thread");
     const int64_t j = blockIdx.x * (int64_t)kRelightThreads + threadIdx.x;
-    if (j >= rays) return;
-    const int64_t i = order[j];
+    const bool there = j < rays;
+    const int64_t i = there ? order[j] : 0;
     const float4 d4 = dir[i];
-    MarchState<K, 7> st;
-    if (d4.w > 0.f) {
-        const bool ok = march_forward<K, 7, false>(S, make_ray(ld3r(xg, p0 + i / Sn), mk3(d4.x, d4.y, d4.z)), P,
-                                                   st, nullptr, 0, true);
+    const bool live = there && d4.w > 0.f;
+    MarchState<7> st;
+    const bool ok = march_forward<7, false>(S, make_ray(ld3r(xg, p0 + i / Sn), mk3(d4.x, d4.y, d4.z)), P, st, nullptr,
+                                            0, live, warp_scratch<false>());
+    if (!there) return;
+    if (live) {
         if (!ok) atomicOr(S.status, kErrStackOverflow);
     } else {
 #pragma unroll
@@ -403,39 +402,34 @@ __global__ void __launch_bounds__(kRelightThreads, 6) k_relight_trace(SceneView 
 
 // The same traces in compacted rounds: round 1 on every sorted ray; rays
 // still marching store their state (C[7], D, T, hit count, next key) at
-// their sorted position and are regrouped, in sorted order, for rounds 2
-// and 3; the rest run to completion. Per ray the rounds and their
-// arithmetic are march_forward's (per lane), so the results are the same.
-enum RelightRound { kRelFirst = 0, kRelNext = 1, kRelLast = 2 };
+// their sorted position and are regrouped, in sorted order, into warps that
+// run to completion. Per ray the rounds and their arithmetic are
+// march_forward's, so the results are the same.
+enum RelightRound { kRelFirst = 0, kRelLast = 1 };
 constexpr int kRelightStateF4 = 4;
 
-template <int K, int MODE>
+template <int MODE>
 __global__ void __launch_bounds__(kRelightThreads, 6) k_relight_round(
     SceneView S, TraceParams P, const float* __restrict__ xg, int64_t p0, int Sn, const float4* __restrict__ dir,
     const int32_t* __restrict__ order, int64_t rays, float4* __restrict__ res, const int32_t* __restrict__ list,
     const uint32_t* __restrict__ count, float4* __restrict__ state, uint32_t* __restrict__ flags) {
-    static_assert(kRelightThreads == trace_threads<K>(), "k-buffer slots are laid out per block thread");
     const int64_t t = blockIdx.x * (int64_t)kRelightThreads + threadIdx.x;
     const int64_t n = MODE == kRelFirst ? rays : (int64_t)*count;
-    if (t >= n) return;
-    const int64_t j = MODE == kRelFirst ? t : (int64_t)list[t];
+    if (__all_sync(kFullWarp, t >= n)) return;   // nothing for this warp
+    const bool there = t < n;
+    const int64_t j = !there ? 0 : (MODE == kRelFirst ? t : (int64_t)list[t]);
     const int64_t i = order[j];
     const float4 d4 = dir[i];
-    MarchState<K, 7> st;
+    const bool live = there && d4.w > 0.f;
+    if (MODE == kRelFirst && there && !live) {
+        res[2 * i] = make_float4(0.f, 0.f, 0.f, 0.f);
+        res[2 * i + 1] = make_float4(0.f, 0.f, 0.f, 1.f);
+    }
+    MarchState<7> st;
+    st.init();
     uint64_t last_key = depth_key(P.t_min, 0.f);
     int32_t last_u = INT32_MAX;
-    if (MODE == kRelFirst) {
-#pragma unroll
-        for (int c = 0; c < 7; ++c) st.C[c] = 0.f;
-        st.D = 0.f;
-        st.T = 1.f;
-        st.nh = 0;
-        if (!(d4.w > 0.f)) {
-            res[2 * i] = make_float4(0.f, 0.f, 0.f, 0.f);
-            res[2 * i + 1] = make_float4(0.f, 0.f, 0.f, 1.f);
-            return;
-        }
-    } else {
+    if (MODE != kRelFirst) {
         float w[16];
 #pragma unroll
         for (int q = 0; q < kRelightStateF4; ++q) {
@@ -451,13 +445,15 @@ __global__ void __launch_bounds__(kRelightThreads, 6) k_relight_round(
         last_u = __float_as_int(w[12]);
     }
     const Ray ray = make_ray(ld3r(xg, p0 + i / Sn), mk3(d4.x, d4.y, d4.z));
-    KBuffer<K, trace_threads<K>()> kb;
+    KBuffer<kBufferCap> kb;
     kb.bind();
-    bool ok = true, done = false;
+    float4* scratch = warp_scratch<false>();
+    bool ok = true, done = !live, packet = false;
     do {
-        ok &= collect_round(S, ray, P, last_key, last_u, kb);
-        done = blend_round<K, 7>(S, P, kb, st, nullptr, 0, last_key, last_u);
-    } while (MODE == kRelLast && !done);
+        ok &= collect<false>(S, ray, P, last_key, last_u, st.T, kb, !done, packet, scratch);
+        if (!done) done = blend_round<7>(S, ray, P, kb, st, nullptr, 0, last_key, last_u);
+    } while (MODE == kRelLast && __any_sync(kFullWarp, !done));
+    if (!live) return;
     if (!ok) atomicOr(S.status, kErrStackOverflow);
     if (done) {
         res[2 * i] = make_float4(st.C[0], st.C[1], st.C[2], st.C[3]);
@@ -510,7 +506,6 @@ inline unsigned grid_for(int64_t n, int t) { return (unsigned)((n + t - 1) / t >
 
 constexpr int64_t kRelightChunkRays = int64_t(1) << 26;
 
-template <int K>
 cudaError_t relight_wave(const SceneView& S, const uint32_t* bounds, const EnvMaps& M, const float* x,
                          const float* n, const float* a, const float* r, const float* wo, int64_t P, int Sn,
                          uint64_t seed, const TraceParams& TP, float* rgb, float* vis, float* ind, cudaStream_t st) {
@@ -544,31 +539,20 @@ cudaError_t relight_wave(const SceneView& S, const uint32_t* bounds, const EnvMa
         e = sort_pairs(key, val, ktmp, vtmp, hist, rays, st);
         if (e != cudaSuccess) break;
         if (S.n == 0) {
-            k_relight_trace<K><<<grid_for(rays, kRelightThreads), kRelightThreads, 0, st>>>(S, TP, x, p0, Sn, dir,
-                                                                                          val, rays, res);
+            k_relight_trace<<<grid_for(rays, kRelightThreads), kRelightThreads, 0, st>>>(S, TP, x, p0, Sn, dir, val,
+                                                                                       rays, res);
             count_launches(1);
         } else {
             const unsigned g = grid_for(rays, kRelightThreads);
             e = cudaMemsetAsync(flags, 0, sizeof(uint32_t) * (rays + 1), st);
             if (e != cudaSuccess) break;
-            k_relight_round<K, kRelFirst><<<g, kRelightThreads, 0, st>>>(S, TP, x, p0, Sn, dir, val, rays, res, list,
-                                                                          count, state, flags);
-            count_launches(1);
-            for (int round = 2; round <= 4 && e == cudaSuccess; ++round) {
-                e = flags_to_list(flags, rays, count + 1, list, count, st);
-                if (e != cudaSuccess) break;
-                if (round < 4) {
-                    e = cudaMemsetAsync(flags, 0, sizeof(uint32_t) * (rays + 1), st);
-                    if (e != cudaSuccess) break;
-                    k_relight_round<K, kRelNext><<<g, kRelightThreads, 0, st>>>(S, TP, x, p0, Sn, dir, val, rays, res,
-                                                                                 list, count, state, flags);
-                } else {
-                    k_relight_round<K, kRelLast><<<g, kRelightThreads, 0, st>>>(S, TP, x, p0, Sn, dir, val, rays, res,
-                                                                                 list, count, state, flags);
-                }
-                count_launches(1);
-            }
+            k_relight_round<kRelFirst><<<g, kRelightThreads, 0, st>>>(S, TP, x, p0, Sn, dir, val, rays, res, list,
+                                                                      count, state, flags);
+            e = flags_to_list(flags, rays, count + 1, list, count, st);
             if (e != cudaSuccess) break;
+            k_relight_round<kRelLast><<<g, kRelightThreads, 0, st>>>(S, TP, x, p0, Sn, dir, val, rays, res, list,
+                                                                     count, state, flags);
+            count_launches(2);
         }
         k_relight_shade<<<grid_for(np, kRelightThreads / 32), kRelightThreads, 0, st>>>(M, n, a, r, wo, p0, np, Sn,
                                                                                        dir, res, rgb, vis, ind);
@@ -679,34 +663,17 @@ irgs_status launch_relight(const SceneView& S, const uint32_t* bounds, irgs_envm
     if (P == 0) return IRGS_OK;
     const TraceParams TP = to_params(p);
     const EnvMaps M{m->env, m->irr, m->pref, m->lut, m->row_cdf, m->col_cdf, m->H, m->W};
+    if (p.k != 8 && p.k != 16) return IRGS_ERR_UNSUPPORTED;
     cudaError_t e = cudaSuccess;
     if ((p.flags & IRGS_FLAG_PER_THREAD) != 0u) {
         // fused: a warp per point tracing its own samples
         const int64_t blocks = (P + kRelightThreads / 32 - 1) / (kRelightThreads / 32);
-        switch (p.k) {
-            case 8:
-                k_relight<8><<<(unsigned)blocks, kRelightThreads, 0, st>>>(S, M, x, n, albedo, rough, wo, P,
-                                                                          n_samples, seed, TP, rgb, vis, ind);
-                break;
-            case 16:
-                k_relight<16><<<(unsigned)blocks, kRelightThreads, 0, st>>>(S, M, x, n, albedo, rough, wo, P,
-                                                                           n_samples, seed, TP, rgb, vis, ind);
-                break;
-            default: return IRGS_ERR_UNSUPPORTED;
-        }
+        k_relight<<<(unsigned)blocks, kRelightThreads, 0, st>>>(S, M, x, n, albedo, rough, wo, P, n_samples, seed, TP,
+                                                                rgb, vis, ind);
         count_launches(1);
         e = cudaGetLastError();
     } else {
-        switch (p.k) {
-            case 8:
-                e = relight_wave<8>(S, bounds, M, x, n, albedo, rough, wo, P, n_samples, seed, TP, rgb, vis, ind, st);
-                break;
-            case 16:
-                e = relight_wave<16>(S, bounds, M, x, n, albedo, rough, wo, P, n_samples, seed, TP, rgb, vis, ind,
-                                     st);
-                break;
-            default: return IRGS_ERR_UNSUPPORTED;
-        }
+        e = relight_wave(S, bounds, M, x, n, albedo, rough, wo, P, n_samples, seed, TP, rgb, vis, ind, st);
     }
     if (e == cudaErrorMemoryAllocation) return IRGS_ERR_OOM;
     return e == cudaSuccess ? IRGS_OK : IRGS_ERR_CUDA;

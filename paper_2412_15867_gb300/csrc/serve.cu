@@ -52,7 +52,7 @@ struct irgs_server_s {
 namespace irgs {
 namespace {
 
-constexpr int kServeThreads = 128;
+constexpr int kServeThreads = kTraceThreads;
 constexpr int kServeK = 16;
 constexpr size_t kHeaderBytes = 16;
 
@@ -88,7 +88,6 @@ __global__ void k_camera_rays(irgs_camera c, int64_t first, int64_t count, float
 }
 
 __global__ void __launch_bounds__(kServeThreads) k_serve(ServeArgs A) {
-    static_assert(kServeThreads == trace_threads<kServeK>(), "k-buffer slots are laid out per block thread");
     __shared__ int s_tile;
     const int n_tiles = A.header[1];
     for (;;) {
@@ -115,8 +114,8 @@ __global__ void __launch_bounds__(kServeThreads) k_serve(ServeArgs A) {
                     camera_ray(job.cam, p, o, d);
                 }
                 const Ray ray = make_ray(o, d);
-                MarchState<kServeK, 10> st;
-                const bool ok = march_forward<kServeK, 10, true>(S, ray, P, st, nullptr, 0, live);
+                MarchState<10> st;
+                const bool ok = march_forward<10, true>(S, ray, P, st, nullptr, 0, live, warp_scratch<true>());
                 if (!live) continue;
                 if (!ok) atomicOr(S.status, kErrStackOverflow);
                 if (render) {

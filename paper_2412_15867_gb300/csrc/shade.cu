@@ -32,10 +32,10 @@
 namespace irgs {
 namespace {
 
-constexpr int kShadeThreads = 128;
+constexpr int kShadeThreads = kTraceThreads;
 __device__ __forceinline__ f3 ld3(const float* p, int64_t i) { return mk3(p[3 * i], p[3 * i + 1], p[3 * i + 2]); }
 
-template <int K, bool WARP>
+template <bool PACKET>
 __global__ void __launch_bounds__(kShadeThreads) k_shade(SceneView S, const float* __restrict__ xg,
                                                          const float* __restrict__ ng, const float* __restrict__ ag,
                                                          const float* __restrict__ rg, const float* __restrict__ wog,
@@ -43,13 +43,12 @@ __global__ void __launch_bounds__(kShadeThreads) k_shade(SceneView S, const floa
                                                          int nd, int ns, int mode, uint64_t seed, TraceParams TP,
                                                          float* __restrict__ rgb, float* __restrict__ vis,
                                                          float* __restrict__ ind) {
-    static_assert(kShadeThreads == trace_threads<K>(), "k-buffer slots are laid out per block thread");
     const int lane = threadIdx.x & 31;
     const int64_t p = blockIdx.x * (int64_t)(kShadeThreads / 32) + (threadIdx.x >> 5);
     if (p >= Pn) return;
     ShadeSums o;
-    shade_point_warp<K, WARP>(S, ld3(xg, p), ld3(ng, p), ld3(wog, p), ld3(ag, p), rg[p], (uint64_t)p, nd, ns, mode,
-                              seed, env, H, W, TP, o);
+    shade_point_warp<PACKET>(S, ld3(xg, p), ld3(ng, p), ld3(wog, p), ld3(ag, p), rg[p], (uint64_t)p, nd, ns, mode,
+                             seed, env, H, W, TP, o);
     if (lane == 0) {
         for (int c = 0; c < 3; ++c) rgb[3 * p + c] = o.rgb[c];
         if (vis != nullptr) vis[p] = o.vis;
@@ -58,16 +57,14 @@ __global__ void __launch_bounds__(kShadeThreads) k_shade(SceneView S, const floa
     }
 }
 
-template <int K, bool WARP>
+template <bool PACKET>
 __global__ void __launch_bounds__(kShadeThreads) k_shade_backward(
     SceneView S, const float* __restrict__ xg, const float* __restrict__ ng, const float* __restrict__ ag,
     const float* __restrict__ rg, const float* __restrict__ wog, int64_t Pn, const float* __restrict__ env, int H,
     int W, int nd, int ns, int mode, uint64_t seed, TraceParams TP, const float* __restrict__ g_rgb,
     float* __restrict__ g_albedo, float* __restrict__ g_rough, float* __restrict__ g_env,
     float* __restrict__ acc_rows) {
-    static_assert(kShadeThreads == trace_threads<K>(), "k-buffer slots are laid out per block thread");
-    __shared__ float4 rows_all[kShadeThreads * GradRow<3>::kStride / 4];
-    float* rows = reinterpret_cast<float*>(rows_all) + (threadIdx.x & ~31) * GradRow<3>::kStride;
+    float4* scratch = warp_memory<replay_f4<3, PACKET>()>();
     const int lane = threadIdx.x & 31;
     const int64_t p = blockIdx.x * (int64_t)(kShadeThreads / 32) + (threadIdx.x >> 5);
     if (p >= Pn) return;
@@ -81,15 +78,13 @@ __global__ void __launch_bounds__(kShadeThreads) k_shade_backward(
     bool ok = true;
     for (int base = 0; base < St; base += 32) {
         const ShadeSample d = draw_sample(F, mode, (uint64_t)p, base + lane, St, nd, seed);
-        if (!WARP && !d.valid) continue;
         const Ray ray = make_ray(x, d.wi);
-        MarchState<K, 3> st;
-        ok &= march_forward<K, 3, WARP>(S, ray, TP, st, nullptr, 0, d.valid);
+        MarchState<3> st;
+        ok &= march_forward<3, PACKET>(S, ray, TP, st, nullptr, 0, d.valid, scratch);
         float gL[3] = {0.f, 0.f, 0.f}, gO = 0.f;
         if (d.valid) sample_grad(F, d, mode, nd, ns, St, av, g, st.C, st.T, env, H, W, g_env, ga, gr, gL, gO);
         const bool live = d.valid && st.nh > 0;
-        if (!WARP && !live) continue;
-        ok &= march_backward<K, 3, WARP>(S, ray, TP, live, st.nh, st.C, st.D, st.T, gL, 0.f, gO, acc_rows, rows);
+        ok &= march_backward<3, PACKET>(S, ray, TP, live, st.nh, st.C, st.D, st.T, gL, 0.f, gO, acc_rows, scratch);
     }
     if (!ok) atomicOr(S.status, kErrStackOverflow);
 #pragma unroll
@@ -144,19 +139,10 @@ irgs_status launch_shade_mc(const SceneView& S, const float* x, const float* n, 
     const int mode = shade_mode(p);
     const int64_t blocks = (P + (kShadeThreads / 32) - 1) / (kShadeThreads / 32);
     const bool warp = (p.flags & IRGS_FLAG_WARP) != 0u;
-#define IRGS_SHADE_LAUNCH(KK, WW)                                                                        \
-    k_shade<KK, WW><<<(unsigned)blocks, kShadeThreads, 0, st>>>(S, x, n, albedo, rough, wo, P, env, H, W, \
-                                                               n_diffuse, n_spec, mode, seed, TP, rgb, vis, ind)
-    switch (p.k) {
-        case 8:
-            if (warp) IRGS_SHADE_LAUNCH(8, true); else IRGS_SHADE_LAUNCH(8, false);
-            break;
-        case 16:
-            if (warp) IRGS_SHADE_LAUNCH(16, true); else IRGS_SHADE_LAUNCH(16, false);
-            break;
-        default: return IRGS_ERR_UNSUPPORTED;
-    }
-#undef IRGS_SHADE_LAUNCH
+    if (p.k != 8 && p.k != 16) return IRGS_ERR_UNSUPPORTED;
+    const auto kernel = warp ? k_shade<true> : k_shade<false>;
+    kernel<<<(unsigned)blocks, kShadeThreads, 0, st>>>(S, x, n, albedo, rough, wo, P, env, H, W, n_diffuse, n_spec,
+                                                       mode, seed, TP, rgb, vis, ind);
     count_launches(1);
     return cudaGetLastError() == cudaSuccess ? IRGS_OK : IRGS_ERR_CUDA;
 }
@@ -171,6 +157,7 @@ irgs_status launch_shade_mc_backward(const SceneView& S, const int32_t* perm, co
     const TraceParams TP = to_params(p);
     const int mode = shade_mode(p);
     const bool warp = (p.flags & IRGS_FLAG_WARP) != 0u;
+    if (p.k != 8 && p.k != 16) return IRGS_ERR_UNSUPPORTED;
     constexpr int N = GradRow<3>::N;
     const size_t bytes = sizeof(float) * N * (size_t)(S.n > 0 ? S.n : 1);
     float* acc_rows = nullptr;
@@ -180,20 +167,9 @@ irgs_status launch_shade_mc_backward(const SceneView& S, const int32_t* perm, co
     e = cudaMemsetAsync(acc_rows, 0, bytes, st);
     if (e == cudaSuccess) {
         const int64_t blocks = (P + (kShadeThreads / 32) - 1) / (kShadeThreads / 32);
-#define IRGS_SHADE_BWD(KK, WW)                                                                                     \
-    k_shade_backward<KK, WW><<<(unsigned)blocks, kShadeThreads, 0, st>>>(S, x, n, albedo, rough, wo, P, env, H, W, \
-                                                                        n_diffuse, n_spec, mode, seed, TP, g_rgb,  \
-                                                                        g_albedo, g_rough, g_env, acc_rows)
-        switch (p.k) {
-            case 8:
-                if (warp) IRGS_SHADE_BWD(8, true); else IRGS_SHADE_BWD(8, false);
-                break;
-            case 16:
-                if (warp) IRGS_SHADE_BWD(16, true); else IRGS_SHADE_BWD(16, false);
-                break;
-            default: e = cudaErrorInvalidValue;
-        }
-#undef IRGS_SHADE_BWD
+        const auto kernel = warp ? k_shade_backward<true> : k_shade_backward<false>;
+        kernel<<<(unsigned)blocks, kShadeThreads, 0, st>>>(S, x, n, albedo, rough, wo, P, env, H, W, n_diffuse, n_spec,
+                                                           mode, seed, TP, g_rgb, g_albedo, g_rough, g_env, acc_rows);
         if (e == cudaSuccess) {
             if (S.n > 0)
                 k_grad_scatter<3><<<(unsigned)((S.n + 255) / 256), 256, 0, st>>>(perm, S.n, acc_rows, TP.fc, S.F,
@@ -204,7 +180,6 @@ irgs_status launch_shade_mc_backward(const SceneView& S, const int32_t* perm, co
         }
     }
     const cudaError_t ef = cudaFreeAsync(acc_rows, st);
-    if (e == cudaErrorInvalidValue) return IRGS_ERR_UNSUPPORTED;
     return (e == cudaSuccess && ef == cudaSuccess) ? IRGS_OK : IRGS_ERR_CUDA;
 }
 

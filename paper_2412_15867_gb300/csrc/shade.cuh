@@ -266,10 +266,10 @@ struct ShadeSums {
 };
 
 // All 32 lanes of a warp call this with the same point; every lane returns
-// the point's sums. WARP selects the warp-coherent traversal. With TRACED the
+// the point's sums. PACKET selects the packet traversal. With TRACED the
 // samples' traces were made beforehand: traced[s] = (L_ind, V) of sample s
 // of this point (the same values the march gives), and nothing is traced.
-template <int K, bool WARP, bool TRACED = false>
+template <bool PACKET, bool TRACED = false>
 __device__ __forceinline__ void shade_point_warp(const SceneView& S, f3 x, f3 n_in, f3 wo_in, f3 a, float rough,
                                                  uint64_t p, int nd, int ns, int mode, uint64_t seed,
                                                  const float* __restrict__ env, int H, int W, const TraceParams& TP,
@@ -279,11 +279,11 @@ __device__ __forceinline__ void shade_point_warp(const SceneView& S, f3 x, f3 n_
     const int St = nd + ns;
     float sd[3] = {0.f, 0.f, 0.f}, ss[3] = {0.f, 0.f, 0.f}, si[3] = {0.f, 0.f, 0.f}, sv = 0.f, cnt = 0.f;
     // lane l takes samples l, l + 32, ...; the trip count is the same for the
-    // whole warp so the warp-coherent walk keeps every lane in the loop
+    // whole warp so the walk keeps every lane in the loop
     for (int base = 0; base < St; base += 32) {
         const ShadeSample d = draw_sample(F, mode, p, base + lane, St, nd, seed);
-        if ((TRACED || !WARP) && !d.valid) continue;
-        MarchState<K, 3> st;
+        if (TRACED && !d.valid) continue;
+        MarchState<3> st;
         if (TRACED) {
             const float4 t = __ldg(traced + base + lane);
             st.C[0] = t.x;
@@ -292,7 +292,7 @@ __device__ __forceinline__ void shade_point_warp(const SceneView& S, f3 x, f3 n_
             st.T = t.w;
         } else {
             const Ray ray = make_ray(x, d.wi);
-            const bool ok = march_forward<K, 3, WARP>(S, ray, TP, st, nullptr, 0, d.valid);
+            const bool ok = march_forward<3, PACKET>(S, ray, TP, st, nullptr, 0, d.valid, warp_scratch<PACKET>());
             if (!d.valid) continue;
             if (!ok) atomicOr(S.status, kErrStackOverflow);
         }

@@ -36,7 +36,7 @@
 namespace irgs {
 namespace {
 
-constexpr int kWaveThreads = 128;
+constexpr int kWaveThreads = kTraceThreads;
 constexpr int64_t kWaveChunkRays = int64_t(1) << 26;
 constexpr int kWaveSavedHits = 64;   // 12% of secondary rays blend more than 32 hits, 0.02% more than 64
 constexpr int kWaveReplayBlocks = 1024;   // grid-stride blocks for the few rays whose hit list did not fit
@@ -72,23 +72,22 @@ __global__ void k_wave_gen(const float* __restrict__ xg, const float* __restrict
 // Trace the rays in regrouped order; res[i] = (L_ind, V).
 // With SAVE the blended hit ids (user order, -1 terminated) and the hit
 // counts are kept for the backward.
-template <int K, bool SAVE>
+template <bool SAVE>
 __global__ void __launch_bounds__(kWaveThreads, 6) k_wave_trace(SceneView S, TraceParams P,
                                                                 const float* __restrict__ xg, int64_t p0, int St,
                                                                 const float4* __restrict__ dir,
                                                                 const int32_t* __restrict__ order, int64_t rays,
                                                                 float4* __restrict__ res, int32_t* __restrict__ nh,
                                                                 int32_t* __restrict__ ids, int max_ids) {
-    static_assert(kWaveThreads == trace_threads<K>(), "k-buffer slots are laid out per block thread");
     const int64_t j = blockIdx.x * (int64_t)kWaveThreads + threadIdx.x;
     const int64_t i = j < rays ? order[j] : 0;
     const float4 d4 = dir[i];
     const bool live = j < rays && d4.w != 0.f;
     const int64_t p = p0 + i / St;
     const Ray ray = make_ray(ld3w(xg, p), mk3(d4.x, d4.y, d4.z));
-    MarchState<K, 3> st;
+    MarchState<3> st;
     int32_t* my_ids = (SAVE && live) ? ids + i * (int64_t)max_ids : nullptr;
-    const bool ok = march_forward<K, 3, false>(S, ray, P, st, my_ids, max_ids, live);
+    const bool ok = march_forward<3, false>(S, ray, P, st, my_ids, max_ids, live, warp_scratch<false>());
     if (j >= rays) return;
     if (!live) {   // every sample gets an entry, so no reader sees unwritten scratch
         res[i] = make_float4(0.f, 0.f, 0.f, 0.f);
@@ -105,40 +104,36 @@ __global__ void __launch_bounds__(kWaveThreads, 6) k_wave_trace(SceneView S, Tra
 
 // The same traces in compacted rounds: round 1 on every ray of the order;
 // rays still marching store their state (C, D, T, hit count, next key) at
-// their sorted position and are regrouped, keeping the sorted order, for
-// rounds 2 and 3; the rest run to completion. Per ray the rounds and their
-// arithmetic are march_forward's (per lane), so the results are the same.
-enum WaveRound { kWaveFirst = 0, kWaveNext = 1, kWaveLast = 2 };
+// their sorted position and are regrouped, keeping the sorted order, into
+// warps that run to completion. Per ray the rounds and their arithmetic are
+// march_forward's, so the results are the same.
+enum WaveRound { kWaveFirst = 0, kWaveLast = 1 };
 constexpr int kWaveStateF4 = 3;   // C[3], D, T, hit count, next key (2 words), next user index
 
-template <int K, bool SAVE, int MODE>
+template <bool SAVE, int MODE>
 __global__ void __launch_bounds__(kWaveThreads, 6) k_wave_round(
     SceneView S, TraceParams P, const float* __restrict__ xg, int64_t p0, int St, const float4* __restrict__ dir,
     const int32_t* __restrict__ order, int64_t rays, float4* __restrict__ res, int32_t* __restrict__ nh,
     int32_t* __restrict__ ids, int max_ids, const int32_t* __restrict__ list, const uint32_t* __restrict__ count,
     float4* __restrict__ state, uint32_t* __restrict__ flags) {
-    static_assert(kWaveThreads == trace_threads<K>(), "k-buffer slots are laid out per block thread");
     const int64_t t = blockIdx.x * (int64_t)kWaveThreads + threadIdx.x;
     const int64_t n = MODE == kWaveFirst ? rays : (int64_t)*count;
-    if (t >= n) return;
-    const int64_t j = MODE == kWaveFirst ? t : (int64_t)list[t];
+    if (__all_sync(kFullWarp, t >= n)) return;   // nothing for this warp
+    const bool there = t < n;
+    const int64_t j = !there ? 0 : (MODE == kWaveFirst ? t : (int64_t)list[t]);
     const int64_t i = order[j];
     const float4 d4 = dir[i];
-    if (MODE == kWaveFirst && d4.w == 0.f) {   // every sample gets an entry, so no reader sees unwritten scratch
+    const bool live = there && d4.w != 0.f;
+    if (MODE == kWaveFirst && there && !live) {   // every sample gets an entry, so no reader sees unwritten scratch
         res[i] = make_float4(0.f, 0.f, 0.f, 0.f);
         if (SAVE) nh[i] = 0;
-        return;
     }
     const Ray ray = make_ray(ld3w(xg, p0 + i / St), mk3(d4.x, d4.y, d4.z));
-    MarchState<K, 3> st;
+    MarchState<3> st;
+    st.init();
     uint64_t last_key = depth_key(P.t_min, 0.f);
     int32_t last_u = INT32_MAX;
-    if (MODE == kWaveFirst) {
-        st.C[0] = st.C[1] = st.C[2] = 0.f;
-        st.D = 0.f;
-        st.T = 1.f;
-        st.nh = 0;
-    } else {
+    if (MODE != kWaveFirst) {
         const float4 a = state[j * kWaveStateF4], b = state[j * kWaveStateF4 + 1], c = state[j * kWaveStateF4 + 2];
         st.C[0] = a.x; st.C[1] = a.y; st.C[2] = a.z;
         st.D = a.w;
@@ -148,13 +143,15 @@ __global__ void __launch_bounds__(kWaveThreads, 6) k_wave_round(
         last_u = __float_as_int(c.x);
     }
     int32_t* my_ids = SAVE ? ids + i * (int64_t)max_ids : nullptr;
-    KBuffer<K, trace_threads<K>()> kb;
+    KBuffer<kBufferCap> kb;
     kb.bind();
-    bool ok = true, done = false;
+    float4* scratch = warp_scratch<false>();
+    bool ok = true, done = !live, packet = false;
     do {
-        ok &= collect_round(S, ray, P, last_key, last_u, kb);
-        done = blend_round<K, 3>(S, P, kb, st, my_ids, max_ids, last_key, last_u);
-    } while (MODE == kWaveLast && !done);
+        ok &= collect<false>(S, ray, P, last_key, last_u, st.T, kb, !done, packet, scratch);
+        if (!done) done = blend_round<3>(S, ray, P, kb, st, my_ids, max_ids, last_key, last_u);
+    } while (MODE == kWaveLast && __any_sync(kFullWarp, !done));
+    if (!live) return;
     if (!ok) atomicOr(S.status, kErrStackOverflow);
     if (done) {
         res[i] = make_float4(st.C[0], st.C[1], st.C[2], st.T);
@@ -172,7 +169,6 @@ __global__ void __launch_bounds__(kWaveThreads, 6) k_wave_round(
 }
 
 // Per-point estimate from the stored traces (warp per point).
-template <int K>
 __global__ void __launch_bounds__(kWaveThreads) k_wave_shade(SceneView S, const float* __restrict__ xg,
                                                              const float* __restrict__ ng,
                                                              const float* __restrict__ ag,
@@ -194,7 +190,7 @@ __global__ void __launch_bounds__(kWaveThreads) k_wave_shade(SceneView S, const 
         o.ind[0] = o.ind[1] = o.ind[2] = 0.f;
         o.vis = 0.f;
     } else {
-        shade_point_warp<K, false, true>(S, ld3w(xg, p), ld3w(ng, p), ld3w(wog, p), ld3w(ag, p), rg[p],
+        shade_point_warp<false, true>(S, ld3w(xg, p), ld3w(ng, p), ld3w(wog, p), ld3w(ag, p), rg[p],
                                          key_base + (uint64_t)p, nd, ns, mode, seed, env, H, W, TP, o, res + k * St);
     }
     if (lane == 0) {
@@ -244,13 +240,13 @@ __global__ void __launch_bounds__(kWaveThreads) k_wave_grad_point(
 
 // Backward of one ray in regrouped order (sorted position j): from its saved
 // hit list (LISTED) or by replaying its march.
-template <int K, bool LISTED>
+template <bool LISTED>
 __device__ __forceinline__ void wave_backward_ray(const SceneView& S, const TraceParams& P,
                                                   const float* __restrict__ xg, int64_t p0, int St,
                                                   const float4* __restrict__ dir, int64_t i,
                                                   const float4* __restrict__ res, int n_hits,
                                                   const int32_t* __restrict__ ids, int max_ids, float4 u4,
-                                                  float* __restrict__ acc_rows, float* rows) {
+                                                  float* __restrict__ acc_rows, float4* scratch, bool live = true) {
     const float4 d4 = dir[i];
     const int64_t p = p0 + i / St;
     const Ray ray = make_ray(ld3w(xg, p), mk3(d4.x, d4.y, d4.z));
@@ -259,10 +255,10 @@ __device__ __forceinline__ void wave_backward_ray(const SceneView& S, const Trac
     const float gC[3] = {u4.x, u4.y, u4.z};
     if (LISTED) {
         listed_backward<3>(S, ray, P, ids + i * (int64_t)max_ids, n_hits, Cf, 0.f, t.w, gC, 0.f, u4.w, acc_rows,
-                           rows);
+                           reinterpret_cast<float*>(scratch));
     } else {
-        const bool ok = march_backward<K, 3, false>(S, ray, P, true, n_hits, Cf, 0.f, t.w, gC, 0.f, u4.w, acc_rows,
-                                                    rows);
+        const bool ok = march_backward<3, false>(S, ray, P, live, n_hits, Cf, 0.f, t.w, gC, 0.f, u4.w, acc_rows,
+                                                 scratch);
         if (!ok) atomicOr(S.status, kErrStackOverflow);
     }
 }
@@ -270,7 +266,6 @@ __device__ __forceinline__ void wave_backward_ray(const SceneView& S, const Trac
 // Backward from the saved hit lists, one thread per sorted ray; rays whose
 // list did not fit (more than max_ids hits) are appended to replay_list for
 // k_wave_replay.
-template <int K>
 __global__ void __launch_bounds__(kWaveThreads) k_wave_backward(SceneView S, TraceParams P,
                                                                 const float* __restrict__ xg, int64_t p0, int St,
                                                                 const float4* __restrict__ dir,
@@ -282,9 +277,7 @@ __global__ void __launch_bounds__(kWaveThreads) k_wave_backward(SceneView S, Tra
                                                                 float* __restrict__ acc_rows,
                                                                 int32_t* __restrict__ replay_list,
                                                                 uint32_t* __restrict__ replay_count) {
-    static_assert(kWaveThreads == trace_threads<K>(), "k-buffer slots are laid out per block thread");
-    __shared__ float4 rows_all[kWaveThreads * GradRow<3>::kStride / 4];
-    float* rows = reinterpret_cast<float*>(rows_all) + (threadIdx.x & ~31) * GradRow<3>::kStride;
+    float4* scratch = warp_memory<32 * GradRow<3>::kStride / 4>();
     const int64_t j = blockIdx.x * (int64_t)kWaveThreads + threadIdx.x;
     if (j >= rays) return;
     const int64_t i = order[j];
@@ -296,13 +289,12 @@ __global__ void __launch_bounds__(kWaveThreads) k_wave_backward(SceneView S, Tra
         replay_list[atomicAdd(replay_count, 1u)] = (int32_t)j;
         return;
     }
-    wave_backward_ray<K, true>(S, P, xg, p0, St, dir, i, res, n_hits, ids, max_ids, u4, acc_rows, rows);
+    wave_backward_ray<true>(S, P, xg, p0, St, dir, i, res, n_hits, ids, max_ids, u4, acc_rows, scratch);
 }
 
 // The rays of replay_list replay their march backwards (the list's length is
 // what the listing launch left in replay_count). Consecutive entries go to
 // different blocks, so the few long replays spread over every SM.
-template <int K>
 __global__ void __launch_bounds__(kWaveThreads) k_wave_replay(SceneView S, TraceParams P,
                                                               const float* __restrict__ xg, int64_t p0, int St,
                                                               const float4* __restrict__ dir,
@@ -313,13 +305,14 @@ __global__ void __launch_bounds__(kWaveThreads) k_wave_replay(SceneView S, Trace
                                                               float* __restrict__ acc_rows,
                                                               const int32_t* __restrict__ replay_list,
                                                               const uint32_t* __restrict__ replay_count) {
-    static_assert(kWaveThreads == trace_threads<K>(), "k-buffer slots are laid out per block thread");
-    __shared__ float4 rows_all[kWaveThreads * GradRow<3>::kStride / 4];
-    float* rows = reinterpret_cast<float*>(rows_all) + (threadIdx.x & ~31) * GradRow<3>::kStride;
+    float4* scratch = warp_memory<replay_f4<3, false>()>();
     const int64_t n = *replay_count;
-    for (int64_t t = threadIdx.x * (int64_t)gridDim.x + blockIdx.x; t < n; t += (int64_t)gridDim.x * kWaveThreads) {
-        const int64_t i = order[replay_list[t]];
-        wave_backward_ray<K, false>(S, P, xg, p0, St, dir, i, res, nh[i], nullptr, 0, up[i], acc_rows, rows);
+    for (int64_t t = threadIdx.x * (int64_t)gridDim.x + blockIdx.x; __any_sync(kFullWarp, t < n);
+         t += (int64_t)gridDim.x * kWaveThreads) {
+        const bool live = t < n;   // lanes without a ray follow the warp
+        const int64_t i = order[live ? replay_list[t] : 0];
+        wave_backward_ray<false>(S, P, xg, p0, St, dir, i, res, live ? nh[i] : 0, nullptr, 0, up[i], acc_rows, scratch,
+                                 live);
     }
 }
 
@@ -393,14 +386,14 @@ int64_t chunk_points(int St) {
 
 // Trace the sorted rays of one chunk into w.res (and, with SAVE, the hit
 // counts and lists): compacted rounds when the scene has surfels.
-template <int K, bool SAVE>
+template <bool SAVE>
 cudaError_t wave_trace(const SceneView& S, const TraceParams& TP, const float* x, int64_t p0, int St, int64_t rays,
                        WaveScratch& w, cudaStream_t st) {
     int32_t* ids = SAVE ? w.ids : nullptr;
     int32_t* nh = SAVE ? w.nh : nullptr;
     const int max_ids = SAVE ? kWaveSavedHits : 0;
     if (S.n == 0) {
-        k_wave_trace<K, SAVE><<<grid_for(rays, kWaveThreads), kWaveThreads, 0, st>>>(S, TP, x, p0, St, w.dir, w.val,
+        k_wave_trace<SAVE><<<grid_for(rays, kWaveThreads), kWaveThreads, 0, st>>>(S, TP, x, p0, St, w.dir, w.val,
                                                                                     rays, w.res, nh, ids, max_ids);
         count_launches(1);
         return cudaGetLastError();
@@ -408,30 +401,16 @@ cudaError_t wave_trace(const SceneView& S, const TraceParams& TP, const float* x
     const unsigned g = grid_for(rays, kWaveThreads);
     cudaError_t e = cudaMemsetAsync(w.flags, 0, sizeof(uint32_t) * (rays + 1), st);
     if (e != cudaSuccess) return e;
-    k_wave_round<K, SAVE, kWaveFirst><<<g, kWaveThreads, 0, st>>>(S, TP, x, p0, St, w.dir, w.val, rays, w.res, nh, ids,
-                                                                  max_ids, w.list, w.count, w.state, w.flags);
-    count_launches(1);
-    for (int round = 2; round <= 4 && e == cudaSuccess; ++round) {
-        e = flags_to_list(w.flags, rays, w.count + 1, w.list, w.count, st);
-        if (e != cudaSuccess) break;
-        if (round < 4) {
-            e = cudaMemsetAsync(w.flags, 0, sizeof(uint32_t) * (rays + 1), st);
-            if (e != cudaSuccess) break;
-            k_wave_round<K, SAVE, kWaveNext><<<g, kWaveThreads, 0, st>>>(S, TP, x, p0, St, w.dir, w.val, rays, w.res,
-                                                                         nh, ids, max_ids, w.list, w.count, w.state,
-                                                                         w.flags);
-        } else {
-            k_wave_round<K, SAVE, kWaveLast><<<g, kWaveThreads, 0, st>>>(S, TP, x, p0, St, w.dir, w.val, rays, w.res,
-                                                                         nh, ids, max_ids, w.list, w.count, w.state,
-                                                                         w.flags);
-        }
-        count_launches(1);
-        e = cudaGetLastError();
-    }
-    return e;
+    k_wave_round<SAVE, kWaveFirst><<<g, kWaveThreads, 0, st>>>(S, TP, x, p0, St, w.dir, w.val, rays, w.res, nh, ids,
+                                                               max_ids, w.list, w.count, w.state, w.flags);
+    e = flags_to_list(w.flags, rays, w.count + 1, w.list, w.count, st);
+    if (e != cudaSuccess) return e;
+    k_wave_round<SAVE, kWaveLast><<<g, kWaveThreads, 0, st>>>(S, TP, x, p0, St, w.dir, w.val, rays, w.res, nh, ids,
+                                                              max_ids, w.list, w.count, w.state, w.flags);
+    count_launches(2);
+    return cudaGetLastError();
 }
 
-template <int K>
 cudaError_t wave_forward(const SceneView& S, const uint32_t* bounds, const float* x, const float* n, const float* a,
                          const float* r, const float* wo, int64_t P, const float* env, int H, int W, int nd, int ns,
                          int mode, uint64_t seed, const TraceParams& TP, float* rgb, float* vis, float* ind,
@@ -448,9 +427,9 @@ cudaError_t wave_forward(const SceneView& S, const uint32_t* bounds, const float
                                                         w.key, w.val, key_base, valid);
         e = sort_pairs(w.key, w.val, w.key_tmp, w.val_tmp, w.hist, rays, st);
         if (e != cudaSuccess) break;
-        e = wave_trace<K, false>(S, TP, x, p0, St, rays, w, st);
+        e = wave_trace<false>(S, TP, x, p0, St, rays, w, st);
         if (e != cudaSuccess) break;
-        k_wave_shade<K><<<grid_for(np, kWaveThreads / 32), kWaveThreads, 0, st>>>(
+        k_wave_shade<<<grid_for(np, kWaveThreads / 32), kWaveThreads, 0, st>>>(
             S, x, n, a, r, wo, p0, np, env, H, W, nd, ns, mode, seed, TP, w.res, rgb, vis, ind, key_base, valid);
         count_launches(2);
         e = cudaGetLastError();
@@ -459,7 +438,6 @@ cudaError_t wave_forward(const SceneView& S, const uint32_t* bounds, const float
     return e != cudaSuccess ? e : ef;
 }
 
-template <int K>
 cudaError_t wave_backward(const SceneView& S, const int32_t* perm, const uint32_t* bounds, const float* x,
                           const float* n, const float* a, const float* r, const float* wo, int64_t P,
                           const float* env, int H, int W, int nd, int ns, int mode, uint64_t seed,
@@ -484,15 +462,15 @@ cudaError_t wave_backward(const SceneView& S, const int32_t* perm, const uint32_
         e = sort_pairs(w.key, w.val, w.key_tmp, w.val_tmp, w.hist, rays, st);
         if (e != cudaSuccess) break;
         const unsigned g = grid_for(rays, kWaveThreads);
-        e = wave_trace<K, true>(S, TP, x, p0, St, rays, w, st);
+        e = wave_trace<true>(S, TP, x, p0, St, rays, w, st);
         if (e != cudaSuccess) break;
         k_wave_grad_point<<<grid_for(np, kWaveThreads / 32), kWaveThreads, 0, st>>>(
             n, a, r, wo, p0, np, env, H, W, nd, ns, mode, seed, w.res, g_rgb, g_albedo, g_rough, g_env, w.up);
         e = cudaMemsetAsync(w.count, 0, sizeof(uint32_t), st);
         if (e != cudaSuccess) break;
-        k_wave_backward<K><<<g, kWaveThreads, 0, st>>>(S, TP, x, p0, St, w.dir, w.val, rays, w.res, w.nh, w.ids,
+        k_wave_backward<<<g, kWaveThreads, 0, st>>>(S, TP, x, p0, St, w.dir, w.val, rays, w.res, w.nh, w.ids,
                                                        kWaveSavedHits, w.up, acc_rows, w.list, w.count);
-        k_wave_replay<K><<<kWaveReplayBlocks, kWaveThreads, 0, st>>>(S, TP, x, p0, St, w.dir, w.val, w.res, w.nh,
+        k_wave_replay<<<kWaveReplayBlocks, kWaveThreads, 0, st>>>(S, TP, x, p0, St, w.dir, w.val, w.res, w.nh,
                                                                      w.up, acc_rows, w.list, w.count);
         count_launches(4);
         e = cudaGetLastError();
@@ -523,15 +501,9 @@ irgs_status launch_shade_wave(const SceneView& S, const uint32_t* bounds, const 
                               uint64_t key_base, const float* valid) {
     if (P == 0) return IRGS_OK;
     const TraceParams TP = to_params(p);
-    switch (p.k) {
-        case 8:
-            return to_status(wave_forward<8>(S, bounds, x, n, albedo, rough, wo, P, env, H, W, n_diffuse, n_spec,
-                                             mode, seed, TP, rgb, vis, ind, st, key_base, valid));
-        case 16:
-            return to_status(wave_forward<16>(S, bounds, x, n, albedo, rough, wo, P, env, H, W, n_diffuse, n_spec,
-                                              mode, seed, TP, rgb, vis, ind, st, key_base, valid));
-        default: return IRGS_ERR_UNSUPPORTED;
-    }
+    if (p.k != 8 && p.k != 16) return IRGS_ERR_UNSUPPORTED;
+    return to_status(wave_forward(S, bounds, x, n, albedo, rough, wo, P, env, H, W, n_diffuse, n_spec, mode, seed, TP,
+                                  rgb, vis, ind, st, key_base, valid));
 }
 
 irgs_status launch_shade_wave_backward(const SceneView& S, const int32_t* perm, const uint32_t* bounds,
@@ -543,17 +515,10 @@ irgs_status launch_shade_wave_backward(const SceneView& S, const int32_t* perm, 
                                        float* g_opacity, float* g_features, cudaStream_t st) {
     if (P == 0) return IRGS_OK;
     const TraceParams TP = to_params(p);
-    switch (p.k) {
-        case 8:
-            return to_status(wave_backward<8>(S, perm, bounds, x, n, albedo, rough, wo, P, env, H, W, n_diffuse,
-                                              n_spec, mode, seed, TP, g_rgb, g_albedo, g_rough, g_env, g_means,
-                                              g_quats, g_scales, g_opacity, g_features, st));
-        case 16:
-            return to_status(wave_backward<16>(S, perm, bounds, x, n, albedo, rough, wo, P, env, H, W, n_diffuse,
-                                               n_spec, mode, seed, TP, g_rgb, g_albedo, g_rough, g_env, g_means,
-                                               g_quats, g_scales, g_opacity, g_features, st));
-        default: return IRGS_ERR_UNSUPPORTED;
-    }
+    if (p.k != 8 && p.k != 16) return IRGS_ERR_UNSUPPORTED;
+    return to_status(wave_backward(S, perm, bounds, x, n, albedo, rough, wo, P, env, H, W, n_diffuse, n_spec, mode,
+                                   seed, TP, g_rgb, g_albedo, g_rough, g_env, g_means, g_quats, g_scales, g_opacity,
+                                   g_features, st));
 }
 
 }  // namespace irgs

@@ -1,4 +1,4 @@
-// Per-ray traversal of the LBVH with a register k-buffer and front-to-back
+// Traversal of the BVH with a shared-memory k-buffer and front-to-back
 // compositing -- Trace(r_o, r_d) of IRGS Eq. 8 with the intersection of Eq. 6,
 // the response of Eq. 7 and the blending of Eq. 2. Shared by the forward,
 // backward and shading kernels, which must reproduce each other's hit order
@@ -20,23 +20,32 @@ struct TraceParams {
 
 struct Ray {
     f3 o, d;           // origin and direction as given
-    f3 inv;            // 1/d with zero components replaced (slab test only)
-    f3 oinv;           // o * inv
     float inv_dd;      // 1 / |d|^2
     float graze;       // 1e-8 |d|
-    int nrx, nry, nrz; // row of a wide node holding each axis' entry plane (lo if inv >= 0, else hi)
 };
 
 __device__ __forceinline__ Ray make_ray(f3 o, f3 d) {
     Ray r;
     r.o = o;
     r.d = d;
-    auto safe = [](float x) { return fabsf(x) < 1e-20f ? copysignf(1e-20f, x) : x; };
-    r.inv = mk3(1.0f / safe(d.x), 1.0f / safe(d.y), 1.0f / safe(d.z));
-    r.oinv = mk3(o.x * r.inv.x, o.y * r.inv.y, o.z * r.inv.z);
     float dd = fmaf(d.x, d.x, fmaf(d.y, d.y, d.z * d.z));
     r.inv_dd = 1.0f / dd;
     r.graze = 1e-8f * sqrtf(dd);
+    return r;
+}
+
+// A ray's slab-test form.
+struct RayBox {
+    f3 inv;            // 1/d with zero components replaced
+    f3 oinv;           // o * inv
+    int nrx, nry, nrz; // row of a wide node holding each axis' entry plane (lo if inv >= 0, else hi)
+};
+
+__device__ __forceinline__ RayBox make_ray_box(const Ray& ray) {
+    RayBox r;
+    auto safe = [](float x) { return fabsf(x) < 1e-20f ? copysignf(1e-20f, x) : x; };
+    r.inv = mk3(1.0f / safe(ray.d.x), 1.0f / safe(ray.d.y), 1.0f / safe(ray.d.z));
+    r.oinv = mk3(ray.o.x * r.inv.x, ray.o.y * r.inv.y, ray.o.z * r.inv.z);
     r.nrx = r.inv.x >= 0.f ? 0 : 3;
     r.nry = r.inv.y >= 0.f ? 1 : 4;
     r.nrz = r.inv.z >= 0.f ? 2 : 5;
@@ -59,14 +68,13 @@ struct HitGeom {
 //   dl  = mu - o' = fma(-t_r, d, a_hi) + a_lo          (small, nearly exact)
 //   tau = t_r + n.dl / n.d,  p - mu = (tau - t_r) d - dl.
 // The depth is returned as the exact pair (kh, kl) = two_sum(t_r, tau - t_r).
-// A candidate whose rounded depth kh lies outside [kh_lo, kh_hi] is rejected
-// before the support and opacity tests (callers pass bounds that only cut
-// candidates their own key tests would reject).
-template <bool GEOM>
-__device__ __forceinline__ bool surfel_hit(const float4& r0, const float4& r1, const float4& r2, const float4& r3,
-                                           const Ray& ray, float amin, float amax, float& kh, float& kl,
-                                           float& alpha, HitGeom* g, float kh_lo = -INFINITY,
-                                           float kh_hi = INFINITY) {
+// surfel_depth: that depth; false where the ray grazes the plane (|n.d| <
+// 1e-8 |d|).
+struct DepthParts {
+    float dlx, dly, dlz, den, tp;
+};
+__device__ __forceinline__ bool surfel_depth(const float4& r0, const float4& r3, const Ray& ray, float& kh, float& kl,
+                                             DepthParts* g = nullptr) {
     float ahx, alx, ahy, aly, ahz, alz;
     two_sum(r0.x, -ray.o.x, ahx, alx);
     two_sum(r0.y, -ray.o.y, ahy, aly);
@@ -81,10 +89,25 @@ __device__ __forceinline__ bool surfel_hit(const float4& r0, const float4& r1, c
     float num = __fmaf_rn(r3.x, dlx, __fmaf_rn(r3.y, dly, __fmul_rn(r3.z, dlz)));
     float tp = __fdiv_rn(num, den);
     two_sum(tr, tp, kh, kl);
+    if (g != nullptr) *g = {dlx, dly, dlz, den, tp};
+    return true;
+}
+
+// The whole test. A candidate whose rounded depth kh lies outside [kh_lo,
+// kh_hi] is rejected before the support and opacity tests (callers pass
+// bounds that only cut candidates their own key tests would reject).
+template <bool GEOM>
+__device__ __forceinline__ bool surfel_hit(const float4& r0, const float4& r1, const float4& r2, const float4& r3,
+                                           const Ray& ray, float amin, float amax, float& kh, float& kl,
+                                           float& alpha, HitGeom* g, float kh_lo = -INFINITY,
+                                           float kh_hi = INFINITY) {
+    DepthParts p;
+    if (!surfel_depth(r0, r3, ray, kh, kl, &p)) return false;
+    const f3 d = ray.d;
     if (kh < kh_lo || kh > kh_hi) return false;
-    float ex = __fmaf_rn(tp, d.x, -dlx);
-    float ey = __fmaf_rn(tp, d.y, -dly);
-    float ez = __fmaf_rn(tp, d.z, -dlz);
+    float ex = __fmaf_rn(p.tp, d.x, -p.dlx);
+    float ey = __fmaf_rn(p.tp, d.y, -p.dly);
+    float ez = __fmaf_rn(p.tp, d.z, -p.dlz);
     float u = __fmaf_rn(ex, r1.x, __fmaf_rn(ey, r1.y, __fmul_rn(ez, r1.z)));
     float v = __fmaf_rn(ex, r2.x, __fmaf_rn(ey, r2.y, __fmul_rn(ez, r2.z)));
     float rho2 = __fmaf_rn(u, u, __fmul_rn(v, v));
@@ -99,24 +122,9 @@ __device__ __forceinline__ bool surfel_hit(const float4& r0, const float4& r1, c
         g->v = v;
         g->G = G;
         g->a_raw = a_raw;
-        g->den = den;
+        g->den = p.den;
     }
     return true;
-}
-
-__device__ __forceinline__ void slab2(const Node& nd, const Ray& r, float& tn0, float& tf0, float& tn1,
-                                      float& tf1) {
-    // child 0: lo = (a.x,a.y,a.z) hi = (a.w,b.x,b.y); child 1: lo = (b.z,b.w,c.x) hi = (c.y,c.z,c.w)
-    float x0 = fmaf(nd.a.x, r.inv.x, -r.oinv.x), x1 = fmaf(nd.a.w, r.inv.x, -r.oinv.x);
-    float y0 = fmaf(nd.a.y, r.inv.y, -r.oinv.y), y1 = fmaf(nd.b.x, r.inv.y, -r.oinv.y);
-    float z0 = fmaf(nd.a.z, r.inv.z, -r.oinv.z), z1 = fmaf(nd.b.y, r.inv.z, -r.oinv.z);
-    tn0 = fmaxf(fmaxf(fminf(x0, x1), fminf(y0, y1)), fminf(z0, z1));
-    tf0 = fminf(fminf(fmaxf(x0, x1), fmaxf(y0, y1)), fmaxf(z0, z1));
-    x0 = fmaf(nd.b.z, r.inv.x, -r.oinv.x); x1 = fmaf(nd.c.y, r.inv.x, -r.oinv.x);
-    y0 = fmaf(nd.b.w, r.inv.y, -r.oinv.y); y1 = fmaf(nd.c.z, r.inv.y, -r.oinv.y);
-    z0 = fmaf(nd.c.x, r.inv.z, -r.oinv.z); z1 = fmaf(nd.c.w, r.inv.z, -r.oinv.z);
-    tn1 = fmaxf(fmaxf(fminf(x0, x1), fminf(y0, y1)), fminf(z0, z1));
-    tf1 = fminf(fminf(fmaxf(x0, x1), fmaxf(y0, y1)), fmaxf(z0, z1));
 }
 
 __device__ __forceinline__ float max3f(float a, float b, float c) {
@@ -130,34 +138,6 @@ __device__ __forceinline__ float min3f(float a, float b, float c) {
     return r;
 }
 
-__device__ __forceinline__ WideNode load_wide(const WideNode* w, int i) {
-    const float4* p = reinterpret_cast<const float4*>(w + i);
-    WideNode n;
-    n.lox = ldg4(p);
-    n.loy = ldg4(p + 1);
-    n.loz = ldg4(p + 2);
-    n.hix = ldg4(p + 3);
-    n.hiy = ldg4(p + 4);
-    n.hiz = ldg4(p + 5);
-    n.child = ldg4i(reinterpret_cast<const int4*>(p + 6));
-    return n;
-}
-
-// Slab intervals of the four children of a wide node.
-__device__ __forceinline__ void slab4(const WideNode& w, const Ray& r, float tn[4], float tf[4]) {
-    const float lx[4] = {w.lox.x, w.lox.y, w.lox.z, w.lox.w}, hx[4] = {w.hix.x, w.hix.y, w.hix.z, w.hix.w};
-    const float ly[4] = {w.loy.x, w.loy.y, w.loy.z, w.loy.w}, hy[4] = {w.hiy.x, w.hiy.y, w.hiy.z, w.hiy.w};
-    const float lz[4] = {w.loz.x, w.loz.y, w.loz.z, w.loz.w}, hz[4] = {w.hiz.x, w.hiz.y, w.hiz.z, w.hiz.w};
-#pragma unroll
-    for (int k = 0; k < 4; ++k) {
-        const float x0 = fmaf(lx[k], r.inv.x, -r.oinv.x), x1 = fmaf(hx[k], r.inv.x, -r.oinv.x);
-        const float y0 = fmaf(ly[k], r.inv.y, -r.oinv.y), y1 = fmaf(hy[k], r.inv.y, -r.oinv.y);
-        const float z0 = fmaf(lz[k], r.inv.z, -r.oinv.z), z1 = fmaf(hz[k], r.inv.z, -r.oinv.z);
-        tn[k] = max3f(fminf(x0, x1), fminf(y0, y1), fminf(z0, z1));
-        tf[k] = min3f(fmaxf(x0, x1), fmaxf(y0, y1), fmaxf(z0, z1));
-    }
-}
-
 // A wide node's child boxes as the ray meets them: for each axis the plane
 // it enters through (lo where 1/d >= 0, else hi) and the one it leaves
 // through, selected by which rows are loaded.
@@ -166,7 +146,7 @@ struct WideNodeRay {
     int4 child;
 };
 
-__device__ __forceinline__ WideNodeRay load_wide_ray(const WideNode* w, int i, const Ray& r) {
+__device__ __forceinline__ WideNodeRay load_wide_ray(const WideNode* w, int i, const RayBox& r) {
     const float4* p = reinterpret_cast<const float4*>(w + i);
     WideNodeRay n;
     n.nx = ldg4(p + r.nrx);
@@ -179,11 +159,10 @@ __device__ __forceinline__ WideNodeRay load_wide_ray(const WideNode* w, int i, c
     return n;
 }
 
-// Slab intervals of the four children from the entry / exit planes: the same
-// values slab4 gives (fma(v, inv, -oinv) is monotone in v for a fixed sign
-// of inv, so the entry plane's distance is the minimum of the pair), with
-// no per-axis min/max.
-__device__ __forceinline__ void slab4_ray(const WideNodeRay& w, const Ray& r, float tn[4], float tf[4]) {
+// Slab intervals of the four children from the entry / exit planes
+// (fma(v, inv, -oinv) is monotone in v for a fixed sign of inv, so the entry
+// plane's distance is the smaller of the pair without a min/max).
+__device__ __forceinline__ void slab4_ray(const WideNodeRay& w, const RayBox& r, float tn[4], float tf[4]) {
     const float nx[4] = {w.nx.x, w.nx.y, w.nx.z, w.nx.w}, fx[4] = {w.fx.x, w.fx.y, w.fx.z, w.fx.w};
     const float ny[4] = {w.ny.x, w.ny.y, w.ny.z, w.ny.w}, fy[4] = {w.fy.x, w.fy.y, w.fy.z, w.fy.w};
     const float nz[4] = {w.nz.x, w.nz.y, w.nz.z, w.nz.w}, fz[4] = {w.fz.x, w.fz.y, w.fz.z, w.fz.w};
@@ -199,325 +178,530 @@ __device__ __forceinline__ void slab4_ray(const WideNodeRay& w, const Ray& r, fl
 // Conservative slack on depths compared against box intervals.
 __device__ __forceinline__ float tslack(float t) { return 1e-5f * (1.0f + fabsf(t)); }
 
-__device__ __forceinline__ Node load_node(const Node* nodes, int i) {
-    const float4* p = reinterpret_cast<const float4*>(nodes + i);
-    Node nd;
-    nd.a = ldg4(p);
-    nd.b = ldg4(p + 1);
-    nd.c = ldg4(p + 2);
-    nd.d = ldg4i(reinterpret_cast<const int4*>(p + 3));
-    return nd;
+__device__ __forceinline__ float key_depth(uint64_t k) { return __uint_as_float((uint32_t)(k >> 32)); }
+
+// ---------------------------------------------------------------------------
+// Threads per block of every tracing kernel (k-buffer slots and leaf queues
+// are laid out per block thread).
+constexpr int kTraceThreads = 128;
+
+// Entries of the k-buffer. Results do not depend on it (the buffer holds the
+// nearest hits after the last blended one, whatever its size), so the size a
+// caller asks for does not select code. 32 entries hold every hit of most
+// rays that the transmittance cut below leaves.
+constexpr int kBufferCap = 32;
+
+// Exact depth remainder kl and user index of surfel m, whose hit at the same
+// rounded depth ties with another: out of line, since ties are rare.
+static __device__ __noinline__ float2 tie_of(const float4* rec, int32_t m, f3 o, f3 d, float inv_dd) {
+    Ray r;
+    r.o = o;
+    r.d = d;
+    r.inv_dd = inv_dd;
+    r.graze = 0.f;
+    const float4* R = rec + (int64_t)m * kRecF4;
+    const float4 r2 = ldg4(R + 2);
+    float kh, kl;
+    surfel_depth(ldg4(R), ldg4(R + 3), r, kh, kl);
+    return make_float2(kl, r2.w);
 }
 
-// User index of the surfel in Morton slot m (carried in its record's r2.w).
-__device__ __forceinline__ int32_t uid_of(const float4* rec, int32_t m) {
-    return __float_as_int(__ldg(&rec[(int64_t)m * kRecF4 + 2].w));
-}
-
-// k-buffer of the K nearest hits after `last`, sorted by (key, user index),
-// kept in shared memory as 16-byte entries {key (8 B), Morton index, alpha}:
-// slot j of thread t lives at [j * THREADS + t], so a warp touching the same
-// slot reads consecutive 16-byte words, and one shift step of the insertion
-// is one 128-bit load and one 128-bit store. Insertion shifts only the
-// entries behind the new one (hits mostly arrive front to back, so the shift
-// is usually short); the last entry is cached in registers for the cheap
-// "does it fit" test and the traversal's far bound. Two hits with the same
-// exact depth key are ordered by user index, which is read from the
-// record only on that (rare) tie.
-template <int K, int THREADS>
+// k-buffer of the nearest hits after the last blended one, ascending in
+// (depth, user index), in shared memory as 8-byte entries: x the bits of the
+// rounded depth kh, y the Morton index with the hit's optical depth in the
+// top byte. Slot j of thread t lives at [j * kTraceThreads + t], so a warp
+// touching one slot reads consecutive words. Two hits with the same rounded
+// depth are ordered by the exact remainder and then the user index, both
+// recomputed on that (rare) tie; alpha is recomputed when a hit is blended.
+//
+// The buffer is closed when it is full or when its hits alone bring the
+// transmittance below T_min: the optical depths, floor(-16 log2(1 - alpha))
+// each, add up to `need`, and entries behind the shortest such prefix are
+// dropped. A closed buffer bounds the walk by its last depth. The sums round
+// down, so a prefix is never cut short; if the blend does not end inside a
+// closed buffer, another round continues behind its last entry.
+template <int CAP>
 struct KBuffer {
-    static constexpr int kThreads = THREADS;
-    uint4* e;   // x, y: key (low, high); z: Morton index; w: alpha bits
+    uint2* e;
     int cnt;
-    uint64_t tail_key;
-    int32_t tail_m;
+    uint32_t sum, need, id_mask;
+    uint32_t tail;   // depth bits of the last entry of a closed buffer
 
+    // The kernel's one shared array of entries.
     __device__ __forceinline__ void bind() {
-        __shared__ uint4 s_e[K * THREADS];
+        __shared__ uint2 s_e[CAP * kTraceThreads];
         e = s_e + threadIdx.x;
         cnt = 0;
     }
-    __device__ __forceinline__ static uint64_t key_of(const uint4& v) {
-        return ((uint64_t)v.y << 32) | (uint64_t)v.x;
+    // An empty buffer for a ray of transmittance T (T >= T_min).
+    __device__ __forceinline__ void open(int64_t n, float T, float T_min) {
+        cnt = 0;
+        sum = 0u;
+        const bool packs = n <= (int64_t)1 << 24;   // 24-bit Morton indices leave a byte for the optical depth
+        id_mask = packs ? 0xffffffu : 0xffffffffu;
+        // optical depth that is surely past T_min; never reached when T_min = 0
+        const float bits = 16.f * __log2f(__fdividef(T, T_min)) + 2.f;
+        need = packs && T_min > 0.f && bits < 1e9f ? (uint32_t)fmaxf(bits, 1.f) : 0xffffffffu;
     }
-    __device__ __forceinline__ void clear() { cnt = 0; }
-    __device__ __forceinline__ bool full() const { return cnt == K; }
-    __device__ __forceinline__ uint64_t key_at(int j) const { return key_of(e[j * THREADS]); }
-    __device__ __forceinline__ int32_t m_at(int j) const { return (int32_t)e[j * THREADS].z; }
-    __device__ __forceinline__ float a_at(int j) const { return __uint_as_float(e[j * THREADS].w); }
-    // does the hit (k, user index u) belong before the full buffer's last entry?
-    __device__ __forceinline__ bool fits(uint64_t k, int32_t u, const float4* rec) const {
-        return cnt < K || k < tail_key || (k == tail_key && u < uid_of(rec, tail_m));
+    __device__ __forceinline__ bool closed() const { return cnt == CAP || sum >= need; }
+    __device__ __forceinline__ int32_t m_at(int j) const { return (int32_t)(e[j * kTraceThreads].y & id_mask); }
+    // does a hit at (kb = bits of kh, kl, user index u) come before entry v?
+    __device__ __forceinline__ bool before(uint32_t kb, float kl, int32_t u, const uint2& v, const float4* rec,
+                                           const Ray& ray) const {
+        if (kb != v.x) return kb < v.x;
+        const float2 t = tie_of(rec, (int32_t)(v.y & id_mask), ray.o, ray.d, ray.inv_dd);
+        return kl < t.x || (kl == t.x && u < __float_as_int(t.y));
     }
-    // insert (k, Morton index mm, user index u, alpha aa); the caller checked fits()
-    __device__ __forceinline__ void insert(uint64_t k, int32_t mm, int32_t u, float aa, const float4* rec) {
-        int j = (cnt < K ? cnt : K - 1) - 1;
-        while (j >= 0) {
-            const uint4 v = e[j * THREADS];
-            const uint64_t kj = key_of(v);
-            if (!(k < kj || (k == kj && u < uid_of(rec, (int32_t)v.z)))) break;
-            e[(j + 1) * THREADS] = v;
+    // Insert a hit unless the buffer is closed and it lies behind the last
+    // entry. Returns whether it went in.
+    __device__ __forceinline__ bool insert(float kh, float kl, int32_t m, int32_t u, float alpha, const float4* rec,
+                                           const Ray& ray) {
+        const uint32_t kb = __float_as_uint(kh + 0.0f);
+        const bool was_closed = closed();
+        if (was_closed &&
+            !(kb < tail || (kb == tail && before(kb, kl, u, e[(cnt - 1) * kTraceThreads], rec, ray))))
+            return false;
+        int j = cnt - 1;
+        if (cnt == CAP) {
+            sum -= id_mask == 0xffffffu ? e[j * kTraceThreads].y >> 24 : 0u;
             --j;
+        } else {
+            ++cnt;
         }
-        e[(j + 1) * THREADS] = make_uint4((uint32_t)k, (uint32_t)(k >> 32), (uint32_t)mm, __float_as_uint(aa));
-        if (cnt < K) ++cnt;
-        if (cnt == K) {
-            const uint4 t = e[(K - 1) * THREADS];
-            tail_key = key_of(t);
-            tail_m = (int32_t)t.z;
+        for (; j >= 0; --j) {
+            const uint2 v = e[j * kTraceThreads];
+            if (!before(kb, kl, u, v, rec, ray)) break;
+            e[(j + 1) * kTraceThreads] = v;
         }
+        uint32_t q = 0u;
+        if (id_mask == 0xffffffu) q = (uint32_t)fminf(fmaxf(-16.f * __log2f(1.f - alpha), 0.f), 255.f);
+        e[(j + 1) * kTraceThreads] = make_uint2(kb, (uint32_t)m | q << 24);
+        sum += q;
+        if (closed()) {
+            uint2 t = e[(cnt - 1) * kTraceThreads];
+            while (need != 0xffffffffu && cnt > 1 && sum - (t.y >> 24) >= need) {
+                sum -= t.y >> 24;
+                --cnt;
+                t = e[(cnt - 1) * kTraceThreads];
+            }
+            tail = t.x;
+        }
+        return true;
     }
 };
-
-// Threads per block of the tracing kernels for a k-buffer of K entries
-// (the shared-memory k-buffer takes K * THREADS * 16 bytes).
-template <int K>
-__host__ __device__ constexpr int trace_threads() { return K > 16 ? 64 : 128; }
-
-__device__ __forceinline__ float key_depth(uint64_t k) { return __uint_as_float((uint32_t)(k >> 32)); }
 
 // Per-ray traversal counters of the diagnostic build (STATS = true).
 struct TraceStats {
     int rounds, nodes, leaves, inserts;
 };
 
-// Test surfel m against the ray and insert it into the k-buffer if its
-// (key, user index) lies strictly after (last_key, last_u) and before the
-// buffer's last entry.
+// Shared working memory of one warp. The packet walk keeps its stack, its
+// pending leaves and the records of a batch of 32 leaves; the per-ray walk
+// its leaf queues (in the records' place).
+constexpr int kPacketStack = 192;
+constexpr int kLeafQueue = 12;   // pending leaves per ray
+struct PacketScratch {
+    float4 rec[32 * kRecF4];
+    uint2 stack[kPacketStack];   // (wide node, entry depth bits)
+    uint32_t leaf[64];
+    float mid[8];                // origin and direction of the ray the leaves are ordered for
+};
+constexpr int kQueueF4 = kLeafQueue * 32 / 4;
+static_assert(kQueueF4 <= 32 * kRecF4, "the leaf queues take the records' place");
+
+static_assert(sizeof(PacketScratch) % sizeof(float4) == 0, "per-warp slots stay aligned");
+// float4s of working memory that one warp's walk takes.
+template <bool PACKET>
+__host__ __device__ constexpr int scratch_f4() { return PACKET ? (int)(sizeof(PacketScratch) / sizeof(float4)) : kQueueF4; }
+
+// This warp's part of a block's working memory, F4 float4s per warp.
+template <int F4>
+__device__ __forceinline__ float4* warp_memory() {
+    __shared__ float4 s_warp[kTraceThreads / 32 * F4];
+    return s_warp + (threadIdx.x >> 5) * F4;
+}
+template <bool PACKET>
+__device__ __forceinline__ float4* warp_scratch() { return warp_memory<scratch_f4<PACKET>()>(); }
+
+// One ray against surfel records: into the buffer if its hit lies strictly
+// after (last_key, last_u) and before t_max and the buffer's last entry.
 template <class KB, bool STATS = false>
-__device__ __forceinline__ void leaf_insert(const SceneView& S, const Ray& ray, const TraceParams& P, int32_t m,
-                                            uint64_t last_key, int32_t last_u, KB& kb, float& t_hi,
-                                            TraceStats* ts = nullptr) {
+__device__ __forceinline__ bool leaf_insert(const SceneView& S, const Ray& ray, const TraceParams& P, int32_t m,
+                                            const float4& r0, const float4& r1, const float4& r2, const float4& r3,
+                                            uint64_t last_key, int32_t last_u, KB& kb, float& t_hi, TraceStats* ts) {
     if (STATS) ts->leaves++;
-    const float4* R = S.rec + (int64_t)m * kRecF4;
-    const float4 r0 = ldg4(R), r1 = ldg4(R + 1), r2 = ldg4(R + 2), r3 = ldg4(R + 3);
     float kh, kl, a;
-    // a rounded depth below the last blended key's, or above the full
+    // a rounded depth below the last blended key's, or above the closed
     // buffer's last entry (t_hi, else t_max), cannot pass the key tests
     // below; kh >= key_depth(last_key) >= t_min >= 0 also makes the key
     // order that of the depths, and the first round's last_key = (t_min, 0)
     // with last_u = INT32_MAX admits exactly the depths beyond t_min
     if (!surfel_hit<false>(r0, r1, r2, r3, ray, P.alpha_min, P.alpha_max, kh, kl, a, nullptr, key_depth(last_key),
                            t_hi))
-        return;
+        return false;
     const uint64_t key = depth_key(kh, kl);
     const int32_t u = __float_as_int(r2.w);
     const bool after = key > last_key || (key == last_key && u > last_u);
-    const bool before = kh < P.t_max || (kh == P.t_max && kl < 0.f);
-    if (after && before && kb.fits(key, u, S.rec)) {
-        if (STATS) ts->inserts++;
-        kb.insert(key, m, u, a, S.rec);
-        if (kb.full()) t_hi = key_depth(kb.tail_key);
-    }
-}
-
-// One round: gather the K nearest hits strictly after (last_key, last_u).
-// Returns false if the traversal stack overflowed.
-template <class KB, bool STATS = false>
-__device__ __forceinline__ bool collect_round(const SceneView& S, const Ray& ray, const TraceParams& P,
-                                              uint64_t last_key, int32_t last_u, KB& kb,
-                                              TraceStats* ts = nullptr) {
-    int2 stack[kStackSize];   // (node, entry depth bits): one 8-byte word per entry
-    int sp = 0;
-    int2 top = make_int2(0, 0);
-    bool has_top = false;
-    bool ok = true;
-    kb.clear();
-    const float t_lo = key_depth(last_key);
-    const float lo_c = t_lo - tslack(t_lo);
-    float t_hi = P.t_max;
-    int ni = 0;
-    // each wide node is fetched at most once per round in a valid tree
-    const int max_visits = S.n + 64 < (int64_t)INT32_MAX ? (int)(S.n + 64) : INT32_MAX;
-    for (int visits = 0;; ++visits) {
-        if (visits > max_visits) {
-            ok = false;
-            break;
-        }
-        const WideNodeRay nd = load_wide_ray(S.wide, ni, ray);
-        if (STATS) ts->nodes++;
-        float tn[4], tf[4];
-        slab4_ray(nd, ray, tn, tf);
-        const int c[4] = {nd.child.x, nd.child.y, nd.child.z, nd.child.w};
-        float hi_c = t_hi + tslack(t_hi);
-        bool h[4];
-#pragma unroll
-        for (int k = 0; k < 4; ++k) h[k] = tn[k] <= tf[k] && tf[k] >= lo_c && tn[k] <= hi_c;   // empty slots: empty box
-        {
-            // lanes of a warp walk different nodes here: each tests its own
-            // needed leaves in one loop, so lanes run their i-th leaf test
-            // together whatever slot it sits in (slot order kept per lane)
-            unsigned mask = 0u;
-#pragma unroll
-            for (int k = 0; k < 4; ++k) mask |= (h[k] && c[k] < 0) ? (1u << k) : 0u;
-            while (mask != 0u) {
-                const int k = __ffs(mask) - 1;
-                mask &= mask - 1u;
-                const int ck = k == 0 ? c[0] : k == 1 ? c[1] : k == 2 ? c[2] : c[3];
-                leaf_insert<KB, STATS>(S, ray, P, ~ck, last_key, last_u, kb, t_hi, ts);
-            }
-        }
-        hi_c = t_hi + tslack(t_hi);
-        // internal children still in reach: descend into the nearest, push the rest far first
-        float t[4];
-        int nv = 0;
-#pragma unroll
-        for (int k = 0; k < 4; ++k) {
-            const bool v = h[k] && c[k] >= 0 && tn[k] <= hi_c;
-            t[k] = v ? tn[k] : INFINITY;
-            nv += v;
-        }
-        if (nv == 0) {
-            bool found = false;
-            if (has_top) {   // the most recent entry, kept in registers
-                has_top = false;
-                if (__int_as_float(top.y) <= hi_c) {
-                    ni = top.x;
-                    found = true;
-                }
-            }
-            while (!found && sp > 0) {
-                --sp;
-                const int2 e = stack[sp];
-                if (__int_as_float(e.y) <= hi_c) {
-                    ni = e.x;
-                    found = true;
-                }
-            }
-            if (!found) break;
-            continue;
-        }
-        // repeatedly take the farthest remaining child onto the stack
-        for (int r = 0; r < nv - 1; ++r) {
-            int far = -1;
-            float tfar = -INFINITY;
-#pragma unroll
-            for (int k = 0; k < 4; ++k)
-                if (t[k] != INFINITY && t[k] >= tfar) {
-                    tfar = t[k];
-                    far = k;
-                }
-            int2 ent = make_int2(0, 0);
-#pragma unroll
-            for (int k = 0; k < 4; ++k)
-                if (k == far) {
-                    ent = make_int2(c[k], __float_as_int(t[k]));
-                    t[k] = INFINITY;
-                }
-            if (has_top) {
-                if (sp < kStackSize) stack[sp++] = top;
-                else ok = false;
-            }
-            top = ent;
-            has_top = true;
-        }
-#pragma unroll
-        for (int k = 0; k < 4; ++k)
-            if (t[k] != INFINITY) ni = c[k];
-    }
-    return ok;
+    const bool inside = kh < P.t_max || (kh == P.t_max && kl < 0.f);
+    if (!(after && inside && kb.insert(kh, kl, m, u, a, S.rec, ray))) return false;
+    if (STATS) ts->inserts++;
+    if (kb.closed()) t_hi = __uint_as_float(kb.tail);
+    return true;
 }
 
 constexpr unsigned kFullWarp = 0xffffffffu;
 
-// Warp-coherent round: the 32 lanes of a warp walk one shared traversal
-// stack (entry e lives in register e/32 of lane e%32). A child is visited when
-// any lane's ray overlaps its box inside that lane's (t_lo, t_hi) window;
-// each lane tests leaves with its own ray and keeps its own k-buffer, so the
-// result per ray equals the per-thread round. All 32 lanes must call this
-// together (inactive lanes pass active = false).
+// Upper bound on node fetches of one round in a valid tree.
+__device__ __forceinline__ int visit_cap(const SceneView& S) {
+    return S.n + 64 < (int64_t)INT32_MAX ? (int)(S.n + 64) : INT32_MAX;
+}
+
+// One round, one traversal stack per ray: gather the nearest hits strictly
+// after (last_key, last_u). All 32 lanes call this together (lanes without a
+// ray pass active = false). The lanes of a warp walk different nodes, and on
+// average less than one leaf child per node has to be tested, so testing
+// each node's leaves on the spot leaves most lanes idle; here a lane queues
+// its leaves and the warp takes the step, node visits or leaf tests, that
+// more of its lanes are ready for. Returns false if a stack overflowed.
 template <class KB, bool STATS = false>
-__device__ __forceinline__ bool collect_round_warp(const SceneView& S, const Ray& ray, const TraceParams& P,
-                                                   uint64_t last_key, int32_t last_u, KB& kb, bool active,
-                                                   TraceStats* ts = nullptr) {
-    kb.clear();
-    const int lane = threadIdx.x & 31;
+__device__ __forceinline__ bool collect_round(const SceneView& S, const Ray& ray0, const TraceParams& P,
+                                              uint64_t last_key, int32_t last_u, KB& kb, bool active,
+                                              float4* scratch, TraceStats* ts = nullptr) {
+    uint32_t* queue = reinterpret_cast<uint32_t*>(scratch) + (threadIdx.x & 31);   // entry i at queue[32 i]
+    const RayBox rb = make_ray_box(ray0);
+    int2 stack[kStackSize];   // (node, entry depth bits): one 8-byte word per entry
+    int sp = 0;
+    int2 top = make_int2(0, 0);   // the most recent entry, kept in registers
+    bool has_top = false;
+    bool ok = true;
     const float t_lo = key_depth(last_key);
     const float lo_c = t_lo - tslack(t_lo);
     float t_hi = P.t_max;
-    int st0 = 0, st1 = 0;
-    int sp = 0;
-    bool ok = true;
-    int ni = 0;
-    const int max_visits = S.n + 64 < (int64_t)INT32_MAX ? (int)(S.n + 64) : INT32_MAX;
-    for (int visits = 0;; ++visits) {
-        if (visits > max_visits) {
-            ok = false;
-            break;
-        }
-        const WideNodeRay nd = load_wide_ray(S.wide, ni, ray);
-        if (STATS && active) ts->nodes++;
-        float tn[4], tf[4];
-        slab4_ray(nd, ray, tn, tf);
-        const int c[4] = {nd.child.x, nd.child.y, nd.child.z, nd.child.w};
-        float hi_c = t_hi + tslack(t_hi);
-        bool h[4];
-#pragma unroll
-        for (int k = 0; k < 4; ++k)
-            h[k] = active && tn[k] <= tf[k] && tf[k] >= lo_c && tn[k] <= hi_c;   // empty slots: empty box
-#pragma unroll
-        for (int k = 0; k < 4; ++k)
-            if (h[k] && c[k] < 0) leaf_insert<KB, STATS>(S, ray, P, ~c[k], last_key, last_u, kb, t_hi, ts);
-        hi_c = t_hi + tslack(t_hi);
-        // internal children some lane still needs; order them by the entry
-        // depth seen by the first lane that needs each
-        float t[4] = {INFINITY, INFINITY, INFINITY, INFINITY};
-        int nv = 0;
-        if (max(max(c[0], c[1]), max(c[2], c[3])) >= 0) {   // the node (same for the warp) has internal children
-#pragma unroll
-            for (int k = 0; k < 4; ++k) {
-                const unsigned b = __ballot_sync(kFullWarp, h[k] && c[k] >= 0 && tn[k] <= hi_c);
-                const int src = b ? __ffs(b) - 1 : 0;
-                const float tk = __shfl_sync(kFullWarp, tn[k], src);
-                t[k] = b ? tk : INFINITY;
-                nv += b ? 1 : 0;
+    int ni = active ? 0 : -1;
+    int qn = 0;
+    int visits = visit_cap(S);
+    for (;;) {
+        const bool can_walk = ni >= 0 && qn <= kLeafQueue - 4;
+        const unsigned walk = __ballot_sync(kFullWarp, can_walk);
+        const unsigned have = __ballot_sync(kFullWarp, qn > 0);
+        if ((walk | have) == 0u) break;
+        if (__popc(walk) <= __popc(have)) {
+            if (qn > 0) {
+                --qn;
+                const int32_t m = (int32_t)queue[32 * qn];
+                const float4* R = S.rec + (int64_t)m * kRecF4;
+                const float4 r0 = ldg4(R), r1 = ldg4(R + 1), r2 = ldg4(R + 2), r3 = ldg4(R + 3);
+                leaf_insert<KB, STATS>(S, ray0, P, m, r0, r1, r2, r3, last_key, last_u, kb, t_hi, ts);
             }
-        }
-        if (nv == 0) {
-            if (sp == 0) break;
-            --sp;
-            ni = __shfl_sync(kFullWarp, (sp >> 5) ? st1 : st0, sp & 31);
             continue;
         }
-        for (int r = 0; r < nv - 1; ++r) {
-            int far = -1;
-            float tfar = -INFINITY;
+        if (!can_walk) continue;
+        if (--visits < 0) {   // each wide node is fetched at most once per round in a valid tree
+            ok = false;
+            ni = -1;
+            continue;
+        }
+        const WideNodeRay nd = load_wide_ray(S.wide, ni, rb);
+        if (STATS) ts->nodes++;
+        float tn[4], tf[4];
+        slab4_ray(nd, rb, tn, tf);
+        const int c[4] = {nd.child.x, nd.child.y, nd.child.z, nd.child.w};
+        const float hi_c = t_hi + tslack(t_hi);
+        // children to enter, nearest first: entry depth (its last two bits
+        // give way to the child's number, which only rounds it down)
+        uint32_t key[4];
 #pragma unroll
-            for (int k = 0; k < 4; ++k)
-                if (t[k] != INFINITY && t[k] >= tfar) {
-                    tfar = t[k];
-                    far = k;
-                }
-            int farc = 0;
-#pragma unroll
-            for (int k = 0; k < 4; ++k)
-                if (k == far) {
-                    farc = c[k];
-                    t[k] = INFINITY;
-                }
-            if (sp < kStackSize) {
-                if (lane == (sp & 31)) {
-                    if (sp >> 5) st1 = farc; else st0 = farc;
-                }
-                ++sp;
-            } else {
+        for (int k = 0; k < 4; ++k) {
+            const bool h = tn[k] <= tf[k] && tf[k] >= lo_c && tn[k] <= hi_c;   // empty slots: empty box
+            if (h && c[k] < 0) queue[32 * qn++] = (uint32_t)~c[k];
+            key[k] = h && c[k] >= 0 ? (__float_as_uint(fmaxf(tn[k], 0.f)) & ~3u) | (uint32_t)k : 0xffffffffu;
+        }
+        auto order = [&](int a, int b) {
+            const uint32_t lo = min(key[a], key[b]), hi = max(key[a], key[b]);
+            key[a] = lo;
+            key[b] = hi;
+        };
+        order(0, 1);
+        order(2, 3);
+        order(0, 2);
+        order(1, 3);
+        order(1, 2);
+        auto child_of = [&](uint32_t k) {
+            const uint32_t s = k & 3u;
+            const int lo = (s & 1u) ? c[1] : c[0], hi = (s & 1u) ? c[3] : c[2];
+            return (s & 2u) ? hi : lo;
+        };
+        if (key[0] == 0xffffffffu) {
+            ni = -1;
+            if (has_top) {
+                has_top = false;
+                if (__int_as_float(top.y) <= hi_c) ni = top.x;
+            }
+            while (ni < 0 && sp > 0) {
+                const int2 e = stack[--sp];
+                if (__int_as_float(e.y) <= hi_c) ni = e.x;
+            }
+            continue;
+        }
+        ni = child_of(key[0]);
+        if (key[1] != 0xffffffffu) {
+            if (sp + 3 > kStackSize) {
                 ok = false;
+            } else {
+                if (has_top) stack[sp++] = top;
+                if (key[3] != 0xffffffffu) stack[sp++] = make_int2(child_of(key[3]), (int)(key[3] & ~3u));
+                if (key[2] != 0xffffffffu) stack[sp++] = make_int2(child_of(key[2]), (int)(key[2] & ~3u));
+            }
+            top = make_int2(child_of(key[1]), (int)(key[1] & ~3u));
+            has_top = true;
+        }
+    }
+    __syncwarp();   // the queues' memory may now take another use
+    return ok;
+}
+
+// Bounds of a warp's rays for the packet walk. Axis k is the one the rays
+// mostly run along; z = sign * (x_k - o_k) grows along every ray, and at z a
+// ray is at o_a + s_a z, o_b + s_b z with slopes s = d / |d_k| of any sign.
+struct Packet {
+    int k, a, b;                        // axes
+    float sign;
+    float zo_min, zo_max;               // sign * o_k
+    float oa_min, oa_max, ob_min, ob_max;
+    float sa_min, sa_max, sb_min, sb_max;
+    float dk_min, dk_max;               // |d_k|
+    float o_abs;                        // largest |o| component, for the rounding margin
+    float s_abs;
+};
+
+__device__ __forceinline__ float axis_of(f3 v, int k) { return k == 0 ? v.x : (k == 1 ? v.y : v.z); }
+
+__device__ __forceinline__ float warp_min(float v, bool on) {
+    const uint32_t u = on ? ordered_bits(v + 0.0f) : 0xffffffffu;
+    const uint32_t m = __reduce_min_sync(kFullWarp, u);
+    return __uint_as_float((m & 0x80000000u) ? (m & 0x7fffffffu) : ~m);
+}
+__device__ __forceinline__ float warp_max(float v, bool on) { return -warp_min(-v, on); }
+
+// The packet of the active lanes' rays; false if they do not run together:
+// a common dominant axis and direction along it, and slopes that spread by
+// less than kPacketSpread (a strip of a coarse image; a strip is long and
+// thin, so this alone says little, and collect_packet gives up on packets
+// whose leaves miss most of their rays).
+constexpr float kPacketSpread = 0.7f;
+__device__ __forceinline__ bool make_packet(const Ray& ray, bool active, Packet& p) {
+    const unsigned on = __ballot_sync(kFullWarp, active);
+    if (on == 0u) return false;
+    const int src = __ffs(on) - 1;
+    const float ax = fabsf(__shfl_sync(kFullWarp, ray.d.x, src)), ay = fabsf(__shfl_sync(kFullWarp, ray.d.y, src)),
+                az = fabsf(__shfl_sync(kFullWarp, ray.d.z, src));
+    p.k = ax >= ay && ax >= az ? 0 : (ay >= az ? 1 : 2);
+    p.a = p.k == 2 ? 0 : p.k + 1;
+    p.b = p.a == 2 ? 0 : p.a + 1;
+    p.sign = __shfl_sync(kFullWarp, axis_of(ray.d, p.k), src) >= 0.f ? 1.f : -1.f;
+    const float dk = p.sign * axis_of(ray.d, p.k);
+    const float inv = 1.0f / dk;
+    const float sa = axis_of(ray.d, p.a) * inv, sb = axis_of(ray.d, p.b) * inv;
+    const bool fits = dk > 1e-30f && dk < 1e30f && fabsf(sa) <= 2.5f && fabsf(sb) <= 2.5f &&
+                      fabsf(ray.o.x) < 1e15f && fabsf(ray.o.y) < 1e15f && fabsf(ray.o.z) < 1e15f;
+    if (!__all_sync(kFullWarp, fits || !active)) return false;
+    p.sa_min = warp_min(sa, active);
+    p.sa_max = warp_max(sa, active);
+    p.sb_min = warp_min(sb, active);
+    p.sb_max = warp_max(sb, active);
+    if (!(p.sa_max - p.sa_min <= kPacketSpread && p.sb_max - p.sb_min <= kPacketSpread)) return false;
+    const float zo = p.sign * axis_of(ray.o, p.k), oa = axis_of(ray.o, p.a), ob = axis_of(ray.o, p.b);
+    p.zo_min = warp_min(zo, active);
+    p.zo_max = warp_max(zo, active);
+    p.oa_min = warp_min(oa, active);
+    p.oa_max = warp_max(oa, active);
+    p.ob_min = warp_min(ob, active);
+    p.ob_max = warp_max(ob, active);
+    p.dk_min = warp_min(dk, active);
+    p.dk_max = warp_max(dk, active);
+    p.o_abs = fmaxf(fmaxf(fmaxf(fabsf(p.zo_min), fabsf(p.zo_max)), fmaxf(fabsf(p.oa_min), fabsf(p.oa_max))),
+                    fmaxf(fabsf(p.ob_min), fabsf(p.ob_max)));
+    p.s_abs = 1.f + fmaxf(fmaxf(fabsf(p.sa_min), fabsf(p.sa_max)), fmaxf(fabsf(p.sb_min), fabsf(p.sb_max)));
+    return true;
+}
+
+// Can a ray of the packet meet child `c` of wide node `id` between depths
+// lo_t and hi_t? t_in: a lower bound on the depths inside the box. Margins of
+// 2e-6 of the coordinates involved cover the rounding of every step, and
+// comparisons with NaN keep the child.
+__device__ __forceinline__ bool packet_child(const WideNode* wide, int id, int c, const Packet& p, float lo_t,
+                                             float hi_t, int& child, float& t_in) {
+    const float* w = reinterpret_cast<const float*>(wide + id) + c;   // row r, child c at w[4 r]
+    const float lok = __ldg(w + 4 * p.k), hik = __ldg(w + 4 * (p.k + 3));
+    const float loa = __ldg(w + 4 * p.a), hia = __ldg(w + 4 * (p.a + 3));
+    const float lob = __ldg(w + 4 * p.b), hib = __ldg(w + 4 * (p.b + 3));
+    child = __ldg(reinterpret_cast<const int*>(w) + 24);
+    if (child == kNoChild) return false;
+    const float ez = 2e-6f * (fmaxf(fabsf(lok), fabsf(hik)) + p.o_abs);
+    const float zn = p.sign > 0.f ? lok : -hik, zf = p.sign > 0.f ? hik : -lok;
+    const float z1 = fmaxf(fmaxf(zn - p.zo_max - ez, 0.f), lo_t * p.dk_min);
+    const float z2 = fminf(zf - p.zo_min + ez, hi_t * p.dk_max);
+    t_in = z1 / p.dk_max;
+    if (z2 < z1) return false;
+    const float e = 2e-6f * (p.o_abs + p.s_abs * z2);
+    const float a_lo = p.oa_min + fminf(p.sa_min * z1, p.sa_min * z2), a_hi = p.oa_max + fmaxf(p.sa_max * z1, p.sa_max * z2);
+    const float b_lo = p.ob_min + fminf(p.sb_min * z1, p.sb_min * z2), b_hi = p.ob_max + fmaxf(p.sb_max * z1, p.sb_max * z2);
+    return !(a_hi + e < loa || a_lo - e > hia || b_hi + e < lob || b_lo - e > hib);
+}
+
+// One round for a packet of rays (32 lanes together): the hierarchy is walked
+// once for the warp, 8 nodes a step with one child box per lane against the
+// packet's bounds, and the leaves that remain are tested in batches of 32:
+// their records are fetched one per lane (64 B each, in flight together) and
+// staged in shared memory, put in the order in which the middle ray meets
+// their planes, and then every ray tests every one. What is left per ray is
+// the surfel test itself. Returns 0, or 1 if the stack overflowed, or 2 if
+// the packet gave up (nothing is kept then; the caller walks per ray).
+template <class KB, bool STATS = false>
+__device__ __forceinline__ int collect_packet(const SceneView& S, const Ray& ray, const TraceParams& P,
+                                              uint64_t last_key, int32_t last_u, KB& kb, bool active,
+                                              PacketScratch& ws, TraceStats* ts = nullptr) {
+    Packet pk;
+    if (!make_packet(ray, active, pk)) return 2;
+    const int lane = threadIdx.x & 31;
+    const unsigned lt = (1u << lane) - 1u;
+    {
+        const unsigned on = __ballot_sync(kFullWarp, active);
+        const int mid = (on >> 18) & 1u ? 18 : __ffs(on) - 1;   // lane 18: inside a 4 x 8 or 8 x 4 tile
+        if (lane == mid) {
+            ws.mid[0] = ray.o.x; ws.mid[1] = ray.o.y; ws.mid[2] = ray.o.z;
+            ws.mid[3] = ray.d.x; ws.mid[4] = ray.d.y; ws.mid[5] = ray.d.z;
+        }
+        if (lane == 0) ws.stack[0] = make_uint2(0u, 0u);
+    }
+    __syncwarp();
+    const float t_lo = key_depth(last_key);
+    const float lo_t = fmaxf(warp_min(t_lo - tslack(t_lo), active), 0.f);
+    float t_hi = P.t_max;
+    float hi_t = P.t_max + tslack(P.t_max);
+    int sp = 1, nleaf = 0, status = 0, batches = 0, hits = 0;
+    int visits = visit_cap(S);
+    while (sp > 0 || nleaf > 0) {
+        if (nleaf < 32 && sp > 0) {
+            // near the stack's end only its top is taken, as a plain depth-first walk would
+            const int take = min(sp, sp <= kPacketStack - 96 ? 8 : 1);
+            visits -= take;
+            const int g = lane >> 2;
+            uint2 ent = make_uint2(0u, 0x7f800000u);
+            bool in = g < take;
+            if (in) ent = ws.stack[sp - 1 - g];
+            in = in && __uint_as_float(ent.y) <= hi_t;
+            sp -= take;
+            int child = kNoChild;
+            float t_in = 0.f;
+            if (in) in = packet_child(S.wide, (int)ent.x, lane & 3, pk, lo_t, hi_t, child, t_in);
+            if (STATS && active) ts->nodes += take;
+            const unsigned leaves = __ballot_sync(kFullWarp, in && child < 0);
+            if (in && child < 0) ws.leaf[nleaf + __popc(leaves & lt)] = (uint32_t)~child;
+            nleaf += __popc(leaves);
+            const bool inner = in && child >= 0;
+            const unsigned push = __ballot_sync(kFullWarp, inner);
+            // farther siblings lie deeper, and so do the children of nodes farther down the stack
+            const float td = inner ? t_in : -1.f;
+            int deeper = __popc((push >> (4 * g)) >> 4);
+#pragma unroll
+            for (int x = 1; x < 4; ++x) {
+                const float to = __shfl_xor_sync(kFullWarp, td, x);
+                deeper += to > td || (to == td && (lane ^ x) > lane) ? 1 : 0;
+            }
+            if (sp + __popc(push) > kPacketStack || visits < 0) {
+                status = 1;
+                break;
+            }
+            __syncwarp();   // the popped entries have been read
+            if (inner) ws.stack[sp + deeper] = make_uint2((uint32_t)child, __float_as_uint(t_in));
+            sp += __popc(push);
+            __syncwarp();
+            continue;
+        }
+        const int cnt = min(nleaf, 32);
+        uint32_t key = 0xffffffe0u | (uint32_t)lane;
+        if (lane < cnt) {
+            const int32_t m = (int32_t)ws.leaf[lane];
+            const float4* R = S.rec + (int64_t)m * kRecF4;
+            const float4 r0 = ldg4(R), r1 = ldg4(R + 1), r2 = ldg4(R + 2);
+            float4 r3 = ldg4(R + 3);
+            const f3 n3 = mk3(r3.x, r3.y, r3.z), w = mk3(r0.x - ws.mid[0], r0.y - ws.mid[1], r0.z - ws.mid[2]);
+            const float tau = __fdividef(dot3(n3, w), dot3(n3, mk3(ws.mid[3], ws.mid[4], ws.mid[5])));
+            if (tau > 0.f) key = (__float_as_uint(tau) & ~31u) | (uint32_t)lane;   // order only: any value will do
+            else key = (uint32_t)lane;
+            r3.w = __int_as_float(m);
+            ws.rec[lane * 4] = r0;
+            ws.rec[lane * 4 + 1] = r1;
+            ws.rec[lane * 4 + 2] = r2;
+            ws.rec[lane * 4 + 3] = r3;
+        }
+        // the leaves behind the batch move to the front
+        const uint32_t rest = 32 + lane < nleaf ? ws.leaf[32 + lane] : 0u;
+        __syncwarp();
+        if (32 + lane < nleaf) ws.leaf[lane] = rest;
+        nleaf -= cnt;
+        // bitonic sort of the lanes' keys
+#pragma unroll
+        for (int size = 2; size <= 32; size <<= 1)
+#pragma unroll
+            for (int step = size >> 1; step > 0; step >>= 1) {
+                const uint32_t other = __shfl_xor_sync(kFullWarp, key, step);
+                const bool up = ((lane & size) == 0) == ((lane & step) == 0);
+                key = up ? min(key, other) : max(key, other);
+            }
+        for (int i = 0; i < cnt; ++i) {
+            const float4* R = ws.rec + 4 * (__shfl_sync(kFullWarp, key, i) & 31u);
+            if (active) {
+                const float4 r3 = R[3];
+                hits += leaf_insert<KB, STATS>(S, ray, P, __float_as_int(r3.w), R[0], R[1], R[2], r3, last_key, last_u,
+                                               kb, t_hi, ts);
             }
         }
-#pragma unroll
-        for (int k = 0; k < 4; ++k)
-            if (t[k] != INFINITY) ni = c[k];
+        const float hi = __uint_as_float(__reduce_max_sync(kFullWarp, active ? __float_as_uint(t_hi) : 0u));
+        hi_t = hi + tslack(hi);
+        // a packet whose leaves miss nearly all of its rays is no packet
+        if (++batches % 16 == 0 && __reduce_add_sync(kFullWarp, hits) < 20 * batches) {
+            status = 2;
+            break;
+        }
+        __syncwarp();
     }
-    return ok;
+    __syncwarp();
+    return status;
+}
+
+// One round by the walk that suits the warp's rays: the packet walk where
+// they run together (PACKET), else one stack per ray.
+template <bool PACKET, class KB, bool STATS = false>
+__device__ __forceinline__ bool collect(const SceneView& S, const Ray& ray, const TraceParams& P, uint64_t last_key,
+                                        int32_t last_u, float T, KB& kb, bool active, bool& packet, float4* scratch,
+                                        TraceStats* ts = nullptr) {
+    kb.open(S.n, T, P.T_min);
+    if (PACKET && packet) {
+        const int status = collect_packet<KB, STATS>(S, ray, P, last_key, last_u, kb, active,
+                                                     *reinterpret_cast<PacketScratch*>(scratch), ts);
+        if (status != 2) return status == 0;
+        packet = false;   // the later rounds of the same rays walk per ray at once
+        kb.open(S.n, T, P.T_min);
+    }
+    return collect_round<KB, STATS>(S, ray, P, last_key, last_u, kb, active, scratch, ts);
 }
 
 // Full forward march of one ray: rounds of collect + blend until the
 // transmittance drops below T_min or no further hit exists.
-template <int K, int FB>
+template <int FB>
 struct MarchState {
     float C[FB];
     float D, T;
     int nh;
+    __device__ __forceinline__ void init() {
+#pragma unroll
+        for (int c = 0; c < FB; ++c) C[c] = 0.f;
+        D = 0.f;
+        T = 1.f;
+        nh = 0;
+    }
 };
 
 // The traced channels f[0..fc) of one surfel, zero beyond fc; as 8-byte
@@ -540,67 +724,67 @@ __device__ __forceinline__ void load_channels(const float* __restrict__ f, int f
 }
 
 // Blend the round's buffered hits in order (Eq. 2, Eq. 8) until the
-// transmittance drops below T_min (the crossing hit included). Returns true
-// when the ray is done: terminated, or fewer than K hits were left; else
-// (last_key, last_u) move to the buffer's last entry (its key and user
-// index) for the next round.
-template <int K, int FB, class KB>
-__device__ __forceinline__ bool blend_round(const SceneView& S, const TraceParams& P, const KB& kb,
-                                            MarchState<K, FB>& st, int32_t* ids, int max_ids, uint64_t& last_key,
+// transmittance drops below T_min (the crossing hit included). Each hit is
+// recomputed from its record, with the same arithmetic. Returns true when
+// the ray is done: terminated, or no hit was left outside the buffer; else
+// (last_key, last_u) move to the buffer's last entry for the next round.
+template <int FB, class KB>
+__device__ __forceinline__ bool blend_round(const SceneView& S, const Ray& ray, const TraceParams& P, const KB& kb,
+                                            MarchState<FB>& st, int32_t* ids, int max_ids, uint64_t& last_key,
                                             int32_t& last_u) {
     bool done = false;
+    float kh = 0.f, kl = 0.f;
+    int32_t u = 0;
     for (int j = 0; j < kb.cnt && !done; ++j) {
-        const float a = kb.a_at(j);
         const int32_t m = kb.m_at(j);
-        const float w = __fmul_rn(st.T, a);
+        const float4* R = S.rec + (int64_t)m * kRecF4;
+        const float4 r0 = ldg4(R), r1 = ldg4(R + 1), r2 = ldg4(R + 2), r3 = ldg4(R + 3);
         float fv[FB];
         load_channels<FB>(S.feat + (int64_t)m * S.F + P.off, P.fc, ((S.F | P.off) & 1) == 0, fv);
+        float a;
+        surfel_hit<false>(r0, r1, r2, r3, ray, P.alpha_min, P.alpha_max, kh, kl, a, nullptr);
+        u = __float_as_int(r2.w);
+        const float w = __fmul_rn(st.T, a);
 #pragma unroll
         for (int c = 0; c < FB; ++c)
             if (c < P.fc) st.C[c] = __fmaf_rn(w, fv[c], st.C[c]);
-        st.D = __fmaf_rn(w, key_depth(kb.key_at(j)), st.D);
+        st.D = __fmaf_rn(w, kh + 0.0f, st.D);
         st.T = __fmul_rn(st.T, __fsub_rn(1.0f, a));
-        if (ids != nullptr && st.nh < max_ids) ids[st.nh] = __float_as_int(__ldg(&S.rec[(int64_t)m * kRecF4 + 2].w));
+        if (ids != nullptr && st.nh < max_ids) ids[st.nh] = u;
         st.nh++;
         if (st.T < P.T_min) done = true;
     }
     if (!done) {
-        if (kb.cnt < K) {
+        if (!kb.closed()) {
             done = true;
         } else {
-            last_key = kb.tail_key;
-            last_u = uid_of(S.rec, kb.tail_m);
+            last_key = depth_key(kh, kl);
+            last_u = u;
         }
     }
     return done;
 }
 
-// WARP = true: all 32 lanes of the warp call this together (lanes without a
-// ray pass live = false) and traverse warp-coherently.
-template <int K, int FB, bool WARP, bool STATS = false>
+// The rounds of one ray until it is done. All 32 lanes of the warp call this
+// together (lanes without a ray pass live = false).
+template <int FB, bool PACKET, int CAP = kBufferCap, bool STATS = false>
 __device__ __forceinline__ bool march_forward(const SceneView& S, const Ray& ray, const TraceParams& P,
-                                              MarchState<K, FB>& st, int32_t* ids, int max_ids,
-                                              bool live = true, TraceStats* ts = nullptr) {
-#pragma unroll
-    for (int c = 0; c < FB; ++c) st.C[c] = 0.f;
-    st.D = 0.f;
-    st.T = 1.f;
-    st.nh = 0;
+                                              MarchState<FB>& st, int32_t* ids, int max_ids, bool live,
+                                              float4* scratch, TraceStats* ts = nullptr) {
+    st.init();
     bool ok = true;
     if (S.n == 0) return ok;
     uint64_t last_key = depth_key(P.t_min, 0.f);
     int32_t last_u = INT32_MAX;
-    KBuffer<K, trace_threads<K>()> kb;
+    KBuffer<CAP> kb;
     kb.bind();
-    bool done = !live;
-    while (WARP ? __any_sync(kFullWarp, !done) : !done) {
+    bool done = !live, packet = true;
+    while (__any_sync(kFullWarp, !done)) {
         if (STATS && !done) ts->rounds++;
-        if (WARP)
-            ok &= collect_round_warp<decltype(kb), STATS>(S, ray, P, last_key, last_u, kb, !done, ts);
-        else
-            ok &= collect_round<decltype(kb), STATS>(S, ray, P, last_key, last_u, kb, ts);
+        ok &= collect<PACKET, KBuffer<CAP>, STATS>(S, ray, P, last_key, last_u, st.T, kb, !done, packet,
+                                                         scratch, ts);
         if (done) continue;
-        done = blend_round<K, FB>(S, P, kb, st, ids, max_ids, last_key, last_u);
+        done = blend_round<FB>(S, ray, P, kb, st, ids, max_ids, last_key, last_u);
     }
     return ok;
 }

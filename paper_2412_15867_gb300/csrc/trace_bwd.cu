@@ -11,7 +11,7 @@
 namespace irgs {
 namespace {
 
-constexpr int kBwdThreads = 128;
+constexpr int kBwdThreads = kTraceThreads;
 
 // Which rays a launch handles.
 enum BwdMode {
@@ -44,21 +44,19 @@ __device__ __forceinline__ void load_ray_grad(RayGrad<FB>& g, int64_t q, const T
     g.Tfin = 1.0f - out_opac[q];
 }
 
-template <int K, int FB, bool WARP, int MODE>
+template <int FB, bool PACKET, int MODE>
 __global__ void __launch_bounds__(kBwdThreads) k_trace_backward(
     SceneView S, const float* __restrict__ ro, const float* __restrict__ rd, int64_t R, TraceParams P,
     const float* __restrict__ out_feat, const float* __restrict__ out_depth, const float* __restrict__ out_opac,
     const int32_t* __restrict__ out_nhits, const int32_t* __restrict__ hit_ids, int max_ids,
     const float* __restrict__ g_featv, const float* __restrict__ g_depthv, const float* __restrict__ g_opacv,
     float* __restrict__ acc_rows) {
-    static_assert(kBwdThreads == trace_threads<K>(), "k-buffer slots are laid out per block thread");
-    __shared__ float4 rows_all[kBwdThreads * GradRow<FB>::kStride / 4];
-    float* rows = reinterpret_cast<float*>(rows_all) + (threadIdx.x & ~31) * GradRow<FB>::kStride;
+    float4* scratch = warp_memory<MODE == kListed ? 32 * GradRow<FB>::kStride / 4 : replay_f4<FB, PACKET>()>();
     const int64_t r = blockIdx.x * (int64_t)kBwdThreads + threadIdx.x;
     if (S.n == 0) return;
     const int nh_total = r < R ? out_nhits[r] : 0;
     const bool mine = nh_total > 0 && (MODE == kReplayAll || (MODE == kListed) == (nh_total <= max_ids));
-    if (MODE == kListed || !WARP) {
+    if (MODE == kListed) {
         if (!mine) return;
     } else if (!__any_sync(kFullWarp, mine)) {
         return;   // the whole warp has nothing to replay
@@ -70,10 +68,10 @@ __global__ void __launch_bounds__(kBwdThreads) k_trace_backward(
     load_ray_grad<FB>(g, q, P, out_feat, out_depth, out_opac, g_featv, g_depthv, g_opacv);
     if (MODE == kListed) {
         listed_backward<FB>(S, ray, P, hit_ids + q * (int64_t)max_ids, nh_total, g.Cf, g.Df, g.Tfin, g.gC, g.gD,
-                            g.gO, acc_rows, rows);
+                            g.gO, acc_rows, reinterpret_cast<float*>(scratch));
     } else {
-        const bool ok = march_backward<K, FB, WARP>(S, ray, P, mine, nh_total, g.Cf, g.Df, g.Tfin, g.gC, g.gD, g.gO,
-                                                    acc_rows, rows);
+        const bool ok = march_backward<FB, PACKET>(S, ray, P, mine, nh_total, g.Cf, g.Df, g.Tfin, g.gC, g.gD, g.gO, acc_rows,
+                                                   scratch);
         if (mine && !ok) atomicOr(S.status, kErrStackOverflow);
     }
 }
@@ -90,7 +88,7 @@ struct BwdArgs {
     float *gm, *gq, *gs, *gop, *gfe;
 };
 
-template <int K, int FB, bool WARP>
+template <int FB, bool PACKET>
 cudaError_t launch(const SceneView& S, const TraceParams& P, const BwdArgs& a, cudaStream_t st) {
     constexpr int N = GradRow<FB>::N;
     const size_t bytes = sizeof(float) * N * (size_t)(S.n > 0 ? S.n : 1);
@@ -102,7 +100,7 @@ cudaError_t launch(const SceneView& S, const TraceParams& P, const BwdArgs& a, c
         const int64_t blocks = (a.R + kBwdThreads - 1) / kBwdThreads;
         const unsigned grid = (unsigned)blocks;
 #define IRGS_BWD(MODE)                                                                                  \
-    k_trace_backward<K, FB, WARP, MODE><<<grid, kBwdThreads, 0, st>>>(S, a.ro, a.rd, a.R, P, a.feat, a.depth, \
+    k_trace_backward<FB, PACKET, MODE><<<grid, kBwdThreads, 0, st>>>(S, a.ro, a.rd, a.R, P, a.feat, a.depth, \
                                                                       a.opac, a.nhits, a.ids, a.max_ids, a.gf, \
                                                                       a.gd, a.go, acc_rows)
         if (a.ids != nullptr) {
@@ -123,16 +121,11 @@ cudaError_t launch(const SceneView& S, const TraceParams& P, const BwdArgs& a, c
     return e != cudaSuccess ? e : ef;
 }
 
-template <int K, bool WARP>
+template <bool PACKET>
 cudaError_t launch_f(const SceneView& S, const TraceParams& P, const BwdArgs& a, cudaStream_t st) {
-    if (P.fc <= 3) return launch<K, 3, WARP>(S, P, a, st);
-    if (P.fc <= 10) return launch<K, 10, WARP>(S, P, a, st);
-    return launch<K, 16, WARP>(S, P, a, st);
-}
-
-template <int K>
-cudaError_t launch_k(bool warp, const SceneView& S, const TraceParams& P, const BwdArgs& a, cudaStream_t st) {
-    return warp ? launch_f<K, true>(S, P, a, st) : launch_f<K, false>(S, P, a, st);
+    if (P.fc <= 3) return launch<3, PACKET>(S, P, a, st);
+    if (P.fc <= 10) return launch<10, PACKET>(S, P, a, st);
+    return launch<16, PACKET>(S, P, a, st);
 }
 
 }  // namespace
@@ -148,13 +141,8 @@ irgs_status launch_trace_backward(const SceneView& S, const int32_t* perm, const
     const BwdArgs a{perm,  ro,     rd,      R,       feat,     depth,     opac,      nhits,     hit_ids,
                     hit_ids != nullptr ? max_hit_ids : 0, g_feat, g_depth, g_opac, g_means, g_quats, g_scales,
                     g_opacity, g_features};
-    const bool warp = (p.flags & IRGS_FLAG_PER_THREAD) == 0u;
-    cudaError_t e;
-    switch (p.k) {
-        case 8: e = launch_k<8>(warp, S, P, a, st); break;
-        case 16: e = launch_k<16>(warp, S, P, a, st); break;
-        default: return IRGS_ERR_UNSUPPORTED;
-    }
+    const bool packet = (p.flags & IRGS_FLAG_PER_THREAD) == 0u;
+    const cudaError_t e = packet ? launch_f<true>(S, P, a, st) : launch_f<false>(S, P, a, st);
     if (e == cudaErrorMemoryAllocation) return IRGS_ERR_OOM;
     return e == cudaSuccess ? IRGS_OK : IRGS_ERR_CUDA;
 }

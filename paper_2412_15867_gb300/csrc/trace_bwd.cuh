@@ -196,37 +196,42 @@ __device__ __forceinline__ void backward_hit(const SceneView& S, const Ray& ray,
     st.T = __fmul_rn(st.T, __fsub_rn(1.0f, a));
 }
 
-// Replay of one ray (all 32 lanes together when WARP): the march is repeated
-// with the same traversal and arithmetic as the forward, capped at nh_total
-// composited hits; Cf, Df, Tfin are the forward's outputs and gC, gD, gO the
-// upstream gradients. rows is this warp's [32][N+1] shared scratch. Returns
-// false if a traversal stack overflowed.
-template <int K, int FB, bool WARP>
+// Replay of one ray (all 32 lanes together): the march is repeated with the
+// same order and arithmetic as the forward, capped at nh_total composited
+// hits; Cf, Df, Tfin are the forward's outputs and gC, gD, gO the upstream
+// gradients. scratch is this warp's working memory (replay_f4): the walk's,
+// and between the walks the gradient rows' exchange. Returns false if a
+// traversal stack overflowed.
+template <int FB, bool PACKET>
+__host__ __device__ constexpr int replay_f4() {
+    return scratch_f4<PACKET>() > 32 * GradRow<FB>::kStride / 4 ? scratch_f4<PACKET>() : 32 * GradRow<FB>::kStride / 4;
+}
+template <int FB, bool PACKET>
 __device__ __forceinline__ bool march_backward(const SceneView& S, const Ray& ray, const TraceParams& P, bool live,
                                                int nh_total, const float (&Cf)[FB], float Df, float Tfin,
                                                const float (&gC)[FB], float gD, float gO,
-                                               float* __restrict__ acc_rows, float* rows) {
+                                               float* __restrict__ acc_rows, float4* scratch) {
     BwdAcc<FB> st;
     st.init();
+    float* rows = reinterpret_cast<float*>(scratch);
     int nh = 0;
     uint64_t last_key = depth_key(P.t_min, 0.f);
     int32_t last_u = INT32_MAX;
-    KBuffer<K, trace_threads<K>()> kb;
+    KBuffer<kBufferCap> kb;
     kb.bind();
-    bool ok = true, done = !live;
-    while (WARP ? __any_sync(kFullWarp, !done) : !done) {
-        if (WARP)
-            ok &= collect_round_warp(S, ray, P, last_key, last_u, kb, !done);
-        else
-            ok &= collect_round(S, ray, P, last_key, last_u, kb);
+    bool ok = true, done = !live, packet = true;
+    while (__any_sync(kFullWarp, !done)) {
+        ok &= collect<PACKET>(S, ray, P, last_key, last_u, st.T, kb, !done, packet, scratch);
         if (done) continue;
         for (int j = 0; j < kb.cnt && nh < nh_total; ++j, ++nh)
             backward_hit<FB>(S, ray, P, kb.m_at(j), st, Cf, Df, Tfin, gC, gD, gO, acc_rows, rows);
-        if (nh >= nh_total || kb.cnt < K) {
+        if (nh >= nh_total || !kb.closed()) {
             done = true;
         } else {
-            last_key = kb.tail_key;
-            last_u = uid_of(S.rec, kb.tail_m);
+            const int32_t m = kb.m_at(kb.cnt - 1);
+            const float2 t = tie_of(S.rec, m, ray.o, ray.d, ray.inv_dd);
+            last_key = depth_key(__uint_as_float(kb.tail), t.x);
+            last_u = __float_as_int(t.y);
         }
     }
     return ok;
