@@ -375,7 +375,7 @@ __global__ void k_relight_gen(EnvMaps M, const float* __restrict__ xg, int64_t p
     val[i] = (int32_t)i;
 }
 
-__global__ void __launch_bounds__(kRelightThreads, 6) k_relight_trace(SceneView S, TraceParams P,
+__global__ void __launch_bounds__(kRelightThreads, kRayBlocks) k_relight_trace(SceneView S, TraceParams P,
                                                                       const float* __restrict__ xg, int64_t p0,
                                                                       int Sn, const float4* __restrict__ dir,
                                                                       const int32_t* __restrict__ order,
@@ -409,7 +409,7 @@ enum RelightRound { kRelFirst = 0, kRelLast = 1 };
 constexpr int kRelightStateF4 = 4;
 
 template <int MODE>
-__global__ void __launch_bounds__(kRelightThreads, 6) k_relight_round(
+__global__ void __launch_bounds__(kRelightThreads, kRayBlocks) k_relight_round(
     SceneView S, TraceParams P, const float* __restrict__ xg, int64_t p0, int Sn, const float4* __restrict__ dir,
     const int32_t* __restrict__ order, int64_t rays, float4* __restrict__ res, const int32_t* __restrict__ list,
     const uint32_t* __restrict__ count, float4* __restrict__ state, uint32_t* __restrict__ flags) {
@@ -445,7 +445,7 @@ __global__ void __launch_bounds__(kRelightThreads, 6) k_relight_round(
         last_u = __float_as_int(w[12]);
     }
     const Ray ray = make_ray(ld3r(xg, p0 + i / Sn), mk3(d4.x, d4.y, d4.z));
-    KBuffer<kBufferCap> kb;
+    KBuffer<kRayCap> kb;
     kb.bind();
     float4* scratch = warp_scratch<false>();
     bool ok = true, done = !live, packet = false;

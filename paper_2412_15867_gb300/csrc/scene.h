@@ -149,6 +149,23 @@ cudaError_t flags_to_list(uint32_t* flags, int64_t m, uint32_t* sums, int32_t* l
                           cudaStream_t st);
 
 // trace_fwd.cu
+// The width of the pixel rows that a batch of rays seems to hold, in a device
+// word (0: none) that lives until the object's end, stream-ordered. get() is
+// nullptr where no hint is wanted or none can be had.
+class RowWidth {
+  public:
+    RowWidth(const float* rd, int64_t R, bool wanted, cudaStream_t st);
+    ~RowWidth();
+    RowWidth(const RowWidth&) = delete;
+    RowWidth& operator=(const RowWidth&) = delete;
+    const int32_t* get() const { return width_; }
+
+  private:
+    int32_t* width_ = nullptr;
+    cudaStream_t st_;
+};
+constexpr int64_t kRowMinRays = 1024;   // fewer rays: the look at the rows costs more than it gives
+
 irgs_status launch_trace_forward(const SceneView& sv, const float* ro, const float* rd, int64_t R,
                                  const irgs_trace_params& p, float* feat, float* depth, float* opac,
                                  int32_t* nhits, int32_t* ids, int32_t max_ids, cudaStream_t st);

@@ -87,7 +87,7 @@ __global__ void k_camera_rays(irgs_camera c, int64_t first, int64_t count, float
     rd[3 * i] = d.x; rd[3 * i + 1] = d.y; rd[3 * i + 2] = d.z;
 }
 
-__global__ void __launch_bounds__(kServeThreads) k_serve(ServeArgs A) {
+__global__ void __launch_bounds__(kServeThreads, kPacketBlocks) k_serve(ServeArgs A) {
     __shared__ int s_tile;
     const int n_tiles = A.header[1];
     for (;;) {

@@ -73,7 +73,7 @@ __global__ void k_wave_gen(const float* __restrict__ xg, const float* __restrict
 // With SAVE the blended hit ids (user order, -1 terminated) and the hit
 // counts are kept for the backward.
 template <bool SAVE>
-__global__ void __launch_bounds__(kWaveThreads, 6) k_wave_trace(SceneView S, TraceParams P,
+__global__ void __launch_bounds__(kWaveThreads, kRayBlocks) k_wave_trace(SceneView S, TraceParams P,
                                                                 const float* __restrict__ xg, int64_t p0, int St,
                                                                 const float4* __restrict__ dir,
                                                                 const int32_t* __restrict__ order, int64_t rays,
@@ -111,7 +111,7 @@ enum WaveRound { kWaveFirst = 0, kWaveLast = 1 };
 constexpr int kWaveStateF4 = 3;   // C[3], D, T, hit count, next key (2 words), next user index
 
 template <bool SAVE, int MODE>
-__global__ void __launch_bounds__(kWaveThreads, 6) k_wave_round(
+__global__ void __launch_bounds__(kWaveThreads, kRayBlocks) k_wave_round(
     SceneView S, TraceParams P, const float* __restrict__ xg, int64_t p0, int St, const float4* __restrict__ dir,
     const int32_t* __restrict__ order, int64_t rays, float4* __restrict__ res, int32_t* __restrict__ nh,
     int32_t* __restrict__ ids, int max_ids, const int32_t* __restrict__ list, const uint32_t* __restrict__ count,
@@ -143,7 +143,7 @@ __global__ void __launch_bounds__(kWaveThreads, 6) k_wave_round(
         last_u = __float_as_int(c.x);
     }
     int32_t* my_ids = SAVE ? ids + i * (int64_t)max_ids : nullptr;
-    KBuffer<kBufferCap> kb;
+    KBuffer<kRayCap> kb;
     kb.bind();
     float4* scratch = warp_scratch<false>();
     bool ok = true, done = !live, packet = false;

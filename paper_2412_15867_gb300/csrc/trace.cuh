@@ -185,11 +185,15 @@ __device__ __forceinline__ float key_depth(uint64_t k) { return __uint_as_float(
 // are laid out per block thread).
 constexpr int kTraceThreads = 128;
 
-// Entries of the k-buffer. Results do not depend on it (the buffer holds the
-// nearest hits after the last blended one, whatever its size), so the size a
-// caller asks for does not select code. 32 entries hold every hit of most
-// rays that the transmittance cut below leaves.
-constexpr int kBufferCap = 32;
+// Entries of the k-buffer, for packets and for rays on their own. Results do
+// not depend on it (the buffer holds the nearest hits after the last blended
+// one, whatever its size), so the size a caller asks for selects no code.
+constexpr int kPacketCap = 32;
+constexpr int kRayCap = 24;
+constexpr int kPacketBlocks = 4;   // resident blocks per SM that the kernels are compiled for
+constexpr int kRayBlocks = 6;
+template <bool PACKET>
+__host__ __device__ constexpr int walk_cap() { return PACKET ? kPacketCap : kRayCap; }
 
 // Exact depth remainder kl and user index of surfel m, whose hit at the same
 // rounded depth ties with another: out of line, since ties are rare.
@@ -268,10 +272,29 @@ struct KBuffer {
         } else {
             ++cnt;
         }
-        for (; j >= 0; --j) {
-            const uint2 v = e[j * kTraceThreads];
-            if (!before(kb, kl, u, v, rec, ray)) break;
-            e[(j + 1) * kTraceThreads] = v;
+        // entries behind the new one move up, four at a time: their loads are in
+        // flight together (one by one, a warp waits out a shared-memory round
+        // trip per entry of its longest shift)
+        bool found = false;
+        while (!found && j >= 0) {
+            uint2 v[4];
+#pragma unroll
+            for (int i = 0; i < 4; ++i) v[i] = j >= i ? e[(j - i) * kTraceThreads] : make_uint2(0u, 0u);
+            int moved = 0;   // entries are in order: those behind the new one come first
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                if (j >= i && kb < v[i].x) {
+                    e[(j - i + 1) * kTraceThreads] = v[i];
+                    ++moved;
+                }
+            }
+            j -= moved;
+            if (moved == 4) continue;
+            found = j < 0 || !before(kb, kl, u, e[j * kTraceThreads], rec, ray);
+            if (!found) {   // a tie, and the entry comes after
+                e[(j + 1) * kTraceThreads] = e[j * kTraceThreads];
+                --j;
+            }
         }
         uint32_t q = 0u;
         if (id_mask == 0xffffffu) q = (uint32_t)fminf(fmaxf(-16.f * __log2f(1.f - alpha), 0.f), 255.f);
@@ -298,7 +321,7 @@ struct TraceStats {
 // Shared working memory of one warp. The packet walk keeps its stack, its
 // pending leaves and the records of a batch of 32 leaves; the per-ray walk
 // its leaf queues (in the records' place).
-constexpr int kPacketStack = 192;
+constexpr int kPacketStack = 184;
 constexpr int kLeafQueue = 12;   // pending leaves per ray
 struct PacketScratch {
     float4 rec[32 * kRecF4];
@@ -313,6 +336,23 @@ static_assert(sizeof(PacketScratch) % sizeof(float4) == 0, "per-warp slots stay 
 // float4s of working memory that one warp's walk takes.
 template <bool PACKET>
 __host__ __device__ constexpr int scratch_f4() { return PACKET ? (int)(sizeof(PacketScratch) / sizeof(float4)) : kQueueF4; }
+
+// Ray number of slot t when warps are made of 4 x 8 pixel tiles of an image
+// of *width columns (rays row by row; nullptr or 0: the rays' own order). A
+// packet of a tile meets a third of the leaves that one of a row strip
+// does. A permutation of [0, R): the last rows that do not fill a band of
+// eight keep their order.
+__device__ __forceinline__ int64_t tiled_ray(int64_t t, int64_t R, const int32_t* __restrict__ width) {
+    const uint32_t W = width != nullptr ? (uint32_t)__ldg(width) : 0u;
+    if (W == 0u) return t;
+    const int64_t band = t / (8 * (int64_t)W) * (8 * (int64_t)W);
+    if (band + 8 * (int64_t)W > R) return t;
+    const uint32_t u = (uint32_t)(t - band), full = W / 4 * 32, c = W % 4;   // whole tiles, then the columns left over
+    const uint32_t v = u - full;
+    const uint32_t col = u < full ? u / 32 * 4 + u % 4 : W / 4 * 4 + v % (c != 0u ? c : 1u);
+    const uint32_t row = u < full ? u % 32 / 4 : v / (c != 0u ? c : 1u);
+    return band + (int64_t)row * W + col;
+}
 
 // This warp's part of a block's working memory, F4 float4s per warp.
 template <int F4>
@@ -549,13 +589,43 @@ __device__ __forceinline__ bool packet_child(const WideNode* wide, int id, int c
     return !(a_hi + e < loa || a_lo - e > hia || b_hi + e < lob || b_lo - e > hib);
 }
 
+// Can a ray of the packet meet the support disk of a surfel? The disk against
+// the packet's four side planes, x_j - s x_k sign >= c (or <= c): the largest
+// value of such a form over the disk is its value at the centre plus
+// rho_c |(U.N, V.N)| with U = s_u t_u, V = s_v t_v. The box of a tilted disk is
+// much larger than the disk, so this drops half of the leaves whose boxes
+// the packet meets; the margins are far above the rounding of the test.
+__device__ __forceinline__ bool packet_disk(const Packet& p, const float4& r0, const float4& r1, const float4& r2) {
+    if (!(r1.w >= 0.f)) return false;
+    const f3 mu = mk3(r0.x, r0.y, r0.z), tu = mk3(r1.x, r1.y, r1.z), tv = mk3(r2.x, r2.y, r2.z);
+    const float iu = __fdividef(1.f, dot3(tu, tu)), iv = __fdividef(1.f, dot3(tv, tv));   // s_u^2, s_v^2
+    const float uk = p.sign * axis_of(tu, p.k) * iu, vk = p.sign * axis_of(tv, p.k) * iv;
+    const float mk = p.sign * axis_of(mu, p.k);
+    const float rc2 = r1.w * 1.001f;
+    const float eps = 4e-6f * p.s_abs * (p.o_abs + fabsf(mu.x) + fabsf(mu.y) + fabsf(mu.z));
+    // outside the plane with normal e_j - s e_k by more than the disk's extent
+    auto beyond = [&](float gap, float uj, float vj, float s) {
+        const float a = uj - s * uk, b = vj - s * vk;
+        return gap > eps && (gap - eps) * (gap - eps) > rc2 * (a * a + b * b);
+    };
+    const float ma = axis_of(mu, p.a), ua = axis_of(tu, p.a) * iu, va = axis_of(tv, p.a) * iv;
+    const float mb = axis_of(mu, p.b), ub = axis_of(tu, p.b) * iu, vb = axis_of(tv, p.b) * iv;
+    const float a_lo = p.oa_min - fmaxf(p.sa_min * p.zo_min, p.sa_min * p.zo_max);
+    const float a_hi = p.oa_max - fminf(p.sa_max * p.zo_min, p.sa_max * p.zo_max);
+    const float b_lo = p.ob_min - fmaxf(p.sb_min * p.zo_min, p.sb_min * p.zo_max);
+    const float b_hi = p.ob_max - fminf(p.sb_max * p.zo_min, p.sb_max * p.zo_max);
+    return !(beyond(a_lo - (ma - p.sa_min * mk), ua, va, p.sa_min) || beyond((ma - p.sa_max * mk) - a_hi, ua, va, p.sa_max) ||
+             beyond(b_lo - (mb - p.sb_min * mk), ub, vb, p.sb_min) || beyond((mb - p.sb_max * mk) - b_hi, ub, vb, p.sb_max));
+}
+
 // One round for a packet of rays (32 lanes together): the hierarchy is walked
 // once for the warp, 8 nodes a step with one child box per lane against the
 // packet's bounds, and the leaves that remain are tested in batches of 32:
-// their records are fetched one per lane (64 B each, in flight together) and
-// staged in shared memory, put in the order in which the middle ray meets
-// their planes, and then every ray tests every one. What is left per ray is
-// the surfel test itself. Returns 0, or 1 if the stack overflowed, or 2 if
+// their records are fetched one per lane (64 B each, in flight together),
+// those whose disks miss the packet are dropped, the others staged in shared
+// memory and put in the order in which the middle ray meets their planes, and
+// then every ray tests every one. What is left per ray is the surfel test
+// itself. Returns 0, or 1 if the stack overflowed, or 2 if
 // the packet gave up (nothing is kept then; the caller walks per ray).
 template <class KB, bool STATS = false>
 __device__ __forceinline__ int collect_packet(const SceneView& S, const Ray& ray, const TraceParams& P,
@@ -621,6 +691,7 @@ __device__ __forceinline__ int collect_packet(const SceneView& S, const Ray& ray
         }
         const int cnt = min(nleaf, 32);
         uint32_t key = 0xffffffe0u | (uint32_t)lane;
+        bool keep = false;
         if (lane < cnt) {
             const int32_t m = (int32_t)ws.leaf[lane];
             const float4* R = S.rec + (int64_t)m * kRecF4;
@@ -628,8 +699,9 @@ __device__ __forceinline__ int collect_packet(const SceneView& S, const Ray& ray
             float4 r3 = ldg4(R + 3);
             const f3 n3 = mk3(r3.x, r3.y, r3.z), w = mk3(r0.x - ws.mid[0], r0.y - ws.mid[1], r0.z - ws.mid[2]);
             const float tau = __fdividef(dot3(n3, w), dot3(n3, mk3(ws.mid[3], ws.mid[4], ws.mid[5])));
-            if (tau > 0.f) key = (__float_as_uint(tau) & ~31u) | (uint32_t)lane;   // order only: any value will do
-            else key = (uint32_t)lane;
+            keep = packet_disk(pk, r0, r1, r2);
+            // order only: any value below the dropped lanes' will do
+            if (keep) key = (tau > 0.f && tau < 1e30f ? __float_as_uint(tau) & ~31u : 0u) | (uint32_t)lane;
             r3.w = __int_as_float(m);
             ws.rec[lane * 4] = r0;
             ws.rec[lane * 4 + 1] = r1;
@@ -650,7 +722,8 @@ __device__ __forceinline__ int collect_packet(const SceneView& S, const Ray& ray
                 const bool up = ((lane & size) == 0) == ((lane & step) == 0);
                 key = up ? min(key, other) : max(key, other);
             }
-        for (int i = 0; i < cnt; ++i) {
+        const int kept = __popc(__ballot_sync(kFullWarp, keep));
+        for (int i = 0; i < kept; ++i) {
             const float4* R = ws.rec + 4 * (__shfl_sync(kFullWarp, key, i) & 31u);
             if (active) {
                 const float4 r3 = R[3];
@@ -661,7 +734,7 @@ __device__ __forceinline__ int collect_packet(const SceneView& S, const Ray& ray
         const float hi = __uint_as_float(__reduce_max_sync(kFullWarp, active ? __float_as_uint(t_hi) : 0u));
         hi_t = hi + tslack(hi);
         // a packet whose leaves miss nearly all of its rays is no packet
-        if (++batches % 16 == 0 && __reduce_add_sync(kFullWarp, hits) < 20 * batches) {
+        if (++batches % 16 == 0 && __reduce_add_sync(kFullWarp, hits) < 10 * batches) {
             status = 2;
             break;
         }
@@ -767,7 +840,7 @@ __device__ __forceinline__ bool blend_round(const SceneView& S, const Ray& ray, 
 
 // The rounds of one ray until it is done. All 32 lanes of the warp call this
 // together (lanes without a ray pass live = false).
-template <int FB, bool PACKET, int CAP = kBufferCap, bool STATS = false>
+template <int FB, bool PACKET, int CAP = walk_cap<PACKET>(), bool STATS = false>
 __device__ __forceinline__ bool march_forward(const SceneView& S, const Ray& ray, const TraceParams& P,
                                               MarchState<FB>& st, int32_t* ids, int max_ids, bool live,
                                               float4* scratch, TraceStats* ts = nullptr) {

@@ -50,10 +50,11 @@ __global__ void __launch_bounds__(kBwdThreads) k_trace_backward(
     const float* __restrict__ out_feat, const float* __restrict__ out_depth, const float* __restrict__ out_opac,
     const int32_t* __restrict__ out_nhits, const int32_t* __restrict__ hit_ids, int max_ids,
     const float* __restrict__ g_featv, const float* __restrict__ g_depthv, const float* __restrict__ g_opacv,
-    float* __restrict__ acc_rows) {
+    float* __restrict__ acc_rows, const int32_t* __restrict__ width) {
     float4* scratch = warp_memory<MODE == kListed ? 32 * GradRow<FB>::kStride / 4 : replay_f4<FB, PACKET>()>();
-    const int64_t r = blockIdx.x * (int64_t)kBwdThreads + threadIdx.x;
+    const int64_t t = blockIdx.x * (int64_t)kBwdThreads + threadIdx.x;
     if (S.n == 0) return;
+    const int64_t r = t < R ? tiled_ray(t, R, width) : R;
     const int nh_total = r < R ? out_nhits[r] : 0;
     const bool mine = nh_total > 0 && (MODE == kReplayAll || (MODE == kListed) == (nh_total <= max_ids));
     if (MODE == kListed) {
@@ -99,10 +100,11 @@ cudaError_t launch(const SceneView& S, const TraceParams& P, const BwdArgs& a, c
     if (e == cudaSuccess) {
         const int64_t blocks = (a.R + kBwdThreads - 1) / kBwdThreads;
         const unsigned grid = (unsigned)blocks;
+        const RowWidth w(a.rd, a.R, PACKET, st);
 #define IRGS_BWD(MODE)                                                                                  \
     k_trace_backward<FB, PACKET, MODE><<<grid, kBwdThreads, 0, st>>>(S, a.ro, a.rd, a.R, P, a.feat, a.depth, \
                                                                       a.opac, a.nhits, a.ids, a.max_ids, a.gf, \
-                                                                      a.gd, a.go, acc_rows)
+                                                                      a.gd, a.go, acc_rows, w.get())
         if (a.ids != nullptr) {
             IRGS_BWD(kListed);
             IRGS_BWD(kReplayLong);

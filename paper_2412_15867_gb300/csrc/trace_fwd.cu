@@ -7,18 +7,50 @@
 namespace irgs {
 namespace {
 
+// Rows at least this wide are regrouped (narrower ones are tiles already, or no rows at all).
+constexpr int kMinRowWidth = 32;
+constexpr int kMaxRowWidth = 1 << 15;
+
+// Width of the image whose pixel rows the rays seem to be, else 0: the first
+// neighbours whose directions differ by more than twice the first
+// difference end a row, if the next row starts beside its start. A hint:
+// it only decides which rays share a warp.
+__global__ void __launch_bounds__(1024) k_row_width(const float* __restrict__ rd, int64_t R, int32_t* __restrict__ width) {
+    __shared__ int s_first;
+    if (threadIdx.x == 0) s_first = INT32_MAX;
+    auto diff2 = [&](int64_t i, int64_t j) {
+        const float x = rd[3 * i] - rd[3 * j], y = rd[3 * i + 1] - rd[3 * j + 1], z = rd[3 * i + 2] - rd[3 * j + 2];
+        return x * x + y * y + z * z;
+    };
+    const float unit = diff2(0, 1);
+    const int last = (int)(R - 1 < kMaxRowWidth ? R - 1 : kMaxRowWidth);
+    __syncthreads();
+    for (int i0 = 1; i0 < last; i0 += 1024) {
+        const int i = i0 + threadIdx.x;
+        if (i < last && diff2(i, i + 1) > 4.f * unit) atomicMin(&s_first, i);
+        __syncthreads();
+        if (s_first != INT32_MAX) break;   // the same for every thread: nothing writes it until the next pass
+        __syncthreads();
+    }
+    if (threadIdx.x == 0) {
+        const int64_t w = s_first == INT32_MAX ? 0 : (int64_t)s_first + 1;
+        *width = w >= kMinRowWidth && w < R && diff2(0, w) < 9.f * unit ? (int32_t)w : 0;
+    }
+}
+
 
 template <int FB, bool PACKET>
-__global__ void __launch_bounds__(kTraceThreads, 4) k_trace_forward(SceneView S, const float* __restrict__ ro,
+__global__ void __launch_bounds__(kTraceThreads, kPacketBlocks) k_trace_forward(SceneView S, const float* __restrict__ ro,
                                                                     const float* __restrict__ rd, int64_t R,
                                                                     TraceParams P, float* __restrict__ feat,
                                                                     float* __restrict__ depth,
                                                                     float* __restrict__ opac,
                                                                     int32_t* __restrict__ nhits,
-                                                                    int32_t* __restrict__ ids, int max_ids) {
-    const int64_t r = blockIdx.x * (int64_t)kTraceThreads + threadIdx.x;
-    const bool live = r < R;
-    const int64_t q = live ? r : 0;   // lanes without a ray follow the warp with a dummy ray
+                                                                    int32_t* __restrict__ ids, int max_ids,
+                                                                    const int32_t* __restrict__ width) {
+    const int64_t t = blockIdx.x * (int64_t)kTraceThreads + threadIdx.x;
+    const bool live = t < R;
+    const int64_t r = live ? tiled_ray(t, R, width) : 0, q = r;   // lanes without a ray follow the warp with a dummy ray
     const Ray ray = make_ray(mk3(ro[3 * q], ro[3 * q + 1], ro[3 * q + 2]),
                              mk3(rd[3 * q], rd[3 * q + 1], rd[3 * q + 2]));
     int32_t* my_ids = (ids != nullptr && live) ? ids + r * (int64_t)max_ids : nullptr;
@@ -52,17 +84,19 @@ struct RoundState {
 };
 
 template <int FB, int MODE>
-__global__ void __launch_bounds__(kTraceThreads, 4) k_trace_round(
+__global__ void __launch_bounds__(kTraceThreads, kPacketBlocks) k_trace_round(
     SceneView S, const float* __restrict__ ro, const float* __restrict__ rd, int64_t R, TraceParams P,
     float* __restrict__ feat, float* __restrict__ depth, float* __restrict__ opac, int32_t* __restrict__ nhits,
     int32_t* __restrict__ ids, int max_ids, const int32_t* __restrict__ list, const uint32_t* __restrict__ count,
-    float4* __restrict__ state, uint32_t* __restrict__ flags) {
+    float4* __restrict__ state, uint32_t* __restrict__ flags, const int32_t* __restrict__ width) {
     constexpr int SW = RoundState<FB>::kF4;
     const int64_t t = blockIdx.x * (int64_t)kTraceThreads + threadIdx.x;
     const int64_t n = MODE == kRoundFirst ? R : (int64_t)*count;
     if (__all_sync(kFullWarp, t >= n)) return;   // nothing for this warp
     const bool live = t < n;
-    const int64_t r = live ? (MODE == kRoundFirst ? t : (int64_t)list[t]) : 0;
+    // slot: the ray's place in the order the warps are made in
+    const int64_t slot = live ? (MODE == kRoundFirst ? t : (int64_t)list[t]) : 0;
+    const int64_t r = live ? tiled_ray(slot, R, width) : 0;
     const Ray ray = make_ray(mk3(ro[3 * r], ro[3 * r + 1], ro[3 * r + 2]),
                              mk3(rd[3 * r], rd[3 * r + 1], rd[3 * r + 2]));
     MarchState<FB> st;
@@ -74,7 +108,7 @@ __global__ void __launch_bounds__(kTraceThreads, 4) k_trace_round(
         float w[4 * SW];
 #pragma unroll
         for (int q = 0; q < SW; ++q) {
-            const float4 v = state[r * SW + q];
+            const float4 v = state[slot * SW + q];
             w[4 * q] = v.x; w[4 * q + 1] = v.y; w[4 * q + 2] = v.z; w[4 * q + 3] = v.w;
         }
 #pragma unroll
@@ -86,7 +120,7 @@ __global__ void __launch_bounds__(kTraceThreads, 4) k_trace_round(
         last_u = __float_as_int(w[FB + 5]);
     }
     int32_t* my_ids = (ids != nullptr && live) ? ids + r * (int64_t)max_ids : nullptr;
-    KBuffer<kBufferCap> kb;
+    KBuffer<kPacketCap> kb;
     kb.bind();
     float4* scratch = warp_scratch<true>();
     bool ok = true, done = !live, packet = true;
@@ -117,8 +151,8 @@ __global__ void __launch_bounds__(kTraceThreads, 4) k_trace_round(
 #pragma unroll
         for (int c = FB + 6; c < 4 * SW; ++c) w[c] = 0.f;
 #pragma unroll
-        for (int q = 0; q < SW; ++q) state[r * SW + q] = make_float4(w[4 * q], w[4 * q + 1], w[4 * q + 2], w[4 * q + 3]);
-        flags[r] = 1u;
+        for (int q = 0; q < SW; ++q) state[slot * SW + q] = make_float4(w[4 * q], w[4 * q + 1], w[4 * q + 2], w[4 * q + 3]);
+        flags[slot] = 1u;
     }
 }
 
@@ -128,7 +162,7 @@ constexpr int64_t kRoundMinRays = int64_t(1) << 20;
 template <int FB>
 cudaError_t launch_rounds(const SceneView& S, const float* ro, const float* rd, int64_t R, const TraceParams& P,
                           float* feat, float* depth, float* opac, int32_t* nhits, int32_t* ids, int max_ids,
-                          cudaStream_t st) {
+                          const int32_t* width, cudaStream_t st) {
     constexpr int threads = kTraceThreads;
     constexpr int SW = RoundState<FB>::kF4;
     const int64_t sums = scan_long_words(R + 1);
@@ -148,11 +182,11 @@ cudaError_t launch_rounds(const SceneView& S, const float* ro, const float* rd, 
     e = cudaMemsetAsync(flags, 0, sizeof(uint32_t) * (R + 1), st);
     if (e == cudaSuccess) {
         k_trace_round<FB, kRoundFirst><<<grid, threads, 0, st>>>(S, ro, rd, R, P, feat, depth, opac, nhits, ids,
-                                                                  max_ids, list, count, state, flags);
+                                                                  max_ids, list, count, state, flags, width);
         e = flags_to_list(flags, R, scan_sums, list, count, st);
         if (e == cudaSuccess)
             k_trace_round<FB, kRoundLast><<<grid, threads, 0, st>>>(S, ro, rd, R, P, feat, depth, opac, nhits, ids,
-                                                                    max_ids, list, count, state, flags);
+                                                                    max_ids, list, count, state, flags, width);
         count_launches(2);
     }
     const cudaError_t ef = cudaFreeAsync(base, st);
@@ -163,19 +197,19 @@ cudaError_t launch_rounds(const SceneView& S, const float* ro, const float* rd, 
 template <int FB, bool PACKET>
 cudaError_t launch(const SceneView& S, const float* ro, const float* rd, int64_t R, const TraceParams& P,
                    float* feat, float* depth, float* opac, int32_t* nhits, int32_t* ids, int max_ids,
-                   cudaStream_t st) {
+                   const int32_t* width, cudaStream_t st) {
     if constexpr (PACKET) {
         // the ray list holds int32 indices; without room for the scratch the
         // single-kernel march below does the same work
         if (R >= kRoundMinRays && R < INT32_MAX && S.n > 0) {
-            const cudaError_t e = launch_rounds<FB>(S, ro, rd, R, P, feat, depth, opac, nhits, ids, max_ids, st);
+            const cudaError_t e = launch_rounds<FB>(S, ro, rd, R, P, feat, depth, opac, nhits, ids, max_ids, width, st);
             if (e != cudaErrorMemoryAllocation) return e;
             cudaGetLastError();   // clear the failed allocation
         }
     }
     const int64_t blocks = (R + kTraceThreads - 1) / kTraceThreads;
     k_trace_forward<FB, PACKET><<<(unsigned)blocks, kTraceThreads, 0, st>>>(S, ro, rd, R, P, feat, depth, opac,
-                                                                           nhits, ids, max_ids);
+                                                                           nhits, ids, max_ids, width);
     count_launches(1);
     return cudaGetLastError();
 }
@@ -184,9 +218,10 @@ template <bool PACKET>
 cudaError_t launch_f(const SceneView& S, const float* ro, const float* rd, int64_t R, const TraceParams& P,
                      float* feat, float* depth, float* opac, int32_t* nhits, int32_t* ids, int max_ids,
                      cudaStream_t st) {
-    if (P.fc <= 3) return launch<3, PACKET>(S, ro, rd, R, P, feat, depth, opac, nhits, ids, max_ids, st);
-    if (P.fc <= 10) return launch<10, PACKET>(S, ro, rd, R, P, feat, depth, opac, nhits, ids, max_ids, st);
-    return launch<16, PACKET>(S, ro, rd, R, P, feat, depth, opac, nhits, ids, max_ids, st);
+    RowWidth w(rd, R, PACKET, st);
+    const auto f = P.fc <= 3 ? launch<3, PACKET> : (P.fc <= 10 ? launch<10, PACKET> : launch<16, PACKET>);
+    const cudaError_t e = f(S, ro, rd, R, P, feat, depth, opac, nhits, ids, max_ids, w.get(), st);
+    return e;
 }
 
 // Diagnostic: the march with a k-buffer of 16 entries and per-ray counters
@@ -211,6 +246,21 @@ __global__ void __launch_bounds__(128) k_trace_stats(SceneView S, const float* _
 }
 
 }  // namespace
+
+RowWidth::RowWidth(const float* rd, int64_t R, bool wanted, cudaStream_t st) : st_(st) {
+    if (!wanted || R < kRowMinRays || R >= INT32_MAX) return;
+    if (scratch_alloc(reinterpret_cast<void**>(&width_), sizeof(int32_t), st) != cudaSuccess) {
+        cudaGetLastError();   // no hint, then
+        width_ = nullptr;
+        return;
+    }
+    k_row_width<<<1, 1024, 0, st>>>(rd, R, width_);
+    count_launches(1);
+}
+
+RowWidth::~RowWidth() {
+    if (width_ != nullptr) cudaFreeAsync(width_, st_);
+}
 
 irgs_status launch_trace_stats(const SceneView& S, const float* ro, const float* rd, int64_t R,
                                const irgs_trace_params& p, int32_t* stats, cudaStream_t st) {
