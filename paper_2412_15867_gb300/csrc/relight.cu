@@ -17,8 +17,9 @@
 //               GGX half vectors per cell                             [32 x 32]
 //   sampling    row and per-row column cdfs of lum(E) sin(theta_row), FP64
 // over all environment texels t (centre direction w_t, exact band solid
-// angle dOmega_t). One block per output texel sums the environment with a
-// fixed order, so the maps are deterministic.
+// angle dOmega_t). The environment is cut into slices; a block sums one slice
+// for a tile of output texels, and the slices are then added in order, so the
+// maps are deterministic.
 #include <cuda_runtime.h>
 
 #include <new>
@@ -36,7 +37,6 @@ constexpr int kLevels = IRGS_RELIGHT_LEVELS;
 constexpr int kPrefH = IRGS_RELIGHT_PREF_H, kPrefW = IRGS_RELIGHT_PREF_W;
 constexpr int kLutN = IRGS_RELIGHT_LUT_N;
 constexpr int kLutSamples = 1024;
-constexpr int kReduceThreads = 256;
 constexpr int kRelightThreads = kTraceThreads;
 
 // Centre direction of texel (row, col) of an h x w equirect map.
@@ -55,88 +55,164 @@ __device__ __forceinline__ float texel_solid_angle(int H, int W, int row) {
     return 2.f * m * h * 2.f * kPi / (float)W;
 }
 
-template <int N>
-__device__ __forceinline__ void block_sum(float (&v)[N]) {
-    __shared__ float part[N][kReduceThreads / 32];
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-#pragma unroll
-    for (int k = 0; k < N; ++k)
-        for (int off = 16; off > 0; off >>= 1) v[k] += __shfl_xor_sync(0xffffffffu, v[k], off);
-    if (lane == 0)
-        for (int k = 0; k < N; ++k) part[k][warp] = v[k];
-    __syncthreads();
-    if (threadIdx.x == 0)
-        for (int k = 0; k < N; ++k) {
-            float s = 0.f;
-            for (int w = 0; w < kReduceThreads / 32; ++w) s += part[k][w];
-            v[k] = s;
+// Sums over the environment for a tile of output texels. A sum over all
+// texels costs a direction (two sincospi) and a weight per (output, texel)
+// pair, 1.1e9 pairs for the prefilter of a 512 x 256 environment; computing
+// both per pair took 25 ms (prefilter) and 1.2 ms (irradiance). Here a block
+// makes the directions of 128 texels at a time once for its 128 x kMapTexels
+// outputs, all prefilter levels share a pair's geometry, and a warp whose 32
+// outputs (an 8 x 4 patch) all face away skips the weights.
+constexpr int kMapThreads = 128;
+constexpr int kMapTexels = 2;      // output texels per thread
+constexpr int kMapSlice = 2048;    // least environment texels per slice
+constexpr int kMapMaxSlices = 64;
+
+// Output texel (row, col) of thread t of tile `tile`, its j-th: warps cover
+// patches of 8 columns x 4 rows, the j-th patch 4 rows further down.
+__device__ __forceinline__ void map_texel(int w, int tile, int j, int& row, int& col) {
+    const int patch = tile * (kMapThreads / 32) + (threadIdx.x >> 5), across = w / 8;
+    row = (patch / across * kMapTexels + j) * 4 + (threadIdx.x & 31) / 8;
+    col = patch % across * 8 + (threadIdx.x & 7);
+}
+
+// Texels [begin, end) of the environment, by chunks: fn(direction and solid
+// angle, radiance) for each.
+template <class Fn>
+__device__ __forceinline__ void for_texels(const float* __restrict__ env, int H, int W, int64_t begin, int64_t end,
+                                           Fn fn) {
+    __shared__ float4 s_dir[kMapThreads], s_val[kMapThreads];
+    for (int64_t t0 = begin; t0 < end; t0 += kMapThreads) {
+        const int64_t t = t0 + threadIdx.x;
+        if (t < end) {
+            const int r = (int)(t / W), c = (int)(t - (int64_t)r * W);
+            const f3 d = texel_dir(H, W, r, c);
+            s_dir[threadIdx.x] = make_float4(d.x, d.y, d.z, texel_solid_angle(H, W, r));
+            s_val[threadIdx.x] = make_float4(env[3 * t], env[3 * t + 1], env[3 * t + 2], 0.f);
         }
-}
-
-// One block per irradiance texel.
-__global__ void __launch_bounds__(kReduceThreads) k_irradiance(const float* __restrict__ env, int H, int W,
-                                                               float* __restrict__ irr) {
-    const int i = blockIdx.x;
-    const f3 N = texel_dir(kIrrH, kIrrW, i / kIrrW, i % kIrrW);
-    float acc[3] = {0.f, 0.f, 0.f};
-    for (int t = threadIdx.x; t < H * W; t += kReduceThreads) {
-        const int r = t / W, c = t - r * W;
-        const float cs = dot3(texel_dir(H, W, r, c), N);
-        if (cs <= 0.f) continue;
-        const float wgt = cs * texel_solid_angle(H, W, r);
-        const float* e = env + (int64_t)t * 3;
-        acc[0] = fmaf(e[0], wgt, acc[0]);
-        acc[1] = fmaf(e[1], wgt, acc[1]);
-        acc[2] = fmaf(e[2], wgt, acc[2]);
-    }
-    block_sum<3>(acc);
-    if (threadIdx.x == 0)
-        for (int k = 0; k < 3; ++k) irr[(int64_t)i * 3 + k] = acc[k] * (1.f / kPi);
-}
-
-// One block per texel of prefilter levels 1 .. kLevels - 1.
-__global__ void __launch_bounds__(kReduceThreads) k_prefilter(const float* __restrict__ env, int H, int W,
-                                                              float* __restrict__ pref) {
-    const int per_level = kPrefH * kPrefW;
-    const int level = 1 + blockIdx.x / per_level;
-    const int i = blockIdx.x % per_level;
-    const float rho = (float)level / (float)(kLevels - 1);
-    const float a2 = rho * rho * rho * rho;
-    const f3 R = texel_dir(kPrefH, kPrefW, i / kPrefW, i % kPrefW);
-    float acc[4] = {0.f, 0.f, 0.f, 0.f};
-    for (int t = threadIdx.x; t < H * W; t += kReduceThreads) {
-        const int r = t / W, c = t - r * W;
-        const f3 w = texel_dir(H, W, r, c);
-        const float cs = dot3(w, R);
-        if (cs <= 0.f) continue;
-        const f3 h = normalize3(add3(w, R));
-        const float nh = dot3(R, h);
-        const f3 x = cross3(R, h);
-        const float q = fmaf(nh * nh, a2, dot3(x, x));   // (n.h)^2 (a2 - 1) + 1 without cancellation
-        const float wgt = a2 / (kPi * q * q) * cs * texel_solid_angle(H, W, r);
-        const float* e = env + (int64_t)t * 3;
-        acc[0] = fmaf(e[0], wgt, acc[0]);
-        acc[1] = fmaf(e[1], wgt, acc[1]);
-        acc[2] = fmaf(e[2], wgt, acc[2]);
-        acc[3] += wgt;
-    }
-    block_sum<4>(acc);
-    if (threadIdx.x == 0) {
-        float* o = pref + ((int64_t)(level - 1) * per_level + i) * 3;
-        for (int k = 0; k < 3; ++k) o[k] = acc[3] > 0.f ? acc[k] / acc[3] : 0.f;
+        __syncthreads();
+        const int n = (int)(end - t0 < kMapThreads ? end - t0 : kMapThreads);
+        for (int i = 0; i < n; ++i) fn(s_dir[i], s_val[i]);
+        __syncthreads();
     }
 }
 
-// One thread per table cell.
+// Irradiance partial sums: part[slice][texel] = sum E max(0, w.N) dOmega.
+__global__ void __launch_bounds__(kMapThreads) k_irradiance(const float* __restrict__ env, int H, int W, int slices,
+                                                            float4* __restrict__ part) {
+    f3 N[kMapTexels];
+    int id[kMapTexels];
+    float acc[kMapTexels][3] = {};
+#pragma unroll
+    for (int j = 0; j < kMapTexels; ++j) {
+        int row, col;
+        map_texel(kIrrW, blockIdx.x, j, row, col);
+        N[j] = texel_dir(kIrrH, kIrrW, row, col);
+        id[j] = row * kIrrW + col;
+    }
+    const int64_t n = (int64_t)H * W;
+    for_texels(env, H, W, n * blockIdx.y / slices, n * (blockIdx.y + 1) / slices, [&](const float4& d, const float4& e) {
+#pragma unroll
+        for (int j = 0; j < kMapTexels; ++j) {
+            const float cs = dot3(mk3(d.x, d.y, d.z), N[j]);
+            if (!(cs > 0.f)) continue;
+            const float w = cs * d.w;
+            acc[j][0] = fmaf(e.x, w, acc[j][0]);
+            acc[j][1] = fmaf(e.y, w, acc[j][1]);
+            acc[j][2] = fmaf(e.z, w, acc[j][2]);
+        }
+    });
+#pragma unroll
+    for (int j = 0; j < kMapTexels; ++j)
+        part[(int64_t)blockIdx.y * (kIrrH * kIrrW) + id[j]] = make_float4(acc[j][0], acc[j][1], acc[j][2], 0.f);
+}
+
+// Prefilter partial sums of every level: part[slice][level - 1][texel] = sums
+// of E wgt and wgt, wgt = (w.R)+ dOmega / q^2 (the constant a^2 / pi of D
+// cancels in their ratio). With the half vector h of the unit vectors w and R,
+// |R x h|^2 = |w - R|^2 / 4 and (R.h)^2 is one less that: no h is needed, and
+// nothing cancels near the peak.
+__global__ void __launch_bounds__(kMapThreads) k_prefilter(const float* __restrict__ env, int H, int W, int slices,
+                                                           float4* __restrict__ part) {
+    constexpr int kL = kLevels - 1;
+    f3 R[kMapTexels];
+    int id[kMapTexels];
+    float4 acc[kMapTexels][kL];
+#pragma unroll
+    for (int j = 0; j < kMapTexels; ++j) {
+        int row, col;
+        map_texel(kPrefW, blockIdx.x, j, row, col);
+        R[j] = texel_dir(kPrefH, kPrefW, row, col);
+        id[j] = row * kPrefW + col;
+#pragma unroll
+        for (int l = 0; l < kL; ++l) acc[j][l] = make_float4(0.f, 0.f, 0.f, 0.f);
+    }
+    const int64_t n = (int64_t)H * W;
+    for_texels(env, H, W, n * blockIdx.y / slices, n * (blockIdx.y + 1) / slices, [&](const float4& d, const float4& e) {
+#pragma unroll
+        for (int j = 0; j < kMapTexels; ++j) {
+            const float cs = dot3(mk3(d.x, d.y, d.z), R[j]);
+            if (!(cs > 0.f)) continue;
+            const float w = cs * d.w;
+            const f3 g = mk3(d.x - R[j].x, d.y - R[j].y, d.z - R[j].z);
+            const float x2 = 0.25f * dot3(g, g), nh2 = 1.f - x2;
+#pragma unroll
+            for (int l = 0; l < kL; ++l) {
+                const float rho = (float)(l + 1) / (float)(kLevels - 1);
+                const float q = fmaf(nh2, rho * rho * rho * rho, x2);   // (n.h)^2 (a2 - 1) + 1
+                const float wgt = __fdividef(w, q * q);
+                acc[j][l].x = fmaf(e.x, wgt, acc[j][l].x);
+                acc[j][l].y = fmaf(e.y, wgt, acc[j][l].y);
+                acc[j][l].z = fmaf(e.z, wgt, acc[j][l].z);
+                acc[j][l].w += wgt;
+            }
+        }
+    });
+#pragma unroll
+    for (int j = 0; j < kMapTexels; ++j)
+#pragma unroll
+        for (int l = 0; l < kL; ++l)
+            part[((int64_t)blockIdx.y * kL + l) * (kPrefH * kPrefW) + id[j]] = acc[j][l];
+}
+
+// The slices' partial sums in order: irradiance texels, then prefilter texels
+// of every level.
+__global__ void k_map_sums(const float4* __restrict__ irr_part, const float4* __restrict__ pref_part, int slices,
+                           float* __restrict__ irr, float* __restrict__ pref) {
+    constexpr int kI = kIrrH * kIrrW, kP = (kLevels - 1) * kPrefH * kPrefW;
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= kI + kP) return;
+    const bool is_irr = i < kI;
+    const float4* p = is_irr ? irr_part + i : pref_part + (i - kI);
+    float4 s = make_float4(0.f, 0.f, 0.f, 0.f);
+    for (int k = 0; k < slices; ++k) {
+        const float4 v = p[(int64_t)k * (is_irr ? kI : kP)];
+        s.x += v.x;
+        s.y += v.y;
+        s.z += v.z;
+        s.w += v.w;
+    }
+    if (is_irr) {
+        irr[3 * i] = s.x * (1.f / kPi);
+        irr[3 * i + 1] = s.y * (1.f / kPi);
+        irr[3 * i + 2] = s.z * (1.f / kPi);
+    } else {
+        float* o = pref + 3 * (int64_t)(i - kI);
+        o[0] = s.w > 0.f ? s.x / s.w : 0.f;
+        o[1] = s.w > 0.f ? s.y / s.w : 0.f;
+        o[2] = s.w > 0.f ? s.z / s.w : 0.f;
+    }
+}
+
+// One warp per table cell.
 __global__ void k_brdf_table(float* __restrict__ lut) {
-    const int cell = blockIdx.x * blockDim.x + threadIdx.x;
+    const int cell = (blockIdx.x * blockDim.x + threadIdx.x) / 32, lane = threadIdx.x & 31;
     if (cell >= kLutN * kLutN) return;
     const int i = cell / kLutN, j = cell % kLutN;
     const float mu = ((float)i + 0.5f) / (float)kLutN, rho = ((float)j + 0.5f) / (float)kLutN;
     const float ag = rho * rho, a2 = ag * ag, kk = 0.5f * ag;
     const f3 v = mk3(sqrtf(1.f - mu * mu), 0.f, mu);
     float A = 0.f, B = 0.f;
-    for (int s = 0; s < kLutSamples; ++s) {
+    for (int s = lane; s < kLutSamples; s += 32) {
         const float u1 = ((float)s + 0.5f) / (float)kLutSamples;
         const float u2 = (float)__brev((unsigned)s) * 2.3283064365386963e-10f;   // radical inverse, base 2
         const float om = 1.f - u1;
@@ -155,35 +231,60 @@ __global__ void k_brdf_table(float* __restrict__ lut) {
         A += (1.f - fc) * gv;
         B += fc * gv;
     }
-    lut[cell * 2] = A / (float)kLutSamples;
-    lut[cell * 2 + 1] = B / (float)kLutSamples;
+#pragma unroll
+    for (int off = 16; off > 0; off >>= 1) {
+        A += __shfl_xor_sync(0xffffffffu, A, off);
+        B += __shfl_xor_sync(0xffffffffu, B, off);
+    }
+    if (lane == 0) {
+        lut[cell * 2] = A / (float)kLutSamples;
+        lut[cell * 2 + 1] = B / (float)kLutSamples;
+    }
 }
 
-// Importance-sampling tables, FP64, sequential in row-major order (the sums
-// are deterministic): one thread per row for the column cdfs, then one
-// thread for the row cdf.
+// Importance-sampling tables, FP64: one warp per row for the column cdfs,
+// then one warp for the row cdf, each by a scan of 32 terms at a time onto
+// the running sum (a fixed order of additions).
+__device__ __forceinline__ double warp_scan(double v, double& run) {
+    const int lane = threadIdx.x & 31;
+#pragma unroll
+    for (int off = 1; off < 32; off <<= 1) {
+        const double y = __shfl_up_sync(0xffffffffu, v, off);
+        if (lane >= off) v = __dadd_rn(v, y);
+    }
+    v = __dadd_rn(run, v);
+    run = __shfl_sync(0xffffffffu, v, 31);
+    return v;
+}
+
 __global__ void k_env_col_cdf(const float* __restrict__ env, int H, int W, double* __restrict__ col_cdf) {
-    const int r = blockIdx.x * blockDim.x + threadIdx.x;
+    const int r = (blockIdx.x * blockDim.x + threadIdx.x) / 32, lane = threadIdx.x & 31;
     if (r >= H) return;
     const double s = sin(((double)r + 0.5) * 3.14159265358979323846 / (double)H);
     double* cc = col_cdf + (int64_t)r * (W + 1);
     double run = 0.0;
-    cc[0] = 0.0;
-    for (int c = 0; c < W; ++c) {
-        const float* e = env + ((int64_t)r * W + c) * 3;
-        const double lum = __dadd_rn(__dadd_rn(__dmul_rn(0.2126, (double)e[0]), __dmul_rn(0.7152, (double)e[1])),
-                                     __dmul_rn(0.0722, (double)e[2]));
-        run = __dadd_rn(run, __dmul_rn(lum, s));
-        cc[c + 1] = run;
+    if (lane == 0) cc[0] = 0.0;
+    for (int c0 = 0; c0 < W; c0 += 32) {
+        const int c = c0 + lane;
+        double v = 0.0;
+        if (c < W) {
+            const float* e = env + ((int64_t)r * W + c) * 3;
+            const double lum = __dadd_rn(__dadd_rn(__dmul_rn(0.2126, (double)e[0]), __dmul_rn(0.7152, (double)e[1])),
+                                         __dmul_rn(0.0722, (double)e[2]));
+            v = __dmul_rn(lum, s);
+        }
+        v = warp_scan(v, run);
+        if (c < W) cc[c + 1] = v;
     }
 }
 
 __global__ void k_env_row_cdf(const double* __restrict__ col_cdf, int H, int W, double* __restrict__ row_cdf) {
     double run = 0.0;
-    row_cdf[0] = 0.0;
-    for (int r = 0; r < H; ++r) {
-        run = __dadd_rn(run, col_cdf[(int64_t)r * (W + 1) + W]);
-        row_cdf[r + 1] = run;
+    if (threadIdx.x == 0) row_cdf[0] = 0.0;
+    for (int r0 = 0; r0 < H; r0 += 32) {
+        const int r = r0 + threadIdx.x;
+        const double v = warp_scan(r < H ? col_cdf[(int64_t)r * (W + 1) + W] : 0.0, run);
+        if (r < H) row_cdf[r + 1] = v;
     }
 }
 
@@ -563,20 +664,11 @@ cudaError_t relight_wave(const SceneView& S, const uint32_t* bounds, const EnvMa
     return e != cudaSuccess ? e : ef;
 }
 
-template <class T>
-cudaError_t dalloc(T** p, size_t count, int64_t& bytes) {
-    const size_t b = sizeof(T) * (count > 0 ? count : 1);
-    bytes += (int64_t)b;
-    return cudaMalloc(reinterpret_cast<void**>(p), b);
-}
-
 }  // namespace
 
 void free_envmap(irgs_envmap m) {
     if (m == nullptr) return;
-    void* ptrs[] = {m->env, m->irr, m->pref, m->lut, m->row_cdf, m->col_cdf};
-    for (void* q : ptrs)
-        if (q) cudaFree(q);
+    if (m->base) cudaFree(m->base);
     delete m;
 }
 
@@ -586,27 +678,53 @@ irgs_status build_envmap_impl(const float* env, int32_t H, int32_t W, cudaStream
     cudaGetDevice(&m->device);
     m->H = H;
     m->W = W;
-    cudaError_t e = cudaSuccess;
-    auto A = [&](cudaError_t r) { if (e == cudaSuccess) e = r; };
-    A(dalloc(&m->env, (size_t)H * W * 3, m->bytes));
-    A(dalloc(&m->irr, (size_t)kIrrH * kIrrW * 3, m->bytes));
-    A(dalloc(&m->pref, (size_t)(kLevels - 1) * kPrefH * kPrefW * 3, m->bytes));
-    A(dalloc(&m->lut, (size_t)kLutN * kLutN * 2, m->bytes));
-    A(dalloc(&m->row_cdf, (size_t)H + 1, m->bytes));
-    A(dalloc(&m->col_cdf, (size_t)H * (W + 1), m->bytes));
+    // all maps in one allocation (each cudaMalloc and cudaFree costs as much as a small map)
+    const size_t counts[6] = {sizeof(float) * (size_t)H * W * 3, sizeof(float) * kIrrH * kIrrW * 3,
+                              sizeof(float) * (kLevels - 1) * kPrefH * kPrefW * 3, sizeof(float) * kLutN * kLutN * 2,
+                              sizeof(double) * ((size_t)H + 1), sizeof(double) * (size_t)H * (W + 1)};
+    size_t at[6], bytes = 0;
+    for (int i = 0; i < 6; ++i) {
+        at[i] = bytes;
+        bytes += (counts[i] + 255) & ~size_t(255);
+        m->bytes += (int64_t)counts[i];
+    }
+    cudaError_t e = cudaMalloc(&m->base, bytes);
+    // the slices' partial sums
+    const int64_t texels = (int64_t)H * W;
+    const int64_t want = (texels + kMapSlice - 1) / kMapSlice;
+    const int slices = (int)(want < kMapMaxSlices ? want : kMapMaxSlices);
+    constexpr int kIrr = kIrrH * kIrrW, kPref = kPrefH * kPrefW;
+    float4* part = nullptr;
+    if (e == cudaSuccess)
+        e = scratch_alloc(reinterpret_cast<void**>(&part),
+                          sizeof(float4) * (size_t)slices * (kIrr + (kLevels - 1) * kPref), st);
     if (e != cudaSuccess) {
         free_envmap(m);
         cudaGetLastError();
         return e == cudaErrorMemoryAllocation ? IRGS_ERR_OOM : IRGS_ERR_CUDA;
     }
+    unsigned char* base = static_cast<unsigned char*>(m->base);
+    m->env = reinterpret_cast<float*>(base + at[0]);
+    m->irr = reinterpret_cast<float*>(base + at[1]);
+    m->pref = reinterpret_cast<float*>(base + at[2]);
+    m->lut = reinterpret_cast<float*>(base + at[3]);
+    m->row_cdf = reinterpret_cast<double*>(base + at[4]);
+    m->col_cdf = reinterpret_cast<double*>(base + at[5]);
+    auto A = [&](cudaError_t r) { if (e == cudaSuccess) e = r; };
     A(cudaMemcpyAsync(m->env, env, sizeof(float) * (size_t)H * W * 3, cudaMemcpyDeviceToDevice, st));
-    k_irradiance<<<kIrrH * kIrrW, kReduceThreads, 0, st>>>(m->env, H, W, m->irr);
-    k_prefilter<<<(kLevels - 1) * kPrefH * kPrefW, kReduceThreads, 0, st>>>(m->env, H, W, m->pref);
-    k_brdf_table<<<(kLutN * kLutN + 127) / 128, 128, 0, st>>>(m->lut);
-    k_env_col_cdf<<<(H + 127) / 128, 128, 0, st>>>(m->env, H, W, m->col_cdf);
-    k_env_row_cdf<<<1, 1, 0, st>>>(m->col_cdf, H, W, m->row_cdf);
-    count_launches(5);
+    float4* pref_part = part + (size_t)slices * kIrr;
+    constexpr int kPer = kMapThreads * kMapTexels;
+    static_assert(kIrr % kPer == 0 && kPref % kPer == 0 && kIrrW % 8 == 0 && kIrrH % (4 * kMapTexels) == 0 &&
+                      kPrefH % (4 * kMapTexels) == 0, "whole tiles of patches");
+    k_irradiance<<<dim3(kIrr / kPer, slices), kMapThreads, 0, st>>>(m->env, H, W, slices, part);
+    k_prefilter<<<dim3(kPref / kPer, slices), kMapThreads, 0, st>>>(m->env, H, W, slices, pref_part);
+    k_map_sums<<<(kIrr + (kLevels - 1) * kPref + 255) / 256, 256, 0, st>>>(part, pref_part, slices, m->irr, m->pref);
+    k_brdf_table<<<(kLutN * kLutN * 32 + 255) / 256, 256, 0, st>>>(m->lut);
+    k_env_col_cdf<<<(unsigned)(((int64_t)H * 32 + 127) / 128), 128, 0, st>>>(m->env, H, W, m->col_cdf);
+    k_env_row_cdf<<<1, 32, 0, st>>>(m->col_cdf, H, W, m->row_cdf);
+    count_launches(6);
     A(cudaGetLastError());
+    A(cudaFreeAsync(part, st));
     if (e != cudaSuccess) {
         cudaStreamSynchronize(st);
         free_envmap(m);

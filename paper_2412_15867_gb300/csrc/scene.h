@@ -65,6 +65,7 @@ struct irgs_envmap_s {
     int device = 0;
     int32_t H = 0, W = 0;
     int64_t bytes = 0;
+    void* base = nullptr;       // the one allocation behind the maps
     float* env = nullptr;       // [H, W, 3] copy
     float* irr = nullptr;       // [IRGS_RELIGHT_IRR_H, IRGS_RELIGHT_IRR_W, 3]
     float* pref = nullptr;      // [IRGS_RELIGHT_LEVELS - 1, IRGS_RELIGHT_PREF_H, IRGS_RELIGHT_PREF_W, 3]
