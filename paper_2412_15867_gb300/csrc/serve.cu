@@ -3,7 +3,9 @@
 // from the step's tile table with an atomic counter until it is exhausted; a
 // tile is up to a few thousand camera rays. The step (staging copy, counter
 // reset, kernel) can be captured once into a CUDA graph and replayed with new
-// table contents. The shading tiles of the step then run, one request's range
+// table contents. A unit of work is one block's 128 rays of a tile, so a step
+// of a few tiles still fills the GPU (a whole tile per block left a step of
+// 36 tiles on 36 of 152 SMs: two such steps took 46.5 ms of a burst's 64). The shading tiles of the step then run, one request's range
 // of G-buffer points at a time, through the wavefront shading path (secondary
 // rays regrouped by direction and origin, traced in that order, estimated
 // per point), keyed by pixel index, so a pixel's estimate is the one
@@ -35,7 +37,7 @@ struct irgs_server_s {
     int n_scenes = 0;
     int max_jobs = 0, max_tiles = 0;
     size_t stage_bytes = 0;
-    unsigned char* host_stage = nullptr;   // pinned: [header 16 B][jobs][tiles]
+    unsigned char* host_stage = nullptr;   // pinned: [header 16 B][jobs][tiles][first unit of each tile]
     unsigned char* dev_stage = nullptr;
     irgs::SceneView* dev_scenes = nullptr;
     int* dev_next = nullptr;
@@ -58,10 +60,11 @@ constexpr size_t kHeaderBytes = 16;
 
 struct ServeArgs {
     const SceneView* scenes;
-    const int32_t* header;   // [0] jobs, [1] tiles
+    const int32_t* header;   // [0] jobs, [1] tiles, [2] units
     const irgs_job* jobs;
     const irgs_tile* tiles;
-    int* next_tile;
+    const int32_t* first_unit;
+    int* next_unit;
     TraceParams render, gbuf;
 };
 
@@ -88,70 +91,75 @@ __global__ void k_camera_rays(irgs_camera c, int64_t first, int64_t count, float
 }
 
 __global__ void __launch_bounds__(kServeThreads, kPacketBlocks) k_serve(ServeArgs A) {
-    __shared__ int s_tile;
-    const int n_tiles = A.header[1];
+    __shared__ int s_tile, s_chunk;
+    const int n_tiles = A.header[1], n_units = A.header[2];
     for (;;) {
-        if (threadIdx.x == 0) s_tile = atomicAdd(A.next_tile, 1);
+        __syncthreads();   // the last unit has been read
+        if (threadIdx.x == 0) {
+            const int u = atomicAdd(A.next_unit, 1);
+            int lo = 0, hi = n_tiles;   // the last tile whose first unit is at most u (tiles without units share the next one's)
+            while (u < n_units && hi - lo > 1) {
+                const int mid = (lo + hi) >> 1;
+                if (A.first_unit[mid] <= u) lo = mid; else hi = mid;
+            }
+            s_tile = u < n_units ? lo : -1;
+            s_chunk = u < n_units ? u - A.first_unit[lo] : 0;
+        }
         __syncthreads();
         const int t = s_tile;
-        __syncthreads();
-        if (t >= n_tiles) return;
+        if (t < 0) return;
         const irgs_tile tile = A.tiles[t];
         const irgs_job& job = A.jobs[tile.job];
         const SceneView S = A.scenes[job.scene];
-        if (tile.kind == IRGS_TILE_RENDER || tile.kind == IRGS_TILE_GBUFFER) {
-            const bool render = tile.kind == IRGS_TILE_RENDER;
-            const TraceParams& P = render ? A.render : A.gbuf;
-            for (int i0 = 0; i0 < tile.count; i0 += kServeThreads) {
-                const int i = i0 + threadIdx.x;
-                const bool live = i < tile.count;
-                const int64_t p = (int64_t)tile.first + (live ? i : 0);
-                f3 o, d;
-                if (job.ray_o != nullptr) {
-                    o = mk3(job.ray_o[3 * p], job.ray_o[3 * p + 1], job.ray_o[3 * p + 2]);
-                    d = mk3(job.ray_d[3 * p], job.ray_d[3 * p + 1], job.ray_d[3 * p + 2]);
-                } else {
-                    camera_ray(job.cam, p, o, d);
-                }
-                const Ray ray = make_ray(o, d);
-                MarchState<10> st;
-                const bool ok = march_forward<10, true>(S, ray, P, st, nullptr, 0, live, warp_scratch<true>());
-                if (!live) continue;
-                if (!ok) atomicOr(S.status, kErrStackOverflow);
-                if (render) {
-#pragma unroll
-                    for (int c = 0; c < 10; ++c)
-                        if (c < P.fc) job.feat[p * P.fc + c] = st.C[c];
-                    job.depth[p] = st.D;
-                    job.opacity[p] = 1.f - st.T;
-                } else {
-                    // Eq. 9 normalisation by the accumulated opacity, into the
-                    // planar G-buffer of P = width x height pixels
-                    const int64_t Pj = (int64_t)job.cam.width * job.cam.height;
-                    const float O = 1.f - st.T;
-                    float* g = job.gbuffer;
-                    const bool valid = O > 0.5f;
-                    const float inv = valid ? 1.f / O : 0.f;
-                    const f3 x = add3(o, mul3(d, st.D * inv));
-                    f3 nn = mk3(st.C[4], st.C[5], st.C[6]);
-                    const float nl = sqrtf(dot3(nn, nn));
-                    nn = nl > 0.f ? mul3(nn, 1.f / nl) : mk3(0.f, 0.f, 1.f);
-                    float* gx = g + 3 * p;
-                    float* gn = g + 3 * Pj + 3 * p;
-                    float* ga = g + 6 * Pj + 3 * p;
-                    float* gw = g + 10 * Pj + 3 * p;
-                    gx[0] = x.x; gx[1] = x.y; gx[2] = x.z;
-                    gn[0] = nn.x; gn[1] = nn.y; gn[2] = nn.z;
-                    ga[0] = st.C[0] * inv; ga[1] = st.C[1] * inv; ga[2] = st.C[2] * inv;
-                    g[9 * Pj + p] = st.C[3] * inv;
-                    gw[0] = -d.x; gw[1] = -d.y; gw[2] = -d.z;
-                    g[13 * Pj + p] = valid ? 1.f : 0.f;
-                    g[14 * Pj + p] = O;
-                    g[15 * Pj + p] = 0.f;
-                }
-            }
+        const bool render = tile.kind == IRGS_TILE_RENDER;
+        const TraceParams& P = render ? A.render : A.gbuf;
+        const int i = s_chunk * kServeThreads + (int)threadIdx.x;
+        const bool live = i < tile.count;
+        const int64_t p = (int64_t)tile.first + (live ? i : 0);
+        f3 o, d;
+        if (job.ray_o != nullptr) {
+            o = mk3(job.ray_o[3 * p], job.ray_o[3 * p + 1], job.ray_o[3 * p + 2]);
+            d = mk3(job.ray_d[3 * p], job.ray_d[3 * p + 1], job.ray_d[3 * p + 2]);
+        } else {
+            camera_ray(job.cam, p, o, d);
         }
-        // shading tiles run after this kernel through the wavefront path
+        const Ray ray = make_ray(o, d);
+        MarchState<10> st;
+        const bool ok = march_forward<10, true>(S, ray, P, st, nullptr, 0, live, warp_scratch<true>());
+        if (!live) continue;
+        if (!ok) atomicOr(S.status, kErrStackOverflow);
+        if (render) {
+#pragma unroll
+            for (int c = 0; c < 10; ++c)
+                if (c < P.fc) job.feat[p * P.fc + c] = st.C[c];
+            job.depth[p] = st.D;
+            job.opacity[p] = 1.f - st.T;
+        } else {
+            // Eq. 9 normalisation by the accumulated opacity, into the
+            // planar G-buffer of P = width x height pixels
+            const int64_t Pj = (int64_t)job.cam.width * job.cam.height;
+            const float O = 1.f - st.T;
+            float* g = job.gbuffer;
+            const bool valid = O > 0.5f;
+            const float inv = valid ? 1.f / O : 0.f;
+            const f3 x = add3(o, mul3(d, st.D * inv));
+            f3 nn = mk3(st.C[4], st.C[5], st.C[6]);
+            const float nl = sqrtf(dot3(nn, nn));
+            nn = nl > 0.f ? mul3(nn, 1.f / nl) : mk3(0.f, 0.f, 1.f);
+            float* gx = g + 3 * p;
+            float* gn = g + 3 * Pj + 3 * p;
+            float* ga = g + 6 * Pj + 3 * p;
+            float* gw = g + 10 * Pj + 3 * p;
+            gx[0] = x.x; gx[1] = x.y; gx[2] = x.z;
+            gn[0] = nn.x; gn[1] = nn.y; gn[2] = nn.z;
+            ga[0] = st.C[0] * inv; ga[1] = st.C[1] * inv; ga[2] = st.C[2] * inv;
+            g[9 * Pj + p] = st.C[3] * inv;
+            gw[0] = -d.x; gw[1] = -d.y; gw[2] = -d.z;
+            g[13 * Pj + p] = valid ? 1.f : 0.f;
+            g[14 * Pj + p] = O;
+            g[15 * Pj + p] = 0.f;
+        }
+        // shading tiles have no units: they run after this kernel through the wavefront path
     }
 }
 
@@ -176,7 +184,8 @@ ServeArgs args_of(irgs_server s) {
     A.header = reinterpret_cast<const int32_t*>(s->dev_stage);
     A.jobs = reinterpret_cast<const irgs_job*>(s->dev_stage + kHeaderBytes);
     A.tiles = reinterpret_cast<const irgs_tile*>(s->dev_stage + kHeaderBytes + sizeof(irgs_job) * s->max_jobs);
-    A.next_tile = s->dev_next;
+    A.first_unit = reinterpret_cast<const int32_t*>(A.tiles + s->max_tiles);
+    A.next_unit = s->dev_next;
     A.render = s->render;
     A.gbuf = s->gbuf;
     return A;
@@ -228,7 +237,8 @@ irgs_status irgs_server_create(const irgs_scene* scenes, int32_t n_scenes, int32
     s->n_scenes = n_scenes;
     s->max_jobs = max_jobs;
     s->max_tiles = max_tiles;
-    s->stage_bytes = kHeaderBytes + sizeof(irgs_job) * (size_t)max_jobs + sizeof(irgs_tile) * (size_t)max_tiles;
+    s->stage_bytes = kHeaderBytes + sizeof(irgs_job) * (size_t)max_jobs +
+                     (sizeof(irgs_tile) + sizeof(int32_t)) * (size_t)max_tiles;
     s->render = to_params(*render);
     s->shade_params = *shade;
     s->host_views = new (std::nothrow) SceneView[n_scenes];
@@ -287,6 +297,9 @@ irgs_status irgs_server_step(irgs_server s, int32_t n_jobs, int32_t n_tiles, int
     if (!s || n_jobs < 0 || n_jobs > s->max_jobs || n_tiles < 0 || n_tiles > s->max_tiles) return IRGS_ERR_INVALID_ARG;
     const irgs_job* jobs = reinterpret_cast<const irgs_job*>(s->host_stage + kHeaderBytes);
     const irgs_tile* tiles = reinterpret_cast<const irgs_tile*>(s->host_stage + kHeaderBytes + sizeof(irgs_job) * s->max_jobs);
+    int32_t* first_unit = reinterpret_cast<int32_t*>(s->host_stage + kHeaderBytes + sizeof(irgs_job) * s->max_jobs +
+                                                     sizeof(irgs_tile) * (size_t)s->max_tiles);
+    int64_t units = 0;
     for (int t = 0; t < n_tiles; ++t) {   // validate the tables before any device work
         const irgs_tile& tl = tiles[t];
         if (tl.job < 0 || tl.job >= n_jobs || tl.count < 0 || tl.first < 0 || tl.kind < 0 || tl.kind > 2)
@@ -305,10 +318,14 @@ irgs_status irgs_server_step(irgs_server s, int32_t n_jobs, int32_t n_tiles, int
             (!jb.gbuffer || !jb.rgb || !jb.env || jb.env_h <= 0 || jb.env_w <= 0 || jb.n_diffuse < 0 || jb.n_spec < 0 ||
              jb.n_diffuse + jb.n_spec <= 0 || jb.n_diffuse + jb.n_spec > (1 << 24)))
             return IRGS_ERR_INVALID_ARG;
+        first_unit[t] = (int32_t)units;
+        if (tl.kind != IRGS_TILE_SHADE) units += (tl.count + (int64_t)kServeThreads - 1) / kServeThreads;
+        if (units > INT32_MAX / 2) return IRGS_ERR_INVALID_ARG;   // more than 10^11 rays in one step
     }
     int32_t* hdr = reinterpret_cast<int32_t*>(s->host_stage);
     hdr[0] = n_jobs;
     hdr[1] = n_tiles;
+    hdr[2] = (int32_t)units;
     irgs::DeviceGuard dg;
     if (!dg.set(s->device)) return IRGS_ERR_CUDA;
     cudaStream_t caller = static_cast<cudaStream_t>(stream);
