@@ -261,7 +261,7 @@ irgs_status irgs_scene_export_wide(irgs_scene sc, float* nodes, int64_t cap, int
     int64_t nw = 1;
     if (sc->n > 1) {
         uint32_t allocated = 0;   // wide nodes the collapse allocated
-        if (cudaMemcpy(&allocated, sc->wide_counters + 3, sizeof(uint32_t), cudaMemcpyDeviceToHost) != cudaSuccess)
+        if (cudaMemcpy(&allocated, sc->wide_counters + irgs::kWideLevels, sizeof(uint32_t), cudaMemcpyDeviceToHost) != cudaSuccess)
             return IRGS_ERR_CUDA;
         nw = (int64_t)allocated < sc->max_wide ? (int64_t)allocated : sc->max_wide;
     }

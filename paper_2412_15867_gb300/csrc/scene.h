@@ -7,6 +7,10 @@
 
 #include "common.cuh"
 
+namespace irgs {
+constexpr int kWideLevels = 64;   // >= the binary depth: each level of the collapse consumes one binary level at least
+}
+
 struct irgs_scene_s {
     int device = 0;
     int64_t n = 0;
@@ -28,17 +32,17 @@ struct irgs_scene_s {
     uint32_t* status = nullptr;       // device error word
     irgs::WideNode* wide = nullptr;   // [max_wide] 4-wide hierarchy
     int64_t max_wide = 0;
-    int2* wide_frontier = nullptr;    // [2n] (binary node, wide index) frontiers of the collapse
-    uint32_t* wide_counters = nullptr;// [4] rotating frontier sizes, wide nodes allocated
+    int32_t* wide_source = nullptr;   // [max_wide] binary node behind each wide node
+    uint32_t* wide_counters = nullptr;// [kWideLevels + 1] nodes allocated per level of the collapse, and in all
 
-    // build scratch (kept for rebuilds); after the gather, rec_user, box_user,
-    // keys_tmp, vals_tmp and hist serve as the clustering build's working memory
-    float4* rec_user = nullptr;       // [n*4]
-    float* box_user = nullptr;        // [n*6]
+    // build scratch (kept for rebuilds): the sort's second buffers and digit
+    // counts, which serve the clustering too, and the clustering's own
+    float4* rec_user = nullptr;       // [n*4] cluster boxes, two copies
+    float* box_user = nullptr;        // [n*6] kept lists
     uint32_t* keys_tmp = nullptr;     // [n]
     int32_t* vals_tmp = nullptr;      // [n]
-    uint32_t* hist = nullptr;         // [256 * tiles]
-    uint32_t* bounds = nullptr;       // [6] ordered-bit centroid bounds
+    uint32_t* hist = nullptr;         // digit counts, tile counts
+    uint32_t* bounds = nullptr;       // [6] ordered-bit centroid bounds, then the build's control words
     int32_t* leaf_parent = nullptr;   // [n]
     int32_t* node_parent = nullptr;   // [max(n-1,1)]
     uint32_t* refit_flag = nullptr;   // [max(n-1,1)]
