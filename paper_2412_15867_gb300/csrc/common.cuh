@@ -137,6 +137,7 @@ struct SceneView {
     int64_t n;
     int32_t F;
     float alpha_min;
+    uint32_t wide_bits;    // bits that hold any wide node's number, 2 .. 31
 };
 
 }  // namespace irgs

@@ -60,6 +60,8 @@ struct irgs_scene_s {
         v.n = n;
         v.F = F;
         v.alpha_min = alpha_min;
+        v.wide_bits = 2;
+        while (v.wide_bits < 31 && (max_wide >> v.wide_bits) != 0) ++v.wide_bits;
         return v;
     }
 };

@@ -409,10 +409,15 @@ __device__ __forceinline__ bool collect_round(const SceneView& S, const Ray& ray
                                               float4* scratch, TraceStats* ts = nullptr) {
     uint32_t* queue = reinterpret_cast<uint32_t*>(scratch) + (threadIdx.x & 31);   // entry i at queue[32 i]
     const RayBox rb = make_ray_box(ray0);
-    int2 stack[kStackSize];   // (node, entry depth bits): one 8-byte word per entry
+    // An entry is one word: the entry depth's leading bits (rounded down) above
+    // the node's number. The stacks live in local memory and share the L1 with
+    // nodes and records: at two words they took as much of it as those.
+    uint32_t stack[kStackSize];
     int sp = 0;
-    int2 top = make_int2(0, 0);   // the most recent entry, kept in registers
+    uint32_t top = 0u;   // the most recent entry, kept in a register
     bool has_top = false;
+    const uint32_t id_bits = S.wide_bits, id_mask = (1u << id_bits) - 1u;
+    auto entry_depth = [&](uint32_t e) { return __uint_as_float((e & ~id_mask) >> 1); };
     bool ok = true;
     const float t_lo = key_depth(last_key);
     const float lo_c = t_lo - tslack(t_lo);
@@ -471,15 +476,16 @@ __device__ __forceinline__ bool collect_round(const SceneView& S, const Ray& ray
             const int lo = (s & 1u) ? c[1] : c[0], hi = (s & 1u) ? c[3] : c[2];
             return (s & 2u) ? hi : lo;
         };
+        auto entry = [&](uint32_t k) { return ((k << 1) & ~id_mask) | (uint32_t)child_of(k); };
         if (key[0] == 0xffffffffu) {
             ni = -1;
             if (has_top) {
                 has_top = false;
-                if (__int_as_float(top.y) <= hi_c) ni = top.x;
+                if (entry_depth(top) <= hi_c) ni = (int)(top & id_mask);
             }
             while (ni < 0 && sp > 0) {
-                const int2 e = stack[--sp];
-                if (__int_as_float(e.y) <= hi_c) ni = e.x;
+                const uint32_t e = stack[--sp];
+                if (entry_depth(e) <= hi_c) ni = (int)(e & id_mask);
             }
             continue;
         }
@@ -489,10 +495,10 @@ __device__ __forceinline__ bool collect_round(const SceneView& S, const Ray& ray
                 ok = false;
             } else {
                 if (has_top) stack[sp++] = top;
-                if (key[3] != 0xffffffffu) stack[sp++] = make_int2(child_of(key[3]), (int)(key[3] & ~3u));
-                if (key[2] != 0xffffffffu) stack[sp++] = make_int2(child_of(key[2]), (int)(key[2] & ~3u));
+                if (key[3] != 0xffffffffu) stack[sp++] = entry(key[3]);
+                if (key[2] != 0xffffffffu) stack[sp++] = entry(key[2]);
             }
-            top = make_int2(child_of(key[1]), (int)(key[1] & ~3u));
+            top = entry(key[1]);
             has_top = true;
         }
     }

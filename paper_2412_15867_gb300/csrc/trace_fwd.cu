@@ -9,7 +9,7 @@ namespace {
 
 // Rows at least this wide are regrouped (narrower ones are tiles already, or no rows at all).
 constexpr int kMinRowWidth = 32;
-constexpr int kMaxRowWidth = 1 << 15;
+constexpr int kMaxRowWidth = 1 << 13;
 
 // Width of the image whose pixel rows the rays seem to be, else 0: the first
 // neighbours whose directions differ by more than twice the first
