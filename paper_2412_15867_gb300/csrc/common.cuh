@@ -128,6 +128,7 @@ cudaError_t scratch_alloc(void** p, size_t bytes, cudaStream_t st);
 struct SceneView {
     const Node* nodes;     // [max(n-1,1)] binary hierarchy
     const WideNode* wide;  // 4-wide hierarchy traversed by the kernels, root 0
+    const float4* child_box;  // the same child by child: node i, child k at [8 i + 2 k]: {lo, id bits}, {hi, 0}
     const float4* rec;     // [n * 4]
     const float* feat;     // [n, F] Morton order
     const float4* q_raw;   // [n] raw quaternion (w,x,y,z), Morton order

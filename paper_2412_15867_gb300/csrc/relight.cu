@@ -27,6 +27,7 @@
 #include "scene.h"
 #include "shade.cuh"
 #include "trace.cuh"
+#include "trace_warp.cuh"
 #include "wave.cuh"
 
 namespace irgs {
@@ -476,105 +477,62 @@ __global__ void k_relight_gen(EnvMaps M, const float* __restrict__ xg, int64_t p
     val[i] = (int32_t)i;
 }
 
-__global__ void __launch_bounds__(kRelightThreads, kRayBlocks) k_relight_trace(SceneView S, TraceParams P,
-                                                                      const float* __restrict__ xg, int64_t p0,
-                                                                      int Sn, const float4* __restrict__ dir,
-                                                                      const int32_t* __restrict__ order,
-                                                                      int64_t rays, float4* __restrict__ res) {
-    const int64_t j = blockIdx.x * (int64_t)kRelightThreads + threadIdx.x;
-    const bool there = j < rays;
-    const int64_t i = there ? order[j] : 0;
-    const float4 d4 = dir[i];
-    const bool live = there && d4.w > 0.f;
-    MarchState<7> st;
-    const bool ok = march_forward<7, false>(S, make_ray(ld3r(xg, p0 + i / Sn), mk3(d4.x, d4.y, d4.z)), P, st, nullptr,
-                                            0, live, warp_scratch<false>());
-    if (!there) return;
-    if (live) {
-        if (!ok) atomicOr(S.status, kErrStackOverflow);
-    } else {
-#pragma unroll
-        for (int c = 0; c < 7; ++c) st.C[c] = 0.f;
-        st.T = 1.f;
-    }
-    res[2 * i] = make_float4(st.C[0], st.C[1], st.C[2], st.C[3]);
-    res[2 * i + 1] = make_float4(st.C[4], st.C[5], st.C[6], st.T);
-}
-
-// The same traces in compacted rounds: round 1 on every sorted ray; rays
-// still marching store their state (C[7], D, T, hit count, next key) at
-// their sorted position and are regrouped, in sorted order, into warps that
-// run to completion. Per ray the rounds and their arithmetic are
-// march_forward's, so the results are the same.
-enum RelightRound { kRelFirst = 0, kRelLast = 1 };
-constexpr int kRelightStateF4 = 4;
-
-template <int MODE>
-__global__ void __launch_bounds__(kRelightThreads, kRayBlocks) k_relight_round(
-    SceneView S, TraceParams P, const float* __restrict__ xg, int64_t p0, int Sn, const float4* __restrict__ dir,
-    const int32_t* __restrict__ order, int64_t rays, float4* __restrict__ res, const int32_t* __restrict__ list,
-    const uint32_t* __restrict__ count, float4* __restrict__ state, uint32_t* __restrict__ flags) {
-    const int64_t t = blockIdx.x * (int64_t)kRelightThreads + threadIdx.x;
-    const int64_t n = MODE == kRelFirst ? rays : (int64_t)*count;
-    if (__all_sync(kFullWarp, t >= n)) return;   // nothing for this warp
-    const bool there = t < n;
-    const int64_t j = !there ? 0 : (MODE == kRelFirst ? t : (int64_t)list[t]);
-    const int64_t i = order[j];
-    const float4 d4 = dir[i];
-    const bool live = there && d4.w > 0.f;
-    if (MODE == kRelFirst && there && !live) {
-        res[2 * i] = make_float4(0.f, 0.f, 0.f, 0.f);
-        res[2 * i + 1] = make_float4(0.f, 0.f, 0.f, 1.f);
-    }
-    MarchState<7> st;
-    st.init();
-    uint64_t last_key = depth_key(P.t_min, 0.f);
-    int32_t last_u = INT32_MAX;
-    if (MODE != kRelFirst) {
-        float w[16];
-#pragma unroll
-        for (int q = 0; q < kRelightStateF4; ++q) {
-            const float4 v = state[j * kRelightStateF4 + q];
-            w[4 * q] = v.x; w[4 * q + 1] = v.y; w[4 * q + 2] = v.z; w[4 * q + 3] = v.w;
+struct RelightJob {
+    const float* xg;
+    int64_t p0;
+    int Sn;
+    const float4* dir;
+    const int32_t* order;
+    float4* res;
+    int max_ids;
+    __device__ __forceinline__ bool load(int j, f3& o, f3& d) const {
+        const int64_t i = order[j];
+        const float4 d4 = dir[i];
+        if (!(d4.w > 0.f)) {
+            res[2 * i] = make_float4(0.f, 0.f, 0.f, 0.f);
+            res[2 * i + 1] = make_float4(0.f, 0.f, 0.f, 1.f);
+            return false;
         }
-#pragma unroll
-        for (int c = 0; c < 7; ++c) st.C[c] = w[c];
-        st.D = w[7];
-        st.T = w[8];
-        st.nh = __float_as_int(w[9]);
-        last_key = ((uint64_t)__float_as_uint(w[11]) << 32) | (uint64_t)__float_as_uint(w[10]);
-        last_u = __float_as_int(w[12]);
+        o = ld3r(xg, p0 + i / Sn);
+        d = mk3(d4.x, d4.y, d4.z);
+        return true;
     }
-    const Ray ray = make_ray(ld3r(xg, p0 + i / Sn), mk3(d4.x, d4.y, d4.z));
-    KBuffer<kRayCap> kb;
-    kb.bind();
-    float4* scratch = warp_scratch<false>();
-    bool ok = true, done = !live, packet = false;
-    do {
-        ok &= collect<false>(S, ray, P, last_key, last_u, st.T, kb, !done, packet, scratch);
-        if (!done) done = blend_round<7>(S, ray, P, kb, st, nullptr, 0, last_key, last_u);
-    } while (MODE == kRelLast && __any_sync(kFullWarp, !done));
-    if (!live) return;
-    if (!ok) atomicOr(S.status, kErrStackOverflow);
-    if (done) {
+    __device__ __forceinline__ int32_t* ids(int) const { return nullptr; }
+    __device__ __forceinline__ void finish(int j, const MarchState<7>& st) const {
+        const int64_t i = order[j];
         res[2 * i] = make_float4(st.C[0], st.C[1], st.C[2], st.C[3]);
         res[2 * i + 1] = make_float4(st.C[4], st.C[5], st.C[6], st.T);
-    } else {
-        float w[16];
-#pragma unroll
-        for (int c = 0; c < 7; ++c) w[c] = st.C[c];
-        w[7] = st.D;
-        w[8] = st.T;
-        w[9] = __int_as_float(st.nh);
-        w[10] = __uint_as_float((uint32_t)last_key);
-        w[11] = __uint_as_float((uint32_t)(last_key >> 32));
-        w[12] = __int_as_float(last_u);
-        w[13] = w[14] = w[15] = 0.f;
-#pragma unroll
-        for (int q = 0; q < kRelightStateF4; ++q)
-            state[j * kRelightStateF4 + q] = make_float4(w[4 * q], w[4 * q + 1], w[4 * q + 2], w[4 * q + 3]);
-        flags[j] = 1u;
     }
+};
+
+__global__ void __launch_bounds__(kRelightThreads, kRayBlocks) k_relight_trace(SceneView S, TraceParams P,
+                                                                               RelightJob job, int rays,
+                                                                               uint32_t* next) {
+    __shared__ SavedMarch<7> saved;
+    walk_batch<7, kRayCap>(S, P, rays, next, job, saved);
+}
+
+// The same with a warp per ray, for batches that do not fill the chip many
+// times over with a ray per lane: 24.7 ms against 27.5 at 6.4M rays (the lines
+// are those of shading's batches, whose rays are the same kind).
+constexpr int64_t kRelightUnsortedMax = int64_t(1) << 19;   // smaller batches gain less from the order than its sort costs
+constexpr int64_t kRelightWarpMax = int64_t(1) << 23;
+__global__ void __launch_bounds__(kWarpRayThreads, kWarpRayBlocks) k_relight_trace_ray(SceneView S, TraceParams P, RelightJob job,
+                                                                                int rays) {
+    const int j = blockIdx.x * kWarpRays + (threadIdx.x >> 5);
+    f3 o, d;
+    if (j >= rays || !job.load(j, o, d)) return;
+    WarpMarch w;
+    const bool ok = march_warp(S, make_ray(o, d), P, w, job.ids(j), job.max_ids, warp_ray_scratch());
+    MarchState<7> st;
+#pragma unroll
+    for (int c = 0; c < 7; ++c) st.C[c] = __shfl_sync(kFullWarp, w.C, c);
+    st.D = w.D;
+    st.T = w.T;
+    st.nh = w.nh;
+    if ((threadIdx.x & 31) != 0) return;
+    if (!ok) atomicOr(S.status, kErrStackOverflow);
+    job.finish(j, st);
 }
 
 __global__ void __launch_bounds__(kRelightThreads) k_relight_shade(EnvMaps M, const float* __restrict__ ng,
@@ -614,9 +572,7 @@ cudaError_t relight_wave(const SceneView& S, const uint32_t* bounds, const EnvMa
     const int64_t cap = (P < pc ? P : pc) * Sn;
     const int64_t hw = sort_hist_words(cap);
     auto al = [](size_t b) { return (b + 255) & ~size_t(255); };
-    const int64_t sums = scan_long_words(cap + 1);
-    const size_t bytes = al(16 * cap) + 4 * al(4 * cap) + al(4 * hw) + al(32 * cap) + al(4 * (cap + 1)) +
-                         al(4 * cap) + al(4 * (1 + sums)) + al(16 * kRelightStateF4 * cap);
+    const size_t bytes = al(16 * cap) + 4 * al(4 * cap) + al(4 * hw) + al(32 * cap) + al(4);
     unsigned char* base = nullptr;
     cudaError_t e = scratch_alloc(reinterpret_cast<void**>(&base), bytes, st);
     if (e != cudaSuccess) return e;
@@ -629,32 +585,24 @@ cudaError_t relight_wave(const SceneView& S, const uint32_t* bounds, const EnvMa
     int32_t* vtmp = reinterpret_cast<int32_t*>(take(4 * cap));
     uint32_t* hist = reinterpret_cast<uint32_t*>(take(4 * hw));
     float4* res = reinterpret_cast<float4*>(take(32 * cap));
-    uint32_t* flags = reinterpret_cast<uint32_t*>(take(4 * (cap + 1)));
-    int32_t* list = reinterpret_cast<int32_t*>(take(4 * cap));
-    uint32_t* count = reinterpret_cast<uint32_t*>(take(4 * (1 + sums)));
-    float4* state = reinterpret_cast<float4*>(take(16 * kRelightStateF4 * cap));
+    uint32_t* next = reinterpret_cast<uint32_t*>(take(4));
     for (int64_t p0 = 0; p0 < P && e == cudaSuccess; p0 += pc) {
         const int64_t np = P - p0 < pc ? P - p0 : pc;
         const int64_t rays = np * Sn;
         k_relight_gen<<<grid_for(rays, 256), 256, 0, st>>>(M, x, p0, rays, Sn, seed, bounds, dir, key, val);
-        e = sort_pairs(key, val, ktmp, vtmp, hist, rays, st);
+        if (rays > kRelightUnsortedMax) e = sort_pairs(key, val, ktmp, vtmp, hist, rays, st);
         if (e != cudaSuccess) break;
-        if (S.n == 0) {
-            k_relight_trace<<<grid_for(rays, kRelightThreads), kRelightThreads, 0, st>>>(S, TP, x, p0, Sn, dir, val,
-                                                                                       rays, res);
-            count_launches(1);
+        const RelightJob job{x, p0, Sn, dir, val, res, 0};
+        if (rays <= kRelightWarpMax) {
+            k_relight_trace_ray<<<warp_ray_grid(rays), kWarpRayThreads, 0, st>>>(S, TP, job, (int)rays);
         } else {
-            const unsigned g = grid_for(rays, kRelightThreads);
-            e = cudaMemsetAsync(flags, 0, sizeof(uint32_t) * (rays + 1), st);
+            e = cudaMemsetAsync(next, 0, sizeof(uint32_t), st);
+            const unsigned blocks = batch_blocks(k_relight_trace, rays);
+            if (e == cudaSuccess && blocks == 0u) e = cudaGetLastError();
             if (e != cudaSuccess) break;
-            k_relight_round<kRelFirst><<<g, kRelightThreads, 0, st>>>(S, TP, x, p0, Sn, dir, val, rays, res, list,
-                                                                      count, state, flags);
-            e = flags_to_list(flags, rays, count + 1, list, count, st);
-            if (e != cudaSuccess) break;
-            k_relight_round<kRelLast><<<g, kRelightThreads, 0, st>>>(S, TP, x, p0, Sn, dir, val, rays, res, list,
-                                                                     count, state, flags);
-            count_launches(2);
+            k_relight_trace<<<blocks, kRelightThreads, 0, st>>>(S, TP, job, (int)rays, next);
         }
+        count_launches(1);
         k_relight_shade<<<grid_for(np, kRelightThreads / 32), kRelightThreads, 0, st>>>(M, n, a, r, wo, p0, np, Sn,
                                                                                        dir, res, rgb, vis, ind);
         count_launches(2);

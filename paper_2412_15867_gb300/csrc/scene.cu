@@ -982,7 +982,8 @@ __device__ __forceinline__ float box_area(const float b[6]) {
 
 __global__ void __launch_bounds__(kCoopThreads, 1) k_wide(const Node* __restrict__ nodes, int32_t* source,
                                                           uint32_t* counters, uint32_t* ctl, int64_t max_wide,
-                                                          WideNode* __restrict__ wide, uint32_t* status) {
+                                                          WideNode* __restrict__ wide,
+                                                          float4* __restrict__ child_box, uint32_t* status) {
     uint32_t target = 0u;
     const int lane = threadIdx.x & 31;
     uint32_t begin = 0u, end = 1u;
@@ -1073,6 +1074,11 @@ __global__ void __launch_bounds__(kCoopThreads, 1) k_wide(const Node* __restrict
             o.child = make_int4(out[0], out[1], out[2], out[3]);
             o.pad = make_int4(m, 0, 0, 0);
             wide[i] = o;
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+                child_box[8 * (int64_t)i + 2 * k] = make_float4(box[k][0], box[k][1], box[k][2], __int_as_float(out[k]));
+                child_box[8 * (int64_t)i + 2 * k + 1] = make_float4(box[k][3], box[k][4], box[k][5], 0.f);
+            }
         }
         if (!grid_barrier(ctl + kCtlWide, target)) {
             if (threadIdx.x == 0) atomicOr(status, kErrBadTree);
@@ -1086,7 +1092,7 @@ __global__ void __launch_bounds__(kCoopThreads, 1) k_wide(const Node* __restrict
 }
 
 // Wide root of a one-surfel (or empty) scene.
-__global__ void k_wide_tiny(int64_t n, const float* __restrict__ leaf_box, WideNode* wide) {
+__global__ void k_wide_tiny(int64_t n, const float* __restrict__ leaf_box, WideNode* wide, float4* child_box) {
     WideNode o;
     const float e = INFINITY;   // empty slots: lo = +inf, hi = -inf
     float b[6] = {e, e, e, -e, -e, -e};
@@ -1101,6 +1107,12 @@ __global__ void k_wide_tiny(int64_t n, const float* __restrict__ leaf_box, WideN
     o.child = make_int4(n == 1 ? ~0 : kNoChild, kNoChild, kNoChild, kNoChild);
     o.pad = make_int4(n == 1 ? 1 : 0, 0, 0, 0);
     wide[0] = o;
+    child_box[0] = make_float4(b[0], b[1], b[2], __int_as_float(o.child.x));
+    child_box[1] = make_float4(b[3], b[4], b[5], 0.f);
+    for (int k = 1; k < 4; ++k) {
+        child_box[2 * k] = make_float4(e, e, e, __int_as_float(kNoChild));
+        child_box[2 * k + 1] = make_float4(-e, -e, -e, 0.f);
+    }
 }
 
 template <class T>
@@ -1131,7 +1143,7 @@ void free_scene(irgs_scene sc) {
     if (!sc) return;
     void* ptrs[] = {sc->nodes, sc->rec, sc->feat, sc->q_raw, sc->scale, sc->leaf_box, sc->keys,
                     sc->perm, sc->inv_perm, sc->status, sc->rec_user, sc->box_user, sc->keys_tmp, sc->vals_tmp,
-                    sc->hist, sc->bounds, sc->leaf_parent, sc->node_parent, sc->refit_flag, sc->wide,
+                    sc->hist, sc->bounds, sc->leaf_parent, sc->node_parent, sc->refit_flag, sc->wide, sc->child_box,
                     sc->wide_source, sc->wide_counters};
     for (void* p : ptrs)
         if (p) cudaFree(p);
@@ -1197,9 +1209,9 @@ static cudaError_t enqueue_ploc(irgs_scene sc, cudaStream_t st) {
 static cudaError_t enqueue_wide(irgs_scene sc, cudaStream_t st) {
     const cudaError_t e = cudaMemsetAsync(sc->wide_counters, 0, sizeof(uint32_t) * (kWideLevels + 1), st);
     if (e != cudaSuccess) return e;
-    return launch_coop<const Node*, int32_t*, uint32_t*, uint32_t*, int64_t, WideNode*, uint32_t*>(
+    return launch_coop<const Node*, int32_t*, uint32_t*, uint32_t*, int64_t, WideNode*, float4*, uint32_t*>(
         k_wide, sc->device, sc->n, st, sc->nodes, sc->wide_source, sc->wide_counters, sc->bounds, sc->max_wide,
-        sc->wide, sc->status);
+        sc->wide, sc->child_box, sc->status);
 }
 
 // Morton order of the surfels: keys and perm.
@@ -1272,7 +1284,7 @@ static irgs_status enqueue_build(irgs_scene sc, const irgs_surfels* s, cudaStrea
         if (n > 1) {
             A(enqueue_wide(sc, st));
         } else {
-            k_wide_tiny<<<1, 1, 0, st>>>(n, sc->leaf_box, sc->wide);
+            k_wide_tiny<<<1, 1, 0, st>>>(n, sc->leaf_box, sc->wide, sc->child_box);
             count_launches(1);
         }
     }
@@ -1378,6 +1390,7 @@ irgs_status build_scene_impl(const irgs_surfels* s, float alpha_min, uint32_t bu
     // every wide node takes at least one binary internal node
     sc->max_wide = nn + 1;
     A(dalloc(&sc->wide, sc->max_wide, B));
+    A(dalloc(&sc->child_box, 8 * sc->max_wide, B));
     A(dalloc(&sc->wide_source, sc->max_wide, B));
     A(dalloc(&sc->wide_counters, kWideLevels + 1, B));
     if (e != cudaSuccess) {
@@ -1430,7 +1443,7 @@ irgs_status refit_scene_impl(irgs_scene sc, const irgs_surfels* s, cudaStream_t 
         A(enqueue_wide(sc, st));
     } else {
         k_tiny_root<<<1, 1, 0, st>>>(n, sc->leaf_box, sc->nodes);
-        k_wide_tiny<<<1, 1, 0, st>>>(n, sc->leaf_box, sc->wide);
+        k_wide_tiny<<<1, 1, 0, st>>>(n, sc->leaf_box, sc->wide, sc->child_box);
         count_launches(2);
     }
     A(cudaGetLastError());

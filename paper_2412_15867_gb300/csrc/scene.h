@@ -31,6 +31,7 @@ struct irgs_scene_s {
     int32_t* inv_perm = nullptr;      // [n] Morton slot of user index
     uint32_t* status = nullptr;       // device error word
     irgs::WideNode* wide = nullptr;   // [max_wide] 4-wide hierarchy
+    float4* child_box = nullptr;      // [max_wide * 8] the same nodes child by child
     int64_t max_wide = 0;
     int32_t* wide_source = nullptr;   // [max_wide] binary node behind each wide node
     uint32_t* wide_counters = nullptr;// [kWideLevels + 1] nodes allocated per level of the collapse, and in all
@@ -51,6 +52,7 @@ struct irgs_scene_s {
         irgs::SceneView v;
         v.nodes = nodes;
         v.wide = wide;
+        v.child_box = child_box;
         v.rec = rec;
         v.feat = feat;
         v.q_raw = q_raw;

@@ -21,7 +21,7 @@
 // order from their hit lists (rays with longer lists replay the march).
 //
 // Rays are processed in chunks of whole points, at most kWaveChunkRays rays
-// each, so the scratch (~390 bytes per ray with the gradient) stays bounded;
+// each, so the scratch (~330 bytes per ray with the gradient) stays bounded;
 // a chunk is sorted as a whole, and the denser its points the more a warp's
 // regrouped rays share their paths (one chunk of 41M rays traces 6-7%
 // faster than three of at most 2^24).
@@ -30,6 +30,7 @@
 #include "scene.h"
 #include "shade.cuh"
 #include "trace.cuh"
+#include "trace_warp.cuh"
 #include "trace_bwd.cuh"
 #include "wave.cuh"
 
@@ -39,7 +40,16 @@ namespace {
 constexpr int kWaveThreads = kTraceThreads;
 constexpr int64_t kWaveChunkRays = int64_t(1) << 26;
 constexpr int kWaveSavedHits = 64;   // 12% of secondary rays blend more than 32 hits, 0.02% more than 64
-constexpr int kWaveReplayBlocks = 1024;   // grid-stride blocks for the few rays whose hit list did not fit
+// Batches up to this size keep their order: at 61k rays the sort by origin and
+// direction costs more than it gives (1.07 ms for a call without, 1.16 with),
+// at 1M rays it pays (8.20 without, 7.94 with).
+constexpr int64_t kWaveUnsortedMax = int64_t(1) << 19;
+// Batches up to this size take a warp per ray, whose throughput does not depend
+// on the size; a ray per lane catches up only where the pools are refilled many
+// times: 120.5 ms against 114.5 at 41M rays, 24.7 against 27.5 at 6.4M
+// (relighting, the same walk).
+constexpr int64_t kWaveWarpMax = int64_t(1) << 23;
+constexpr int kWaveReplayBlocks = 152 * 4;   // blocks that share the few rays whose hit list did not fit
 
 __device__ __forceinline__ f3 ld3w(const float* p, int64_t i) { return mk3(p[3 * i], p[3 * i + 1], p[3 * i + 2]); }
 
@@ -69,103 +79,71 @@ __global__ void k_wave_gen(const float* __restrict__ xg, const float* __restrict
     val[i] = (int32_t)i;
 }
 
-// Trace the rays in regrouped order; res[i] = (L_ind, V).
-// With SAVE the blended hit ids (user order, -1 terminated) and the hit
-// counts are kept for the backward.
+// Trace the rays in regrouped order; res[i] = (L_ind, V). With SAVE the blended
+// hit ids (user order, -1 terminated) and the hit counts are kept for the
+// backward.
 template <bool SAVE>
-__global__ void __launch_bounds__(kWaveThreads, kRayBlocks) k_wave_trace(SceneView S, TraceParams P,
-                                                                const float* __restrict__ xg, int64_t p0, int St,
-                                                                const float4* __restrict__ dir,
-                                                                const int32_t* __restrict__ order, int64_t rays,
-                                                                float4* __restrict__ res, int32_t* __restrict__ nh,
-                                                                int32_t* __restrict__ ids, int max_ids) {
-    const int64_t j = blockIdx.x * (int64_t)kWaveThreads + threadIdx.x;
-    const int64_t i = j < rays ? order[j] : 0;
-    const float4 d4 = dir[i];
-    const bool live = j < rays && d4.w != 0.f;
-    const int64_t p = p0 + i / St;
-    const Ray ray = make_ray(ld3w(xg, p), mk3(d4.x, d4.y, d4.z));
-    MarchState<3> st;
-    int32_t* my_ids = (SAVE && live) ? ids + i * (int64_t)max_ids : nullptr;
-    const bool ok = march_forward<3, false>(S, ray, P, st, my_ids, max_ids, live, warp_scratch<false>());
-    if (j >= rays) return;
-    if (!live) {   // every sample gets an entry, so no reader sees unwritten scratch
-        res[i] = make_float4(0.f, 0.f, 0.f, 0.f);
-        if (SAVE) nh[i] = 0;
-        return;
+struct WaveJob {
+    const float* xg;
+    int64_t p0;
+    int St;
+    const float4* dir;
+    const int32_t* order;
+    float4* res;
+    int32_t* nh;
+    int32_t* hit_ids;
+    int max_ids;
+    __device__ __forceinline__ bool load(int j, f3& o, f3& d) const {
+        const int64_t i = order[j];
+        const float4 d4 = dir[i];
+        if (d4.w == 0.f) {   // every sample gets an entry, so no reader sees unwritten scratch
+            res[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+            if (SAVE) nh[i] = 0;
+            return false;
+        }
+        o = ld3w(xg, p0 + i / St);
+        d = mk3(d4.x, d4.y, d4.z);
+        return true;
     }
-    if (!ok) atomicOr(S.status, kErrStackOverflow);
-    res[i] = make_float4(st.C[0], st.C[1], st.C[2], st.T);
-    if (SAVE) {
-        nh[i] = st.nh;
-        if (st.nh < max_ids) my_ids[st.nh] = -1;
+    __device__ __forceinline__ int32_t* ids(int j) const {
+        return SAVE ? hit_ids + order[j] * (int64_t)max_ids : nullptr;
     }
-}
-
-// The same traces in compacted rounds: round 1 on every ray of the order;
-// rays still marching store their state (C, D, T, hit count, next key) at
-// their sorted position and are regrouped, keeping the sorted order, into
-// warps that run to completion. Per ray the rounds and their arithmetic are
-// march_forward's, so the results are the same.
-enum WaveRound { kWaveFirst = 0, kWaveLast = 1 };
-constexpr int kWaveStateF4 = 3;   // C[3], D, T, hit count, next key (2 words), next user index
-
-template <bool SAVE, int MODE>
-__global__ void __launch_bounds__(kWaveThreads, kRayBlocks) k_wave_round(
-    SceneView S, TraceParams P, const float* __restrict__ xg, int64_t p0, int St, const float4* __restrict__ dir,
-    const int32_t* __restrict__ order, int64_t rays, float4* __restrict__ res, int32_t* __restrict__ nh,
-    int32_t* __restrict__ ids, int max_ids, const int32_t* __restrict__ list, const uint32_t* __restrict__ count,
-    float4* __restrict__ state, uint32_t* __restrict__ flags) {
-    const int64_t t = blockIdx.x * (int64_t)kWaveThreads + threadIdx.x;
-    const int64_t n = MODE == kWaveFirst ? rays : (int64_t)*count;
-    if (__all_sync(kFullWarp, t >= n)) return;   // nothing for this warp
-    const bool there = t < n;
-    const int64_t j = !there ? 0 : (MODE == kWaveFirst ? t : (int64_t)list[t]);
-    const int64_t i = order[j];
-    const float4 d4 = dir[i];
-    const bool live = there && d4.w != 0.f;
-    if (MODE == kWaveFirst && there && !live) {   // every sample gets an entry, so no reader sees unwritten scratch
-        res[i] = make_float4(0.f, 0.f, 0.f, 0.f);
-        if (SAVE) nh[i] = 0;
-    }
-    const Ray ray = make_ray(ld3w(xg, p0 + i / St), mk3(d4.x, d4.y, d4.z));
-    MarchState<3> st;
-    st.init();
-    uint64_t last_key = depth_key(P.t_min, 0.f);
-    int32_t last_u = INT32_MAX;
-    if (MODE != kWaveFirst) {
-        const float4 a = state[j * kWaveStateF4], b = state[j * kWaveStateF4 + 1], c = state[j * kWaveStateF4 + 2];
-        st.C[0] = a.x; st.C[1] = a.y; st.C[2] = a.z;
-        st.D = a.w;
-        st.T = b.x;
-        st.nh = __float_as_int(b.y);
-        last_key = ((uint64_t)__float_as_uint(b.w) << 32) | (uint64_t)__float_as_uint(b.z);
-        last_u = __float_as_int(c.x);
-    }
-    int32_t* my_ids = SAVE ? ids + i * (int64_t)max_ids : nullptr;
-    KBuffer<kRayCap> kb;
-    kb.bind();
-    float4* scratch = warp_scratch<false>();
-    bool ok = true, done = !live, packet = false;
-    do {
-        ok &= collect<false>(S, ray, P, last_key, last_u, st.T, kb, !done, packet, scratch);
-        if (!done) done = blend_round<3>(S, ray, P, kb, st, my_ids, max_ids, last_key, last_u);
-    } while (MODE == kWaveLast && __any_sync(kFullWarp, !done));
-    if (!live) return;
-    if (!ok) atomicOr(S.status, kErrStackOverflow);
-    if (done) {
+    __device__ __forceinline__ void finish(int j, const MarchState<3>& st) const {
+        const int64_t i = order[j];
         res[i] = make_float4(st.C[0], st.C[1], st.C[2], st.T);
         if (SAVE) {
             nh[i] = st.nh;
-            if (st.nh < max_ids) my_ids[st.nh] = -1;
+            if (st.nh < max_ids) hit_ids[i * max_ids + st.nh] = -1;
         }
-    } else {
-        state[j * kWaveStateF4] = make_float4(st.C[0], st.C[1], st.C[2], st.D);
-        state[j * kWaveStateF4 + 1] = make_float4(st.T, __int_as_float(st.nh), __uint_as_float((uint32_t)last_key),
-                                                  __uint_as_float((uint32_t)(last_key >> 32)));
-        state[j * kWaveStateF4 + 2] = make_float4(__int_as_float(last_u), 0.f, 0.f, 0.f);
-        flags[j] = 1u;
     }
+};
+
+template <bool SAVE>
+__global__ void __launch_bounds__(kWaveThreads, kRayBlocks) k_wave_trace(SceneView S, TraceParams P, WaveJob<SAVE> job,
+                                                                         int rays, uint32_t* next) {
+    __shared__ SavedMarch<3> saved;
+    walk_batch<3, kRayCap>(S, P, rays, next, job, saved);
+}
+
+// The same with a warp per ray, for batches that do not fill the chip with a
+// ray per lane.
+template <bool SAVE>
+__global__ void __launch_bounds__(kWarpRayThreads, kWarpRayBlocks) k_wave_trace_ray(SceneView S, TraceParams P, WaveJob<SAVE> job,
+                                                                                int rays) {
+    const int j = blockIdx.x * kWarpRays + (threadIdx.x >> 5);
+    f3 o, d;
+    if (j >= rays || !job.load(j, o, d)) return;
+    WarpMarch w;
+    const bool ok = march_warp(S, make_ray(o, d), P, w, job.ids(j), job.max_ids, warp_ray_scratch());
+    MarchState<3> st;
+#pragma unroll
+    for (int c = 0; c < 3; ++c) st.C[c] = __shfl_sync(kFullWarp, w.C, c);
+    st.D = w.D;
+    st.T = w.T;
+    st.nh = w.nh;
+    if ((threadIdx.x & 31) != 0) return;
+    if (!ok) atomicOr(S.status, kErrStackOverflow);
+    job.finish(j, st);
 }
 
 // Per-point estimate from the stored traces (warp per point).
@@ -238,31 +216,6 @@ __global__ void __launch_bounds__(kWaveThreads) k_wave_grad_point(
     }
 }
 
-// Backward of one ray in regrouped order (sorted position j): from its saved
-// hit list (LISTED) or by replaying its march.
-template <bool LISTED>
-__device__ __forceinline__ void wave_backward_ray(const SceneView& S, const TraceParams& P,
-                                                  const float* __restrict__ xg, int64_t p0, int St,
-                                                  const float4* __restrict__ dir, int64_t i,
-                                                  const float4* __restrict__ res, int n_hits,
-                                                  const int32_t* __restrict__ ids, int max_ids, float4 u4,
-                                                  float* __restrict__ acc_rows, float4* scratch, bool live = true) {
-    const float4 d4 = dir[i];
-    const int64_t p = p0 + i / St;
-    const Ray ray = make_ray(ld3w(xg, p), mk3(d4.x, d4.y, d4.z));
-    const float4 t = res[i];
-    const float Cf[3] = {t.x, t.y, t.z};
-    const float gC[3] = {u4.x, u4.y, u4.z};
-    if (LISTED) {
-        listed_backward<3>(S, ray, P, ids + i * (int64_t)max_ids, n_hits, Cf, 0.f, t.w, gC, 0.f, u4.w, acc_rows,
-                           reinterpret_cast<float*>(scratch));
-    } else {
-        const bool ok = march_backward<3, false>(S, ray, P, live, n_hits, Cf, 0.f, t.w, gC, 0.f, u4.w, acc_rows,
-                                                 scratch);
-        if (!ok) atomicOr(S.status, kErrStackOverflow);
-    }
-}
-
 // Backward from the saved hit lists, one thread per sorted ray; rays whose
 // list did not fit (more than max_ids hits) are appended to replay_list for
 // k_wave_replay.
@@ -289,30 +242,34 @@ __global__ void __launch_bounds__(kWaveThreads) k_wave_backward(SceneView S, Tra
         replay_list[atomicAdd(replay_count, 1u)] = (int32_t)j;
         return;
     }
-    wave_backward_ray<true>(S, P, xg, p0, St, dir, i, res, n_hits, ids, max_ids, u4, acc_rows, scratch);
+    const float4 d4 = dir[i], t = res[i];
+    const Ray ray = make_ray(ld3w(xg, p0 + i / St), mk3(d4.x, d4.y, d4.z));
+    const float Cf[3] = {t.x, t.y, t.z}, gC[3] = {u4.x, u4.y, u4.z};
+    listed_backward<3>(S, ray, P, ids + i * (int64_t)max_ids, n_hits, Cf, 0.f, t.w, gC, 0.f, u4.w, acc_rows,
+                       reinterpret_cast<float*>(scratch));
 }
 
-// The rays of replay_list replay their march backwards (the list's length is
-// what the listing launch left in replay_count). Consecutive entries go to
-// different blocks, so the few long replays spread over every SM.
-__global__ void __launch_bounds__(kWaveThreads) k_wave_replay(SceneView S, TraceParams P,
-                                                              const float* __restrict__ xg, int64_t p0, int St,
-                                                              const float4* __restrict__ dir,
-                                                              const int32_t* __restrict__ order,
-                                                              const float4* __restrict__ res,
-                                                              const int32_t* __restrict__ nh,
-                                                              const float4* __restrict__ up,
-                                                              float* __restrict__ acc_rows,
-                                                              const int32_t* __restrict__ replay_list,
-                                                              const uint32_t* __restrict__ replay_count) {
-    float4* scratch = warp_memory<replay_f4<3, false>()>();
+// The rays of replay_list replay their march backwards, a warp per ray (the
+// list's length is what the listing launch left in replay_count): as lanes of
+// their own these few hundred longest rays took 0.9 of a gradient's 10.9 ms.
+__global__ void __launch_bounds__(kWarpRayThreads) k_wave_replay(SceneView S, TraceParams P, const float* __restrict__ xg,
+                                                                 int64_t p0, int St, const float4* __restrict__ dir,
+                                                                 const int32_t* __restrict__ order,
+                                                                 const float4* __restrict__ res,
+                                                                 const int32_t* __restrict__ nh,
+                                                                 const float4* __restrict__ up,
+                                                                 float* __restrict__ acc_rows,
+                                                                 const int32_t* __restrict__ replay_list,
+                                                                 const uint32_t* __restrict__ replay_count) {
     const int64_t n = *replay_count;
-    for (int64_t t = threadIdx.x * (int64_t)gridDim.x + blockIdx.x; __any_sync(kFullWarp, t < n);
-         t += (int64_t)gridDim.x * kWaveThreads) {
-        const bool live = t < n;   // lanes without a ray follow the warp
-        const int64_t i = order[live ? replay_list[t] : 0];
-        wave_backward_ray<false>(S, P, xg, p0, St, dir, i, res, live ? nh[i] : 0, nullptr, 0, up[i], acc_rows, scratch,
-                                 live);
+    const int lane = threadIdx.x & 31;
+    for (int64_t t = blockIdx.x * (int64_t)kWarpRays + (threadIdx.x >> 5); t < n; t += (int64_t)gridDim.x * kWarpRays) {
+        const int64_t i = order[replay_list[t]];
+        const float4 d4 = dir[i], c = res[i], u = up[i];
+        const Ray ray = make_ray(ld3w(xg, p0 + i / St), mk3(d4.x, d4.y, d4.z));
+        const float Cf = lane == 0 ? c.x : (lane == 1 ? c.y : c.z), gC = lane == 0 ? u.x : (lane == 1 ? u.y : u.z);
+        const bool ok = backward_warp<3>(S, ray, P, nh[i], Cf, 0.f, c.w, gC, 0.f, u.w, acc_rows, warp_ray_scratch());
+        if (!ok && lane == 0) atomicOr(S.status, kErrStackOverflow);
     }
 }
 
@@ -330,10 +287,8 @@ struct WaveScratch {
     int32_t* nh = nullptr;
     int32_t* ids = nullptr;
     float4* up = nullptr;
-    uint32_t* flags = nullptr;   // [rays + 1] continue flags, then their prefix sums
-    int32_t* list = nullptr;     // [rays] continuing rays (sorted positions)
-    uint32_t* count = nullptr;   // [1] and the scan's tile sums after it
-    float4* state = nullptr;     // [rays * kWaveStateF4] march state between rounds
+    int32_t* list = nullptr;     // [rays] rays to replay (sorted positions; gradient only)
+    uint32_t* count = nullptr;   // [2] the batch's next pool; rays to replay
     unsigned char* base = nullptr;
 
     cudaError_t alloc(int64_t rays, bool backward, cudaStream_t st) {
@@ -347,14 +302,13 @@ struct WaveScratch {
         const size_t o_dir = take(sizeof(float4) * rays), o_key = take(4 * rays), o_val = take(4 * rays);
         const size_t o_kt = take(4 * rays), o_vt = take(4 * rays), o_hist = take(4 * hw);
         const size_t o_res = take(sizeof(float4) * rays);
-        const size_t o_flags = take(4 * (rays + 1)), o_list = take(4 * rays);
-        const size_t o_count = take(4 * (1 + scan_long_words(rays + 1)));
-        const size_t o_state = take(sizeof(float4) * kWaveStateF4 * rays);
-        size_t o_nh = 0, o_ids = 0, o_up = 0;
+        const size_t o_count = take(8);
+        size_t o_nh = 0, o_ids = 0, o_up = 0, o_list = 0;
         if (backward) {
             o_nh = take(4 * rays);
             o_ids = take(sizeof(int32_t) * kWaveSavedHits * rays);
             o_up = take(sizeof(float4) * rays);
+            o_list = take(4 * rays);
         }
         cudaError_t e = scratch_alloc(reinterpret_cast<void**>(&base), off, st);
         if (e != cudaSuccess) return e;
@@ -365,14 +319,12 @@ struct WaveScratch {
         val_tmp = reinterpret_cast<int32_t*>(base + o_vt);
         hist = reinterpret_cast<uint32_t*>(base + o_hist);
         res = reinterpret_cast<float4*>(base + o_res);
-        flags = reinterpret_cast<uint32_t*>(base + o_flags);
-        list = reinterpret_cast<int32_t*>(base + o_list);
         count = reinterpret_cast<uint32_t*>(base + o_count);
-        state = reinterpret_cast<float4*>(base + o_state);
         if (backward) {
             nh = reinterpret_cast<int32_t*>(base + o_nh);
             ids = reinterpret_cast<int32_t*>(base + o_ids);
             up = reinterpret_cast<float4*>(base + o_up);
+            list = reinterpret_cast<int32_t*>(base + o_list);
         }
         return cudaSuccess;
     }
@@ -385,29 +337,23 @@ int64_t chunk_points(int St) {
 }
 
 // Trace the sorted rays of one chunk into w.res (and, with SAVE, the hit
-// counts and lists): compacted rounds when the scene has surfels.
+// counts and lists).
 template <bool SAVE>
 cudaError_t wave_trace(const SceneView& S, const TraceParams& TP, const float* x, int64_t p0, int St, int64_t rays,
                        WaveScratch& w, cudaStream_t st) {
-    int32_t* ids = SAVE ? w.ids : nullptr;
-    int32_t* nh = SAVE ? w.nh : nullptr;
-    const int max_ids = SAVE ? kWaveSavedHits : 0;
-    if (S.n == 0) {
-        k_wave_trace<SAVE><<<grid_for(rays, kWaveThreads), kWaveThreads, 0, st>>>(S, TP, x, p0, St, w.dir, w.val,
-                                                                                    rays, w.res, nh, ids, max_ids);
+    const cudaError_t e = cudaMemsetAsync(w.count, 0, 2 * sizeof(uint32_t), st);
+    if (e != cudaSuccess) return e;
+    const WaveJob<SAVE> job{x, p0, St, w.dir, w.val, w.res, SAVE ? w.nh : nullptr, SAVE ? w.ids : nullptr,
+                            SAVE ? kWaveSavedHits : 0};
+    if (rays <= kWaveWarpMax) {
+        k_wave_trace_ray<SAVE><<<warp_ray_grid(rays), kWarpRayThreads, 0, st>>>(S, TP, job, (int)rays);
         count_launches(1);
         return cudaGetLastError();
     }
-    const unsigned g = grid_for(rays, kWaveThreads);
-    cudaError_t e = cudaMemsetAsync(w.flags, 0, sizeof(uint32_t) * (rays + 1), st);
-    if (e != cudaSuccess) return e;
-    k_wave_round<SAVE, kWaveFirst><<<g, kWaveThreads, 0, st>>>(S, TP, x, p0, St, w.dir, w.val, rays, w.res, nh, ids,
-                                                               max_ids, w.list, w.count, w.state, w.flags);
-    e = flags_to_list(w.flags, rays, w.count + 1, w.list, w.count, st);
-    if (e != cudaSuccess) return e;
-    k_wave_round<SAVE, kWaveLast><<<g, kWaveThreads, 0, st>>>(S, TP, x, p0, St, w.dir, w.val, rays, w.res, nh, ids,
-                                                              max_ids, w.list, w.count, w.state, w.flags);
-    count_launches(2);
+    const unsigned blocks = batch_blocks(k_wave_trace<SAVE>, rays);
+    if (blocks == 0u) return cudaGetLastError();
+    k_wave_trace<SAVE><<<blocks, kWaveThreads, 0, st>>>(S, TP, job, (int)rays, w.count);
+    count_launches(1);
     return cudaGetLastError();
 }
 
@@ -425,7 +371,7 @@ cudaError_t wave_forward(const SceneView& S, const uint32_t* bounds, const float
         const int64_t rays = np * St;
         k_wave_gen<<<grid_for(rays, 256), 256, 0, st>>>(x, n, r, wo, p0, rays, St, nd, mode, seed, bounds, w.dir,
                                                         w.key, w.val, key_base, valid);
-        e = sort_pairs(w.key, w.val, w.key_tmp, w.val_tmp, w.hist, rays, st);
+        if (rays > kWaveUnsortedMax) e = sort_pairs(w.key, w.val, w.key_tmp, w.val_tmp, w.hist, rays, st);
         if (e != cudaSuccess) break;
         e = wave_trace<false>(S, TP, x, p0, St, rays, w, st);
         if (e != cudaSuccess) break;
@@ -459,19 +405,17 @@ cudaError_t wave_backward(const SceneView& S, const int32_t* perm, const uint32_
         const int64_t rays = np * St;
         k_wave_gen<<<grid_for(rays, 256), 256, 0, st>>>(x, n, r, wo, p0, rays, St, nd, mode, seed, bounds, w.dir,
                                                         w.key, w.val, 0ull, nullptr);
-        e = sort_pairs(w.key, w.val, w.key_tmp, w.val_tmp, w.hist, rays, st);
+        if (rays > kWaveUnsortedMax) e = sort_pairs(w.key, w.val, w.key_tmp, w.val_tmp, w.hist, rays, st);
         if (e != cudaSuccess) break;
         const unsigned g = grid_for(rays, kWaveThreads);
         e = wave_trace<true>(S, TP, x, p0, St, rays, w, st);
         if (e != cudaSuccess) break;
         k_wave_grad_point<<<grid_for(np, kWaveThreads / 32), kWaveThreads, 0, st>>>(
             n, a, r, wo, p0, np, env, H, W, nd, ns, mode, seed, w.res, g_rgb, g_albedo, g_rough, g_env, w.up);
-        e = cudaMemsetAsync(w.count, 0, sizeof(uint32_t), st);
-        if (e != cudaSuccess) break;
         k_wave_backward<<<g, kWaveThreads, 0, st>>>(S, TP, x, p0, St, w.dir, w.val, rays, w.res, w.nh, w.ids,
-                                                       kWaveSavedHits, w.up, acc_rows, w.list, w.count);
-        k_wave_replay<<<kWaveReplayBlocks, kWaveThreads, 0, st>>>(S, TP, x, p0, St, w.dir, w.val, w.res, w.nh,
-                                                                     w.up, acc_rows, w.list, w.count);
+                                                       kWaveSavedHits, w.up, acc_rows, w.list, w.count + 1);
+        k_wave_replay<<<kWaveReplayBlocks, kWarpRayThreads, 0, st>>>(S, TP, x, p0, St, w.dir, w.val, w.res, w.nh,
+                                                                     w.up, acc_rows, w.list, w.count + 1);
         count_launches(4);
         e = cudaGetLastError();
     }

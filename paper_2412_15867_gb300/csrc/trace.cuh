@@ -180,6 +180,11 @@ __device__ __forceinline__ float tslack(float t) { return 1e-5f * (1.0f + fabsf(
 
 __device__ __forceinline__ float key_depth(uint64_t k) { return __uint_as_float((uint32_t)(k >> 32)); }
 
+// User index of the surfel in Morton slot m (carried in its record's r2.w).
+__device__ __forceinline__ int32_t uid_of(const float4* rec, int32_t m) {
+    return __float_as_int(__ldg(&rec[(int64_t)m * kRecF4 + 2].w));
+}
+
 // ---------------------------------------------------------------------------
 // Threads per block of every tracing kernel (k-buffer slots and leaf queues
 // are laid out per block thread).
@@ -191,7 +196,7 @@ constexpr int kTraceThreads = 128;
 constexpr int kPacketCap = 32;
 constexpr int kRayCap = 24;
 constexpr int kPacketBlocks = 4;   // resident blocks per SM that the kernels are compiled for
-constexpr int kRayBlocks = 6;
+constexpr int kRayBlocks = 5;
 template <bool PACKET>
 __host__ __device__ constexpr int walk_cap() { return PACKET ? kPacketCap : kRayCap; }
 
@@ -396,6 +401,109 @@ __device__ __forceinline__ int visit_cap(const SceneView& S) {
     return S.n + 64 < (int64_t)INT32_MAX ? (int)(S.n + 64) : INT32_MAX;
 }
 
+// A ray's walk on its own: the node to visit next (-1: none), pending leaves in
+// its queue, and a stack whose most recent entry is kept in a register. An
+// entry is one word: the entry depth's leading bits (rounded down) above the
+// node's number. The stacks live in local memory and share the L1 with nodes
+// and records: at two words they took as much of it as those.
+struct RayWalk {
+    int ni, qn, sp, visits;
+    uint32_t top;
+    bool has_top, ok;
+    float lo_c, t_hi;
+    __device__ __forceinline__ void start(const SceneView& S, const TraceParams& P, uint64_t last_key) {
+        ni = 0;
+        qn = sp = 0;
+        has_top = false;
+        top = 0u;
+        visits = visit_cap(S);
+        const float t_lo = key_depth(last_key);
+        lo_c = t_lo - tslack(t_lo);
+        t_hi = P.t_max;
+    }
+    __device__ __forceinline__ bool can_walk() const { return ni >= 0 && qn <= kLeafQueue - 4; }
+};
+
+// One pending leaf of the ray.
+template <class KB, bool STATS>
+__device__ __forceinline__ void walk_leaf(const SceneView& S, const Ray& ray, const TraceParams& P, uint64_t last_key,
+                                          int32_t last_u, KB& kb, RayWalk& w, const uint32_t* queue, TraceStats* ts) {
+    --w.qn;
+    const int32_t m = (int32_t)queue[32 * w.qn];
+    const float4* R = S.rec + (int64_t)m * kRecF4;
+    const float4 r0 = ldg4(R), r1 = ldg4(R + 1), r2 = ldg4(R + 2), r3 = ldg4(R + 3);
+    leaf_insert<KB, STATS>(S, ray, P, m, r0, r1, r2, r3, last_key, last_u, kb, w.t_hi, ts);
+}
+
+// One node: its leaves that the ray's box test keeps go to the queue, the
+// nearest inner one is next, the others go onto the stack, farthest first.
+template <bool STATS>
+__device__ __forceinline__ void walk_node(const SceneView& S, const RayBox& rb, RayWalk& w, uint32_t* stack,
+                                          uint32_t* queue, TraceStats* ts) {
+    const uint32_t id_mask = (1u << S.wide_bits) - 1u;
+    auto entry_depth = [&](uint32_t e) { return __uint_as_float((e & ~id_mask) >> 1); };
+    if (--w.visits < 0) {   // each wide node is fetched at most once per round in a valid tree
+        w.ok = false;
+        w.ni = -1;
+        return;
+    }
+    const WideNodeRay nd = load_wide_ray(S.wide, w.ni, rb);
+    if (STATS) ts->nodes++;
+    float tn[4], tf[4];
+    slab4_ray(nd, rb, tn, tf);
+    const int c[4] = {nd.child.x, nd.child.y, nd.child.z, nd.child.w};
+    const float hi_c = w.t_hi + tslack(w.t_hi);
+    // children to enter, nearest first: entry depth (its last two bits
+    // give way to the child's number, which only rounds it down)
+    uint32_t key[4];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+        const bool h = tn[k] <= tf[k] && tf[k] >= w.lo_c && tn[k] <= hi_c;   // empty slots: empty box
+        if (h && c[k] < 0) queue[32 * w.qn++] = (uint32_t)~c[k];
+        key[k] = h && c[k] >= 0 ? (__float_as_uint(fmaxf(tn[k], 0.f)) & ~3u) | (uint32_t)k : 0xffffffffu;
+    }
+    auto order = [&](int a, int b) {
+        const uint32_t lo = min(key[a], key[b]), hi = max(key[a], key[b]);
+        key[a] = lo;
+        key[b] = hi;
+    };
+    order(0, 1);
+    order(2, 3);
+    order(0, 2);
+    order(1, 3);
+    order(1, 2);
+    auto child_of = [&](uint32_t k) {
+        const uint32_t s = k & 3u;
+        const int lo = (s & 1u) ? c[1] : c[0], hi = (s & 1u) ? c[3] : c[2];
+        return (s & 2u) ? hi : lo;
+    };
+    auto entry = [&](uint32_t k) { return ((k << 1) & ~id_mask) | (uint32_t)child_of(k); };
+    if (key[0] == 0xffffffffu) {
+        w.ni = -1;
+        if (w.has_top) {
+            w.has_top = false;
+            if (entry_depth(w.top) <= hi_c) w.ni = (int)(w.top & id_mask);
+        }
+        while (w.ni < 0 && w.sp > 0) {
+            const uint32_t e = stack[--w.sp];
+            if (entry_depth(e) <= hi_c) w.ni = (int)(e & id_mask);
+        }
+        return;
+    }
+    w.ni = child_of(key[0]);
+    if (key[1] != 0xffffffffu) {
+        if (w.sp + 3 > kStackSize) {
+            w.ok = false;
+        } else {
+            if (w.has_top) stack[w.sp++] = w.top;
+            if (key[3] != 0xffffffffu) stack[w.sp++] = entry(key[3]);
+            if (key[2] != 0xffffffffu) stack[w.sp++] = entry(key[2]);
+        }
+        w.top = entry(key[1]);
+        w.has_top = true;
+    }
+}
+
 // One round, one traversal stack per ray: gather the nearest hits strictly
 // after (last_key, last_u). All 32 lanes call this together (lanes without a
 // ray pass active = false). The lanes of a warp walk different nodes, and on
@@ -404,106 +512,28 @@ __device__ __forceinline__ int visit_cap(const SceneView& S) {
 // its leaves and the warp takes the step, node visits or leaf tests, that
 // more of its lanes are ready for. Returns false if a stack overflowed.
 template <class KB, bool STATS = false>
-__device__ __forceinline__ bool collect_round(const SceneView& S, const Ray& ray0, const TraceParams& P,
+__device__ __forceinline__ bool collect_round(const SceneView& S, const Ray& ray, const TraceParams& P,
                                               uint64_t last_key, int32_t last_u, KB& kb, bool active,
                                               float4* scratch, TraceStats* ts = nullptr) {
     uint32_t* queue = reinterpret_cast<uint32_t*>(scratch) + (threadIdx.x & 31);   // entry i at queue[32 i]
-    const RayBox rb = make_ray_box(ray0);
-    // An entry is one word: the entry depth's leading bits (rounded down) above
-    // the node's number. The stacks live in local memory and share the L1 with
-    // nodes and records: at two words they took as much of it as those.
+    const RayBox rb = make_ray_box(ray);
     uint32_t stack[kStackSize];
-    int sp = 0;
-    uint32_t top = 0u;   // the most recent entry, kept in a register
-    bool has_top = false;
-    const uint32_t id_bits = S.wide_bits, id_mask = (1u << id_bits) - 1u;
-    auto entry_depth = [&](uint32_t e) { return __uint_as_float((e & ~id_mask) >> 1); };
-    bool ok = true;
-    const float t_lo = key_depth(last_key);
-    const float lo_c = t_lo - tslack(t_lo);
-    float t_hi = P.t_max;
-    int ni = active ? 0 : -1;
-    int qn = 0;
-    int visits = visit_cap(S);
+    RayWalk w;
+    w.ok = true;
+    w.start(S, P, last_key);
+    if (!active) w.ni = -1;
     for (;;) {
-        const bool can_walk = ni >= 0 && qn <= kLeafQueue - 4;
-        const unsigned walk = __ballot_sync(kFullWarp, can_walk);
-        const unsigned have = __ballot_sync(kFullWarp, qn > 0);
+        const unsigned walk = __ballot_sync(kFullWarp, w.can_walk());
+        const unsigned have = __ballot_sync(kFullWarp, w.qn > 0);
         if ((walk | have) == 0u) break;
         if (__popc(walk) <= __popc(have)) {
-            if (qn > 0) {
-                --qn;
-                const int32_t m = (int32_t)queue[32 * qn];
-                const float4* R = S.rec + (int64_t)m * kRecF4;
-                const float4 r0 = ldg4(R), r1 = ldg4(R + 1), r2 = ldg4(R + 2), r3 = ldg4(R + 3);
-                leaf_insert<KB, STATS>(S, ray0, P, m, r0, r1, r2, r3, last_key, last_u, kb, t_hi, ts);
-            }
-            continue;
-        }
-        if (!can_walk) continue;
-        if (--visits < 0) {   // each wide node is fetched at most once per round in a valid tree
-            ok = false;
-            ni = -1;
-            continue;
-        }
-        const WideNodeRay nd = load_wide_ray(S.wide, ni, rb);
-        if (STATS) ts->nodes++;
-        float tn[4], tf[4];
-        slab4_ray(nd, rb, tn, tf);
-        const int c[4] = {nd.child.x, nd.child.y, nd.child.z, nd.child.w};
-        const float hi_c = t_hi + tslack(t_hi);
-        // children to enter, nearest first: entry depth (its last two bits
-        // give way to the child's number, which only rounds it down)
-        uint32_t key[4];
-#pragma unroll
-        for (int k = 0; k < 4; ++k) {
-            const bool h = tn[k] <= tf[k] && tf[k] >= lo_c && tn[k] <= hi_c;   // empty slots: empty box
-            if (h && c[k] < 0) queue[32 * qn++] = (uint32_t)~c[k];
-            key[k] = h && c[k] >= 0 ? (__float_as_uint(fmaxf(tn[k], 0.f)) & ~3u) | (uint32_t)k : 0xffffffffu;
-        }
-        auto order = [&](int a, int b) {
-            const uint32_t lo = min(key[a], key[b]), hi = max(key[a], key[b]);
-            key[a] = lo;
-            key[b] = hi;
-        };
-        order(0, 1);
-        order(2, 3);
-        order(0, 2);
-        order(1, 3);
-        order(1, 2);
-        auto child_of = [&](uint32_t k) {
-            const uint32_t s = k & 3u;
-            const int lo = (s & 1u) ? c[1] : c[0], hi = (s & 1u) ? c[3] : c[2];
-            return (s & 2u) ? hi : lo;
-        };
-        auto entry = [&](uint32_t k) { return ((k << 1) & ~id_mask) | (uint32_t)child_of(k); };
-        if (key[0] == 0xffffffffu) {
-            ni = -1;
-            if (has_top) {
-                has_top = false;
-                if (entry_depth(top) <= hi_c) ni = (int)(top & id_mask);
-            }
-            while (ni < 0 && sp > 0) {
-                const uint32_t e = stack[--sp];
-                if (entry_depth(e) <= hi_c) ni = (int)(e & id_mask);
-            }
-            continue;
-        }
-        ni = child_of(key[0]);
-        if (key[1] != 0xffffffffu) {
-            if (sp + 3 > kStackSize) {
-                ok = false;
-            } else {
-                if (has_top) stack[sp++] = top;
-                if (key[3] != 0xffffffffu) stack[sp++] = entry(key[3]);
-                if (key[2] != 0xffffffffu) stack[sp++] = entry(key[2]);
-            }
-            top = entry(key[1]);
-            has_top = true;
+            if (w.qn > 0) walk_leaf<KB, STATS>(S, ray, P, last_key, last_u, kb, w, queue, ts);
+        } else {
+            if (w.can_walk()) walk_node<STATS>(S, rb, w, stack, queue, ts);
         }
     }
     __syncwarp();   // the queues' memory may now take another use
-    return ok;
+    return w.ok;
 }
 
 // Bounds of a warp's rays for the packet walk. Axis k is the one the rays
@@ -575,13 +605,14 @@ __device__ __forceinline__ bool make_packet(const Ray& ray, bool active, Packet&
 // lo_t and hi_t? t_in: a lower bound on the depths inside the box. Margins of
 // 2e-6 of the coordinates involved cover the rounding of every step, and
 // comparisons with NaN keep the child.
-__device__ __forceinline__ bool packet_child(const WideNode* wide, int id, int c, const Packet& p, float lo_t,
+__device__ __forceinline__ bool packet_child(const float4* boxes, int id, int c, const Packet& p, float lo_t,
                                              float hi_t, int& child, float& t_in) {
-    const float* w = reinterpret_cast<const float*>(wide + id) + c;   // row r, child c at w[4 r]
-    const float lok = __ldg(w + 4 * p.k), hik = __ldg(w + 4 * (p.k + 3));
-    const float loa = __ldg(w + 4 * p.a), hia = __ldg(w + 4 * (p.a + 3));
-    const float lob = __ldg(w + 4 * p.b), hib = __ldg(w + 4 * (p.b + 3));
-    child = __ldg(reinterpret_cast<const int*>(w) + 24);
+    const float4 lo = ldg4(boxes + (int64_t)id * 8 + 2 * c), hi = ldg4(boxes + (int64_t)id * 8 + 2 * c + 1);
+    child = __float_as_int(lo.w);
+    const f3 lo3 = mk3(lo.x, lo.y, lo.z), hi3 = mk3(hi.x, hi.y, hi.z);
+    const float lok = axis_of(lo3, p.k), hik = axis_of(hi3, p.k);
+    const float loa = axis_of(lo3, p.a), hia = axis_of(hi3, p.a);
+    const float lob = axis_of(lo3, p.b), hib = axis_of(hi3, p.b);
     if (child == kNoChild) return false;
     const float ez = 2e-6f * (fmaxf(fabsf(lok), fabsf(hik)) + p.o_abs);
     const float zn = p.sign > 0.f ? lok : -hik, zf = p.sign > 0.f ? hik : -lok;
@@ -670,7 +701,7 @@ __device__ __forceinline__ int collect_packet(const SceneView& S, const Ray& ray
             sp -= take;
             int child = kNoChild;
             float t_in = 0.f;
-            if (in) in = packet_child(S.wide, (int)ent.x, lane & 3, pk, lo_t, hi_t, child, t_in);
+            if (in) in = packet_child(S.child_box, (int)ent.x, lane & 3, pk, lo_t, hi_t, child, t_in);
             if (STATS && active) ts->nodes += take;
             const unsigned leaves = __ballot_sync(kFullWarp, in && child < 0);
             if (in && child < 0) ws.leaf[nleaf + __popc(leaves & lt)] = (uint32_t)~child;
@@ -866,6 +897,141 @@ __device__ __forceinline__ bool march_forward(const SceneView& S, const Ray& ray
         done = blend_round<FB>(S, ray, P, kb, st, ids, max_ids, last_key, last_u);
     }
     return ok;
+}
+
+// A long batch of rays that walk on their own, in the batch's order: each warp
+// takes kPool of them at a time and keeps its lanes filled. A lane whose walk
+// has ended waits until kFinishLanes lanes have (or nothing else is left to
+// do); these blend together, and each then starts its ray's next round or
+// takes the pool's next ray. (With one ray per lane a warp ran its longest
+// ray's walk with few lanes left, and rays that needed more rounds did so in a
+// launch of their own, mostly alone: 15 of 32 lanes per node step, and a third
+// of the time for a sixth of the rays.) Per ray the rounds and their
+// arithmetic are march_forward's, so the results are the same. The batch holds at most 2^31 - kPool rays.
+//
+// Job: bool load(j, o, d): ray j, or false if there is none to trace (the job
+// has dealt with it); int32_t* ids(j), max_ids: where to save its hit ids;
+// void finish(j, st): its blend. `next`: a zeroed counter of the batch.
+constexpr int kPool = 64;
+constexpr int kFinishLanes = 12;
+template <int FB>
+struct SavedMarch {
+    float v[FB + 3][kTraceThreads];   // C, D, T, hits of each thread's ray between rounds
+};
+template <int FB, int CAP, class Job>
+__device__ __forceinline__ void walk_batch(const SceneView& S, const TraceParams& P, int rays, uint32_t* next,
+                                           const Job& job, SavedMarch<FB>& saved) {
+    uint32_t* queue = reinterpret_cast<uint32_t*>(warp_scratch<false>()) + (threadIdx.x & 31);
+    const int lane = threadIdx.x & 31;
+    const unsigned lt = (1u << lane) - 1u;
+    uint32_t stack[kStackSize];
+    KBuffer<CAP> kb;
+    kb.bind();
+    RayWalk w;
+    w.ok = true;
+    w.ni = -1;
+    w.qn = 0;
+    Ray ray = make_ray(mk3(0.f, 0.f, 0.f), mk3(0.f, 0.f, 1.f));
+    RayBox rb = make_ray_box(ray);
+    uint64_t last_key = 0u;
+    int32_t last_u = 0;
+    int j = -1;                      // this lane's ray
+    bool fresh = false;              // in its first round
+    int pool = 0, pool_end = 0;      // the warp's rays not yet taken
+    bool dry = false;                // the batch has no more
+    for (;;) {
+        const unsigned walk = __ballot_sync(kFullWarp, w.can_walk());
+        const unsigned have = __ballot_sync(kFullWarp, w.qn > 0);
+        const unsigned wait = __ballot_sync(kFullWarp, w.ni < 0 && w.qn == 0 && (j >= 0 || !dry));
+        if (__popc(wait) >= kFinishLanes || (walk | have) == 0u) {
+            if (wait == 0u) break;
+            bool want = false;
+            if (w.ni < 0 && w.qn == 0) {
+                want = true;
+                if (j >= 0) {
+                    MarchState<FB> st;
+                    st.init();
+                    if (!fresh) {
+#pragma unroll
+                        for (int c = 0; c < FB; ++c) st.C[c] = saved.v[c][threadIdx.x];
+                        st.D = saved.v[FB][threadIdx.x];
+                        st.T = saved.v[FB + 1][threadIdx.x];
+                        st.nh = __float_as_int(saved.v[FB + 2][threadIdx.x]);
+                    }
+                    if (blend_round<FB>(S, ray, P, kb, st, job.ids(j), job.max_ids, last_key, last_u)) {
+                        job.finish(j, st);
+                        j = -1;
+                    } else {
+#pragma unroll
+                        for (int c = 0; c < FB; ++c) saved.v[c][threadIdx.x] = st.C[c];
+                        saved.v[FB][threadIdx.x] = st.D;
+                        saved.v[FB + 1][threadIdx.x] = st.T;
+                        saved.v[FB + 2][threadIdx.x] = __int_as_float(st.nh);
+                        fresh = false;
+                        want = false;
+                        kb.open(S.n, st.T, P.T_min);
+                        w.start(S, P, last_key);
+                    }
+                }
+            }
+            // new rays for the lanes that want one: the pool's, then one more pool's
+            bool got = false;
+            unsigned need = __ballot_sync(kFullWarp, want);
+#pragma unroll
+            for (int turn = 0; turn < 2; ++turn) {
+                const int mine = pool + __popc(need & lt);
+                if (want && mine < pool_end) {
+                    j = mine;
+                    want = false;
+                    got = true;
+                }
+                pool = min(pool + __popc(need), pool_end);
+                need = __ballot_sync(kFullWarp, want);
+                if (turn == 0 && need != 0u && !dry) {
+                    uint32_t first = 0u;
+                    if (lane == 0) first = atomicAdd(next, 1u);
+                    first = __shfl_sync(kFullWarp, first, 0);
+                    dry = first >= (uint32_t)(rays + kPool - 1) / kPool;
+                    pool = dry ? 0 : (int)first * kPool;
+                    pool_end = dry ? 0 : min(pool + kPool, rays);
+                }
+            }
+            if (got) {
+                f3 o, d;
+                if (job.load(j, o, d)) {
+                    ray = make_ray(o, d);
+                    rb = make_ray_box(ray);
+                    last_key = depth_key(P.t_min, 0.f);
+                    last_u = INT32_MAX;
+                    fresh = true;
+                    kb.open(S.n, 1.f, P.T_min);
+                    w.start(S, P, last_key);
+                } else {
+                    j = -1;
+                }
+            }
+            continue;
+        }
+        if (__popc(walk) <= __popc(have)) {
+            if (w.qn > 0) walk_leaf<KBuffer<CAP>, false>(S, ray, P, last_key, last_u, kb, w, queue, nullptr);
+        } else {
+            if (w.can_walk()) walk_node<false>(S, rb, w, stack, queue, nullptr);
+        }
+    }
+    if (!w.ok) atomicOr(S.status, kErrStackOverflow);
+}
+
+// Blocks of a walk_batch launch: what the device holds, or fewer for a batch
+// that has not a pool for each of their warps. 0 on an error.
+template <class Kernel>
+inline unsigned batch_blocks(Kernel kernel, int64_t rays) {
+    int device = 0, sms = 0, per_sm = 0;
+    if (cudaGetDevice(&device) != cudaSuccess ||
+        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, device) != cudaSuccess ||
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, kTraceThreads, 0) != cudaSuccess)
+        return 0u;
+    const int64_t need = (rays + kTraceThreads - 1) / kTraceThreads, hold = (int64_t)sms * per_sm;
+    return (unsigned)(need < hold ? need : hold);
 }
 
 __host__ __device__ inline TraceParams to_params(const irgs_trace_params& p) {

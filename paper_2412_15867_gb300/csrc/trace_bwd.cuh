@@ -21,6 +21,7 @@
 #include <cuda_runtime.h>
 
 #include "trace.cuh"
+#include "trace_warp.cuh"
 
 namespace irgs {
 
@@ -124,41 +125,19 @@ struct BwdAcc {
     }
 };
 
-// Gradient of the next blended hit, surfel m (Morton slot), given the
-// forward's outputs (Cf, Df, Tfin) and the upstream gradients: recomputes
-// the hit with the forward's arithmetic (bitwise the same alpha and depth),
-// adds its row to the accumulator and advances the running state.
+// The gradient row of one hit of surfel m (Morton slot) with the geometry hg, of
+// alpha a, transmittance T in front of it and weight w = T a, given dL/dalpha =
+// dA and the upstream gradients.
 template <int FB>
-__device__ __forceinline__ void backward_hit(const SceneView& S, const Ray& ray, const TraceParams& P, int32_t m,
-                                             BwdAcc<FB>& st, const float (&Cf)[FB], float Df, float Tfin,
-                                             const float (&gC)[FB], float gD, float gO,
-                                             float* __restrict__ acc_rows, float* rows) {
-    const float4* Rp = S.rec + (int64_t)m * kRecF4;
-    const float4 r0 = ldg4(Rp), r1 = ldg4(Rp + 1), r2 = ldg4(Rp + 2), r3 = ldg4(Rp + 3);
-    float kh, kl, a;
-    HitGeom hg;
-    surfel_hit<true>(r0, r1, r2, r3, ray, P.alpha_min, P.alpha_max, kh, kl, a, &hg);
-    const float tau = kh + 0.0f;
-    const float w = __fmul_rn(st.T, a);
-    float fv[FB];
-    load_channels<FB>(S.feat + (int64_t)m * S.F + P.off, P.fc, ((S.F | P.off) & 1) == 0, fv);
-    float v = __fmul_rn(gD, tau), Sj = 0.f;
-#pragma unroll
-    for (int c = 0; c < FB; ++c) {
-        st.C[c] = c < P.fc ? __fmaf_rn(w, fv[c], st.C[c]) : 0.f;
-        v = fmaf(gC[c], fv[c], v);
-        Sj = fmaf(gC[c], Cf[c] - st.C[c], Sj);
-    }
-    st.D = __fmaf_rn(w, tau, st.D);
-    Sj = fmaf(gD, Df - st.D, Sj);
-    // gradients need no correctly rounded quotients: one 2-ulp reciprocal
-    // (__fdividef) per divisor; every divisor here is a normal number
-    const float dA = st.T * v - (Sj - gO * Tfin) * __fdividef(1.0f, 1.0f - a);
-
+__device__ __forceinline__ void hit_row(const SceneView& S, const Ray& ray, const TraceParams& P, int32_t m,
+                                        const float4& r1, const float4& r2, const float4& r3, const HitGeom& hg,
+                                        float a, float w, float dA, const float (&gC)[FB], float gD,
+                                        GradRow<FB>& gv) {
     const float2 sc = __ldg(&S.scale[m]);
     const float4 q = __ldg(&S.q_raw[m]);
+    // gradients need no correctly rounded quotients: one 2-ulp reciprocal
+    // (__fdividef) per divisor; every divisor here is a normal number
     const float isx = __fdividef(1.0f, sc.x), isy = __fdividef(1.0f, sc.y);
-    GradRow<FB> gv;
     const bool clamped = hg.a_raw >= P.alpha_max;
     const float g_o = clamped ? 0.f : dA * hg.G;
     const float g_rho2 = clamped ? 0.f : -0.5f * dA * a;
@@ -192,8 +171,113 @@ __device__ __forceinline__ void backward_hit(const SceneView& S, const Ray& ray,
     gv.v[9] = -gvv * hg.v * isy;
 #pragma unroll
     for (int c = 0; c < GradRow<FB>::N - 10; ++c) gv.v[10 + c] = c < FB ? w * gC[c] : 0.f;
+}
+
+// Gradient of the next blended hit, surfel m (Morton slot), given the
+// forward's outputs (Cf, Df, Tfin) and the upstream gradients: recomputes
+// the hit with the forward's arithmetic (bitwise the same alpha and depth),
+// adds its row to the accumulator and advances the running state.
+template <int FB>
+__device__ __forceinline__ void backward_hit(const SceneView& S, const Ray& ray, const TraceParams& P, int32_t m,
+                                             BwdAcc<FB>& st, const float (&Cf)[FB], float Df, float Tfin,
+                                             const float (&gC)[FB], float gD, float gO,
+                                             float* __restrict__ acc_rows, float* rows) {
+    const float4* Rp = S.rec + (int64_t)m * kRecF4;
+    const float4 r0 = ldg4(Rp), r1 = ldg4(Rp + 1), r2 = ldg4(Rp + 2), r3 = ldg4(Rp + 3);
+    float kh, kl, a;
+    HitGeom hg;
+    surfel_hit<true>(r0, r1, r2, r3, ray, P.alpha_min, P.alpha_max, kh, kl, a, &hg);
+    const float tau = kh + 0.0f;
+    const float w = __fmul_rn(st.T, a);
+    float fv[FB];
+    load_channels<FB>(S.feat + (int64_t)m * S.F + P.off, P.fc, ((S.F | P.off) & 1) == 0, fv);
+    float v = __fmul_rn(gD, tau), Sj = 0.f;
+#pragma unroll
+    for (int c = 0; c < FB; ++c) {
+        st.C[c] = c < P.fc ? __fmaf_rn(w, fv[c], st.C[c]) : 0.f;
+        v = fmaf(gC[c], fv[c], v);
+        Sj = fmaf(gC[c], Cf[c] - st.C[c], Sj);
+    }
+    st.D = __fmaf_rn(w, tau, st.D);
+    Sj = fmaf(gD, Df - st.D, Sj);
+    const float dA = st.T * v - (Sj - gO * Tfin) * __fdividef(1.0f, 1.0f - a);
+    GradRow<FB> gv;
+    hit_row<FB>(S, ray, P, m, r1, r2, r3, hg, a, w, dA, gC, gD, gv);
     accumulate_row<FB>(gv, m, acc_rows, rows);
     st.T = __fmul_rn(st.T, __fsub_rn(1.0f, a));
+}
+
+// Backward of the warp's ray by a replay with a warp per ray: the rounds and
+// their blend as in march_warp (at most nh_total hits), then every lane the
+// gradient of its own hit. The suffix S_j of a hit is the sum over the round's
+// hits behind it, by a scan, and what the forward's totals leave beyond the
+// round. A ray meets a surfel once, so its rows need no exchange. Cf_lane and
+// gC_lane: channel `lane` of the forward's sums and their upstream gradients.
+template <int FB>
+__device__ __forceinline__ bool backward_warp(const SceneView& S, const Ray& ray, const TraceParams& P, int nh_total,
+                                              float Cf_lane, float Df, float Tfin, float gC_lane, float gD, float gO,
+                                              float* __restrict__ acc_rows, WarpRayScratch& ws) {
+    constexpr int N = GradRow<FB>::N;
+    const int lane = threadIdx.x & 31;
+    const RayBox rb = make_ray_box(ray);
+    uint64_t last_key = depth_key(P.t_min, 0.f);
+    int32_t last_u = INT32_MAX;
+    WarpMarch st;
+    st.init();
+    bool ok = true;
+    float gC[FB];
+#pragma unroll
+    for (int c = 0; c < FB; ++c) gC[c] = __shfl_sync(kFullWarp, gC_lane, c);
+    while (st.nh < nh_total) {
+        WarpHits h;
+        ok &= collect_warp(S, ray, rb, P, last_key, last_u, st.T, ws, h);
+        float T;
+        const int done = blend_warp(S, P, h, nh_total - st.nh, st, T);
+        float beyond = lane < P.fc ? gC_lane * (Cf_lane - st.C) : 0.f;
+#pragma unroll
+        for (int off = 16; off > 0; off >>= 1) beyond += __shfl_xor_sync(kFullWarp, beyond, off);
+        beyond = fmaf(gD, Df - st.D, beyond);
+        float4 r1, r2, r3;
+        HitGeom hg;
+        float a = 0.f, w = 0.f, v = 0.f;
+        if (lane < done) {
+            const float4* Rp = S.rec + (int64_t)h.m * kRecF4;
+            const float4 r0 = ldg4(Rp);
+            r1 = ldg4(Rp + 1);
+            r2 = ldg4(Rp + 2);
+            r3 = ldg4(Rp + 3);
+            float kh, kl;
+            surfel_hit<true>(r0, r1, r2, r3, ray, P.alpha_min, P.alpha_max, kh, kl, a, &hg);
+            w = __fmul_rn(T, a);
+            float fv[FB];
+            load_channels<FB>(S.feat + (int64_t)h.m * S.F + P.off, P.fc, ((S.F | P.off) & 1) == 0, fv);
+            v = __fmul_rn(gD, kh + 0.0f);
+#pragma unroll
+            for (int c = 0; c < FB; ++c) v = fmaf(gC[c], fv[c], v);
+        }
+        float suffix = w * v;   // inclusive: this hit's and those behind it
+#pragma unroll
+        for (int off = 1; off < 32; off <<= 1) {
+            const float y = __shfl_down_sync(kFullWarp, suffix, off);
+            if (lane + off < 32) suffix += y;
+        }
+        float Sj = __shfl_down_sync(kFullWarp, suffix, 1);
+        Sj = (lane == 31 ? 0.f : Sj) + beyond;
+        if (lane < done) {
+            const float dA = T * v - (Sj - gO * Tfin) * __fdividef(1.0f, 1.0f - a);
+            GradRow<FB> gv;
+            hit_row<FB>(S, ray, P, h.m, r1, r2, r3, hg, a, w, dA, gC, gD, gv);
+            float4* dst = reinterpret_cast<float4*>(acc_rows + (int64_t)h.m * N);
+#pragma unroll
+            for (int q = 0; q < N / 4; ++q)
+                atomicAdd(dst + q, make_float4(gv.v[4 * q], gv.v[4 * q + 1], gv.v[4 * q + 2], gv.v[4 * q + 3]));
+        }
+        st.nh += done;
+        if (!h.closed || done == 0) break;
+        last_key = h.key_of(h.cnt - 1);
+        last_u = uid_of(S.rec, __shfl_sync(kFullWarp, h.m, h.cnt - 1));
+    }
+    return ok;
 }
 
 // Replay of one ray (all 32 lanes together): the march is repeated with the

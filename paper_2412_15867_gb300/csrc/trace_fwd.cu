@@ -3,6 +3,7 @@
 
 #include "scene.h"
 #include "trace.cuh"
+#include "trace_warp.cuh"
 
 namespace irgs {
 namespace {
@@ -62,6 +63,30 @@ __global__ void __launch_bounds__(kTraceThreads, kPacketBlocks) k_trace_forward(
 #pragma unroll
     for (int c = 0; c < FB; ++c)
         if (c < P.fc) feat[r * P.fc + c] = st.C[c];
+    depth[r] = st.D;
+    opac[r] = 1.0f - st.T;
+    if (nhits != nullptr) nhits[r] = st.nh;
+}
+
+// One warp per ray.
+__global__ void __launch_bounds__(kWarpRayThreads, kWarpRayBlocks) k_trace_ray(SceneView S, const float* __restrict__ ro,
+                                                                               const float* __restrict__ rd, int64_t R,
+                                                                               TraceParams P, float* __restrict__ feat,
+                                                                               float* __restrict__ depth,
+                                                                               float* __restrict__ opac,
+                                                                               int32_t* __restrict__ nhits,
+                                                                               int32_t* __restrict__ ids, int max_ids) {
+    const int64_t r = blockIdx.x * (int64_t)kWarpRays + (threadIdx.x >> 5);
+    const int lane = threadIdx.x & 31;
+    if (r >= R) return;
+    const Ray ray = make_ray(mk3(ro[3 * r], ro[3 * r + 1], ro[3 * r + 2]), mk3(rd[3 * r], rd[3 * r + 1], rd[3 * r + 2]));
+    int32_t* my_ids = ids != nullptr ? ids + r * (int64_t)max_ids : nullptr;
+    WarpMarch st;
+    const bool ok = march_warp(S, ray, P, st, my_ids, max_ids, warp_ray_scratch());
+    if (lane < P.fc) feat[r * P.fc + lane] = st.C;
+    if (lane != 0) return;
+    if (my_ids != nullptr && st.nh < max_ids) my_ids[st.nh] = -1;   // terminator
+    if (!ok) atomicOr(S.status, kErrStackOverflow);
     depth[r] = st.D;
     opac[r] = 1.0f - st.T;
     if (nhits != nullptr) nhits[r] = st.nh;
@@ -280,6 +305,11 @@ irgs_status launch_trace_forward(const SceneView& S, const float* ro, const floa
                                  int32_t* nhits, int32_t* ids, int32_t max_ids, cudaStream_t st) {
     if (R == 0) return IRGS_OK;
     const TraceParams P = to_params(p);
+    if (p.flags == 0u && R <= kWarpRayMax) {
+        k_trace_ray<<<warp_ray_grid(R), kWarpRayThreads, 0, st>>>(S, ro, rd, R, P, feat, depth, opac, nhits, ids, max_ids);
+        count_launches(1);
+        return cudaGetLastError() == cudaSuccess ? IRGS_OK : IRGS_ERR_CUDA;
+    }
     const bool packet = (p.flags & IRGS_FLAG_PER_THREAD) == 0u;
     const cudaError_t e = packet ? launch_f<true>(S, ro, rd, R, P, feat, depth, opac, nhits, ids, max_ids, st)
                                  : launch_f<false>(S, ro, rd, R, P, feat, depth, opac, nhits, ids, max_ids, st);
