@@ -1317,13 +1317,6 @@ cudaError_t sort_pairs(uint32_t* keys, int32_t* vals, uint32_t* keys_tmp, int32_
     return cudaGetLastError();
 }
 
-cudaError_t scan_exclusive(uint32_t* a, int64_t m, cudaStream_t st) {
-    if (m <= 0) return cudaSuccess;
-    k_scan_exclusive<<<1, 1024, 0, st>>>(a, m);
-    count_launches(1);
-    return cudaGetLastError();
-}
-
 int64_t scan_long_words(int64_t m) { return (m + kScanTile - 1) / kScanTile + 1; }
 
 namespace {
