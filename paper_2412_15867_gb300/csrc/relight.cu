@@ -509,7 +509,7 @@ __global__ void __launch_bounds__(kRelightThreads, kRayBlocks) k_relight_trace(S
                                                                                RelightJob job, int rays,
                                                                                uint32_t* next) {
     __shared__ SavedMarch<7> saved;
-    walk_batch<7, kRayCap>(S, P, rays, next, job, saved);
+    walk_batch<7, kCap>(S, P, rays, next, job, saved);
 }
 
 // The same with a warp per ray, for batches that do not fill the chip many

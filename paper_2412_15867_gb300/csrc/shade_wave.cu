@@ -122,7 +122,7 @@ template <bool SAVE>
 __global__ void __launch_bounds__(kWaveThreads, kRayBlocks) k_wave_trace(SceneView S, TraceParams P, WaveJob<SAVE> job,
                                                                          int rays, uint32_t* next) {
     __shared__ SavedMarch<3> saved;
-    walk_batch<3, kRayCap>(S, P, rays, next, job, saved);
+    walk_batch<3, kCap>(S, P, rays, next, job, saved);
 }
 
 // The same with a warp per ray, for batches that do not fill the chip with a

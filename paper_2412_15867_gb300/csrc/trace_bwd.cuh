@@ -301,7 +301,7 @@ __device__ __forceinline__ bool march_backward(const SceneView& S, const Ray& ra
     int nh = 0;
     uint64_t last_key = depth_key(P.t_min, 0.f);
     int32_t last_u = INT32_MAX;
-    KBuffer<walk_cap<PACKET>()> kb;
+    KBuffer<kCap> kb;
     kb.bind();
     bool ok = true, done = !live, packet = true;
     while (__any_sync(kFullWarp, !done)) {

@@ -145,7 +145,7 @@ __global__ void __launch_bounds__(kTraceThreads, kPacketBlocks) k_trace_round(
         last_u = __float_as_int(w[FB + 5]);
     }
     int32_t* my_ids = (ids != nullptr && live) ? ids + r * (int64_t)max_ids : nullptr;
-    KBuffer<kPacketCap> kb;
+    KBuffer<kCap> kb;
     kb.bind();
     float4* scratch = warp_scratch<true>();
     bool ok = true, done = !live, packet = true;
