@@ -61,12 +61,22 @@ __device__ __forceinline__ float texel_solid_angle(int H, int W, int row) {
 // pair, 1.1e9 pairs for the prefilter of a 512 x 256 environment; computing
 // both per pair took 25 ms (prefilter) and 1.2 ms (irradiance). Here a block
 // makes the directions of 128 texels at a time once for its 128 x kMapTexels
-// outputs, all prefilter levels share a pair's geometry, and a warp whose 32
-// outputs (an 8 x 4 patch) all face away skips the weights.
+// outputs, all prefilter levels share a pair's geometry, and a warp whose
+// outputs (8 x 4 patches) all face away skips the weights.
+//
+// Bound by instruction issue: a thread's two outputs are one packed pair of
+// FP32 lanes, which halves the arithmetic but for the reciprocals (one per output
+// and level). A slice is every so-many-th chunk of 128 texels, so that each sees
+// all of the sphere (contiguous ones face some tiles wholly and others not at
+// all); an odd number of slices walks through the columns of maps of 2^k
+// columns. An environment of 512 x 256 and the relighting of 4,096 points under
+// it take 2.98 ms (3.50 without pairs; 27 prefilter slices, as many blocks as
+// fit at once, 3.18; 127 slices 2.95, for twice the memory).
 constexpr int kMapThreads = 128;
 constexpr int kMapTexels = 2;      // output texels per thread
-constexpr int kMapSlice = 2048;    // least environment texels per slice
-constexpr int kMapMaxSlices = 64;
+constexpr int kMapSlice = 512;     // least environment texels per slice
+constexpr int kPrefSlices = 63;    // x 32 tiles
+constexpr int kIrrSlices = 217;    // x 8 tiles
 
 // Output texel (row, col) of thread t of tile `tile`, its j-th: warps cover
 // patches of 8 columns x 4 rows, the j-th patch 4 rows further down.
@@ -76,55 +86,131 @@ __device__ __forceinline__ void map_texel(int w, int tile, int j, int& row, int&
     col = patch % across * 8 + (threadIdx.x & 7);
 }
 
-// Texels [begin, end) of the environment, by chunks: fn(direction and solid
-// angle, radiance) for each.
+// A pair of FP32 lanes, each rounded as the scalar operation.
+__device__ __forceinline__ uint64_t pack2(float2 a) { return (uint64_t)__float_as_uint(a.y) << 32 | __float_as_uint(a.x); }
+__device__ __forceinline__ float2 unpack2(uint64_t a) {
+    return make_float2(__uint_as_float((uint32_t)a), __uint_as_float((uint32_t)(a >> 32)));
+}
+__device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c) {
+    uint64_t r;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(pack2(a)), "l"(pack2(b)), "l"(pack2(c)));
+    return unpack2(r);
+}
+__device__ __forceinline__ float2 mul2(float2 a, float2 b) {
+    uint64_t r;
+    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(pack2(a)), "l"(pack2(b)));
+    return unpack2(r);
+}
+__device__ __forceinline__ float2 add2(float2 a, float2 b) {
+    uint64_t r;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(pack2(a)), "l"(pack2(b)));
+    return unpack2(r);
+}
+// Within 1 ulp for normal x (the division of __fdividef without its scaling of
+// denormal divisors).
+__device__ __forceinline__ float reciprocal(float x) {
+    float r;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+    return r;
+}
+__device__ __forceinline__ float2 both(float a) { return make_float2(a, a); }
+
+// A texel of the environment: direction, solid angle and radiance, each twice.
+struct MapTexel {
+    float2 dx, dy, dz, omega, ex, ey, ez, pad;
+};
+
+// The texels of slice blockIdx.y: fn(texel, whether the radiance of its chunk
+// is finite) for each. The second is a type: asked per texel and level it took
+// a quarter of the kernel's time.
+template <bool YES>
+struct Finite {};
 template <class Fn>
-__device__ __forceinline__ void for_texels(const float* __restrict__ env, int H, int W, int64_t begin, int64_t end,
-                                           Fn fn) {
-    __shared__ float4 s_dir[kMapThreads], s_val[kMapThreads];
-    for (int64_t t0 = begin; t0 < end; t0 += kMapThreads) {
+__device__ __forceinline__ void for_texels(const float* __restrict__ env, int H, int W, Fn fn) {
+    __shared__ MapTexel s_tex[kMapThreads];
+    const int64_t all = (int64_t)H * W;
+    for (int64_t t0 = (int64_t)blockIdx.y * kMapThreads; t0 < all; t0 += (int64_t)gridDim.y * kMapThreads) {
         const int64_t t = t0 + threadIdx.x;
-        if (t < end) {
+        bool finite = true;
+        if (t < all) {
             const int r = (int)(t / W), c = (int)(t - (int64_t)r * W);
-            const f3 d = texel_dir(H, W, r, c);
-            s_dir[threadIdx.x] = make_float4(d.x, d.y, d.z, texel_solid_angle(H, W, r));
-            s_val[threadIdx.x] = make_float4(env[3 * t], env[3 * t + 1], env[3 * t + 2], 0.f);
+            const f3 d = texel_dir(H, W, r, c), e = mk3(env[3 * t], env[3 * t + 1], env[3 * t + 2]);
+            MapTexel m;
+            m.dx = both(d.x);
+            m.dy = both(d.y);
+            m.dz = both(d.z);
+            m.omega = both(texel_solid_angle(H, W, r));
+            m.ex = both(e.x);
+            m.ey = both(e.y);
+            m.ez = both(e.z);
+            m.pad = both(0.f);
+            s_tex[threadIdx.x] = m;
+            finite = fabsf(e.x) < INFINITY && fabsf(e.y) < INFINITY && fabsf(e.z) < INFINITY;
         }
-        __syncthreads();
-        const int n = (int)(end - t0 < kMapThreads ? end - t0 : kMapThreads);
-        for (int i = 0; i < n; ++i) fn(s_dir[i], s_val[i]);
+        finite = __syncthreads_and(finite);
+        const int n = (int)(all - t0 < kMapThreads ? all - t0 : kMapThreads);
+        if (finite)
+            for (int i = 0; i < n; ++i) fn(s_tex[i], Finite<true>());
+        else
+            for (int i = 0; i < n; ++i) fn(s_tex[i], Finite<false>());
         __syncthreads();
     }
 }
 
-// Irradiance partial sums: part[slice][texel] = sum E max(0, w.N) dOmega.
-__global__ void __launch_bounds__(kMapThreads) k_irradiance(const float* __restrict__ env, int H, int W, int slices,
-                                                            float4* __restrict__ part) {
-    f3 N[kMapTexels];
-    int id[kMapTexels];
-    float acc[kMapTexels][3] = {};
+// Directions of a thread's two outputs, and their texels.
+struct PairDir {
+    float2 x, y, z;
+};
+__device__ __forceinline__ PairDir pair_dir(int h, int w, int (&id)[2]) {
+    static_assert(kMapTexels == 2, "two outputs are a packed pair");
+    f3 d[2];
 #pragma unroll
-    for (int j = 0; j < kMapTexels; ++j) {
+    for (int j = 0; j < 2; ++j) {
         int row, col;
-        map_texel(kIrrW, blockIdx.x, j, row, col);
-        N[j] = texel_dir(kIrrH, kIrrW, row, col);
-        id[j] = row * kIrrW + col;
+        map_texel(w, blockIdx.x, j, row, col);
+        d[j] = texel_dir(h, w, row, col);
+        id[j] = row * w + col;
     }
-    const int64_t n = (int64_t)H * W;
-    for_texels(env, H, W, n * blockIdx.y / slices, n * (blockIdx.y + 1) / slices, [&](const float4& d, const float4& e) {
+    return {make_float2(d[0].x, d[1].x), make_float2(d[0].y, d[1].y), make_float2(d[0].z, d[1].z)};
+}
+
+// Projected solid angle of a texel for a pair of outputs, zero for one that it
+// does not face.
+__device__ __forceinline__ float2 facing(float2 cs, const MapTexel& t) {
+    return make_float2(cs.x > 0.f ? cs.x * t.omega.x : 0.f, cs.y > 0.f ? cs.y * t.omega.y : 0.f);
+}
+
+// acc += radiance x weight. Infinities and NaN must not meet the zero weight of
+// the output that the texel does not face: chunks that hold any take the
+// outputs one by one.
+template <bool FINITE>
+__device__ __forceinline__ void add_weighted(float2* acc, const MapTexel& t, float2 wgt, float2 cs, Finite<FINITE>) {
+    const float2 e[3] = {t.ex, t.ey, t.ez};
 #pragma unroll
-        for (int j = 0; j < kMapTexels; ++j) {
-            const float cs = dot3(mk3(d.x, d.y, d.z), N[j]);
-            if (!(cs > 0.f)) continue;
-            const float w = cs * d.w;
-            acc[j][0] = fmaf(e.x, w, acc[j][0]);
-            acc[j][1] = fmaf(e.y, w, acc[j][1]);
-            acc[j][2] = fmaf(e.z, w, acc[j][2]);
+    for (int c = 0; c < 3; ++c) {
+        if (FINITE) {
+            acc[c] = fma2(e[c], wgt, acc[c]);
+        } else {
+            if (cs.x > 0.f) acc[c].x = fmaf(e[c].x, wgt.x, acc[c].x);
+            if (cs.y > 0.f) acc[c].y = fmaf(e[c].y, wgt.y, acc[c].y);
         }
+    }
+}
+
+// Irradiance partial sums: part[slice][texel] = sum E max(0, w.N) dOmega.
+__global__ void __launch_bounds__(kMapThreads) k_irradiance(const float* __restrict__ env, int H, int W,
+                                                            float4* __restrict__ part) {
+    int id[2];
+    const PairDir N = pair_dir(kIrrH, kIrrW, id);
+    float2 acc[3] = {both(0.f), both(0.f), both(0.f)};
+    for_texels(env, H, W, [&](const MapTexel& t, auto finite) {
+        const float2 cs = fma2(t.dx, N.x, fma2(t.dy, N.y, mul2(t.dz, N.z)));
+        if (!(cs.x > 0.f || cs.y > 0.f)) return;
+        add_weighted(acc, t, facing(cs, t), cs, finite);
     });
-#pragma unroll
-    for (int j = 0; j < kMapTexels; ++j)
-        part[(int64_t)blockIdx.y * (kIrrH * kIrrW) + id[j]] = make_float4(acc[j][0], acc[j][1], acc[j][2], 0.f);
+    float4* out = part + (int64_t)blockIdx.y * (kIrrH * kIrrW);
+    out[id[0]] = make_float4(acc[0].x, acc[1].x, acc[2].x, 0.f);
+    out[id[1]] = make_float4(acc[0].y, acc[1].y, acc[2].y, 0.f);
 }
 
 // Prefilter partial sums of every level: part[slice][level - 1][texel] = sums
@@ -132,60 +218,52 @@ __global__ void __launch_bounds__(kMapThreads) k_irradiance(const float* __restr
 // cancels in their ratio). With the half vector h of the unit vectors w and R,
 // |R x h|^2 = |w - R|^2 / 4 and (R.h)^2 is one less that: no h is needed, and
 // nothing cancels near the peak.
-__global__ void __launch_bounds__(kMapThreads) k_prefilter(const float* __restrict__ env, int H, int W, int slices,
+__global__ void __launch_bounds__(kMapThreads) k_prefilter(const float* __restrict__ env, int H, int W,
                                                            float4* __restrict__ part) {
     constexpr int kL = kLevels - 1;
-    f3 R[kMapTexels];
-    int id[kMapTexels];
-    float4 acc[kMapTexels][kL];
+    int id[2];
+    const PairDir R = pair_dir(kPrefH, kPrefW, id);
+    float2 acc[kL][4];
 #pragma unroll
-    for (int j = 0; j < kMapTexels; ++j) {
-        int row, col;
-        map_texel(kPrefW, blockIdx.x, j, row, col);
-        R[j] = texel_dir(kPrefH, kPrefW, row, col);
-        id[j] = row * kPrefW + col;
+    for (int l = 0; l < kL; ++l)
 #pragma unroll
-        for (int l = 0; l < kL; ++l) acc[j][l] = make_float4(0.f, 0.f, 0.f, 0.f);
-    }
-    const int64_t n = (int64_t)H * W;
-    for_texels(env, H, W, n * blockIdx.y / slices, n * (blockIdx.y + 1) / slices, [&](const float4& d, const float4& e) {
+        for (int c = 0; c < 4; ++c) acc[l][c] = both(0.f);
+    for_texels(env, H, W, [&](const MapTexel& t, auto finite) {
+        const float2 cs = fma2(t.dx, R.x, fma2(t.dy, R.y, mul2(t.dz, R.z)));
+        if (!(cs.x > 0.f || cs.y > 0.f)) return;
+        const float2 w = facing(cs, t);
+        const float2 gx = fma2(R.x, both(-1.f), t.dx), gy = fma2(R.y, both(-1.f), t.dy), gz = fma2(R.z, both(-1.f), t.dz);
+        const float2 x2 = mul2(both(0.25f), fma2(gx, gx, fma2(gy, gy, mul2(gz, gz))));
+        const float2 nh2 = fma2(x2, both(-1.f), both(1.f));
 #pragma unroll
-        for (int j = 0; j < kMapTexels; ++j) {
-            const float cs = dot3(mk3(d.x, d.y, d.z), R[j]);
-            if (!(cs > 0.f)) continue;
-            const float w = cs * d.w;
-            const f3 g = mk3(d.x - R[j].x, d.y - R[j].y, d.z - R[j].z);
-            const float x2 = 0.25f * dot3(g, g), nh2 = 1.f - x2;
-#pragma unroll
-            for (int l = 0; l < kL; ++l) {
-                const float rho = (float)(l + 1) / (float)(kLevels - 1);
-                const float q = fmaf(nh2, rho * rho * rho * rho, x2);   // (n.h)^2 (a2 - 1) + 1
-                const float wgt = __fdividef(w, q * q);
-                acc[j][l].x = fmaf(e.x, wgt, acc[j][l].x);
-                acc[j][l].y = fmaf(e.y, wgt, acc[j][l].y);
-                acc[j][l].z = fmaf(e.z, wgt, acc[j][l].z);
-                acc[j][l].w += wgt;
-            }
+        for (int l = 0; l < kL; ++l) {
+            const float rho = (float)(l + 1) / (float)(kLevels - 1);
+            const float2 q = fma2(nh2, both(rho * rho * rho * rho), x2);   // (n.h)^2 (a2 - 1) + 1
+            const float2 qq = mul2(q, q);
+            const float2 wgt = mul2(w, make_float2(reciprocal(qq.x), reciprocal(qq.y)));
+            add_weighted(acc[l], t, wgt, cs, finite);
+            acc[l][3] = add2(acc[l][3], wgt);
         }
     });
 #pragma unroll
-    for (int j = 0; j < kMapTexels; ++j)
-#pragma unroll
-        for (int l = 0; l < kL; ++l)
-            part[((int64_t)blockIdx.y * kL + l) * (kPrefH * kPrefW) + id[j]] = acc[j][l];
+    for (int l = 0; l < kL; ++l) {
+        float4* out = part + ((int64_t)blockIdx.y * kL + l) * (kPrefH * kPrefW);
+        out[id[0]] = make_float4(acc[l][0].x, acc[l][1].x, acc[l][2].x, acc[l][3].x);
+        out[id[1]] = make_float4(acc[l][0].y, acc[l][1].y, acc[l][2].y, acc[l][3].y);
+    }
 }
 
 // The slices' partial sums in order: irradiance texels, then prefilter texels
 // of every level.
-__global__ void k_map_sums(const float4* __restrict__ irr_part, const float4* __restrict__ pref_part, int slices,
-                           float* __restrict__ irr, float* __restrict__ pref) {
+__global__ void k_map_sums(const float4* __restrict__ irr_part, const float4* __restrict__ pref_part, int irr_slices,
+                           int pref_slices, float* __restrict__ irr, float* __restrict__ pref) {
     constexpr int kI = kIrrH * kIrrW, kP = (kLevels - 1) * kPrefH * kPrefW;
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= kI + kP) return;
     const bool is_irr = i < kI;
     const float4* p = is_irr ? irr_part + i : pref_part + (i - kI);
     float4 s = make_float4(0.f, 0.f, 0.f, 0.f);
-    for (int k = 0; k < slices; ++k) {
+    for (int k = 0; k < (is_irr ? irr_slices : pref_slices); ++k) {
         const float4 v = p[(int64_t)k * (is_irr ? kI : kP)];
         s.x += v.x;
         s.y += v.y;
@@ -639,13 +717,14 @@ irgs_status build_envmap_impl(const float* env, int32_t H, int32_t W, cudaStream
     cudaError_t e = cudaMalloc(&m->base, bytes);
     // the slices' partial sums
     const int64_t texels = (int64_t)H * W;
-    const int64_t want = (texels + kMapSlice - 1) / kMapSlice;
-    const int slices = (int)(want < kMapMaxSlices ? want : kMapMaxSlices);
+    const int64_t want = ((texels + kMapSlice - 1) / kMapSlice) | 1;
+    const int irr_slices = (int)(want < kIrrSlices ? want : kIrrSlices);
+    const int pref_slices = (int)(want < kPrefSlices ? want : kPrefSlices);
     constexpr int kIrr = kIrrH * kIrrW, kPref = kPrefH * kPrefW;
     float4* part = nullptr;
     if (e == cudaSuccess)
         e = scratch_alloc(reinterpret_cast<void**>(&part),
-                          sizeof(float4) * (size_t)slices * (kIrr + (kLevels - 1) * kPref), st);
+                          sizeof(float4) * ((size_t)irr_slices * kIrr + (size_t)pref_slices * (kLevels - 1) * kPref), st);
     if (e != cudaSuccess) {
         free_envmap(m);
         cudaGetLastError();
@@ -660,13 +739,13 @@ irgs_status build_envmap_impl(const float* env, int32_t H, int32_t W, cudaStream
     m->col_cdf = reinterpret_cast<double*>(base + at[5]);
     auto A = [&](cudaError_t r) { if (e == cudaSuccess) e = r; };
     A(cudaMemcpyAsync(m->env, env, sizeof(float) * (size_t)H * W * 3, cudaMemcpyDeviceToDevice, st));
-    float4* pref_part = part + (size_t)slices * kIrr;
+    float4* pref_part = part + (size_t)irr_slices * kIrr;
     constexpr int kPer = kMapThreads * kMapTexels;
     static_assert(kIrr % kPer == 0 && kPref % kPer == 0 && kIrrW % 8 == 0 && kIrrH % (4 * kMapTexels) == 0 &&
                       kPrefH % (4 * kMapTexels) == 0, "whole tiles of patches");
-    k_irradiance<<<dim3(kIrr / kPer, slices), kMapThreads, 0, st>>>(m->env, H, W, slices, part);
-    k_prefilter<<<dim3(kPref / kPer, slices), kMapThreads, 0, st>>>(m->env, H, W, slices, pref_part);
-    k_map_sums<<<(kIrr + (kLevels - 1) * kPref + 255) / 256, 256, 0, st>>>(part, pref_part, slices, m->irr, m->pref);
+    k_irradiance<<<dim3(kIrr / kPer, irr_slices), kMapThreads, 0, st>>>(m->env, H, W, part);
+    k_prefilter<<<dim3(kPref / kPer, pref_slices), kMapThreads, 0, st>>>(m->env, H, W, pref_part);
+    k_map_sums<<<(kIrr + (kLevels - 1) * kPref + 255) / 256, 256, 0, st>>>(part, pref_part, irr_slices, pref_slices, m->irr, m->pref);
     k_brdf_table<<<(kLutN * kLutN * 32 + 255) / 256, 256, 0, st>>>(m->lut);
     k_env_col_cdf<<<(unsigned)(((int64_t)H * 32 + 127) / 128), 128, 0, st>>>(m->env, H, W, m->col_cdf);
     k_env_row_cdf<<<1, 32, 0, st>>>(m->col_cdf, H, W, m->row_cdf);
