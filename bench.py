@@ -65,19 +65,15 @@ def measured_peaks():
 
 
 # DRAM traffic per launch of the dominant kernel, from one ncu capture
-# (dram__bytes_read.sum + dram__bytes_write.sum) scaled per ray; keyed by
-# the hash of the sources it was measured on, the hierarchy's builder
-# included (null once they change).
-# Captured on the 10-camera case (6.4M rays; the ~90 MB scene read is ~3% of
-# it, so the per-ray figure slightly overstates a 64M-ray launch).
-# (Both captures predate only the move of the launchers' host-side scratch
-# allocation to the library's own pool; the kernels' code is unchanged.)
+# (dram__bytes_read.sum + dram__bytes_write.sum) of two cameras' rays (1.28M;
+# the scene read is part of it, so the per-ray figure overstates larger
+# batches) scaled per ray; keyed by the hash of the sources it was measured
+# on, the hierarchy's builder included (null once they change).
 TRAFFIC = {
-    # the four round launches of one forward (6.4M-ray capture): read 425.7 + 924.0 + 359.6 + 87.4 MB,
-    # written 755.7 + 564.5 + 127.5 + 12.6 MB
-    "k_trace_round<16,10,*>": {"bytes_per_ray": (1796.7e6 + 1460.3e6) / 6.4e6, "src_hash": "58027c8418dc"},
-    # the listed backward and the replay of long lists (same case): read 1916.0 + 25.6 MB, written 157.0 MB
-    "k_trace_backward<16,10>": {"bytes_per_ray": (1941.6e6 + 157.0e6) / 6.4e6, "src_hash": "3c7bc3505c68"},
+    # the two rounds of one forward with hit lists: read 232.5, written 170.3 MB
+    "k_trace_round<10,*>": {"bytes_per_ray": 402.8e6 / 1.28e6, "src_hash": "fde6cd71804c"},
+    # the listed backward and the replays of long lists: read 385.7, written 28.3 MB
+    "k_trace_backward<10>": {"bytes_per_ray": 414.0e6 / 1.28e6, "src_hash": "d536dc799342"},
 }
 
 
@@ -419,15 +415,15 @@ def run_ours(args):
     # ---- roofline of the dominant kernel (by time)
     nh = out["n_hits"]
     if bwd_ms >= fwd_ms:
-        kname, kms = "k_trace_backward<16,10>", bwd_ms
+        kname, kms = "k_trace_backward<10>", bwd_ms
         flops = algorithmic_flops(nh, 16, sc.n, F, backward=True, saved_hits=args.saved_hits)
-        src = ["trace.cuh", "trace_bwd.cuh", "trace_bwd.cu", "common.cuh", "scene.cu"]
+        src = ["trace.cuh", "trace_warp.cuh", "trace_bwd.cuh", "trace_bwd.cu", "common.cuh", "scene.cu"]
     else:
         # the forward pass: for batches of 2^20 rays or more its compacted
         # k-buffer rounds and the compaction between them
-        kname, kms = "k_trace_round<16,10,*>", fwd_ms
+        kname, kms = "k_trace_round<10,*>", fwd_ms
         flops = algorithmic_flops(nh, 16, sc.n, F)
-        src = ["trace.cuh", "trace_fwd.cu", "common.cuh", "scene.cu"]
+        src = ["trace.cuh", "trace_warp.cuh", "trace_fwd.cu", "common.cuh", "scene.cu"]
     achieved = flops / (kms * 1e-3) / 1e12
     khash = _kernel_hash(src)
     tr = TRAFFIC.get(kname)

@@ -81,14 +81,16 @@ typedef struct {
 } irgs_trace_params;
 
 /* Traversal policy (results are identical either way, only speed differs).
- * Default for irgs_trace_forward / irgs_trace_backward: warp-coherent -- the
- * 32 rays of a warp walk one shared stack, best for coherent batches such as
- * camera rays in image order. Default for irgs_shade_mc / _backward: the
- * secondary rays of all points are regrouped by direction and origin and
- * traced with one stack per ray. IRGS_FLAG_PER_THREAD forces an independent
+ * Default for irgs_trace_forward / irgs_trace_backward: up to 2^18 rays, a
+ * warp per ray; larger batches as packets -- the 32 rays of a warp walk the
+ * hierarchy together where they run together (pixel rows are cut into tiles
+ * first), else each its own way. Default for irgs_shade_mc / _backward: the
+ * secondary rays of all points are regrouped by direction and origin (above
+ * 2^19 rays) and traced with a warp per ray, above 2^23 rays with a lane per
+ * ray. IRGS_FLAG_PER_THREAD forces an independent
  * stack per ray (for shading: the fused kernel, a warp per point tracing its
- * own samples); IRGS_FLAG_WARP forces the warp-coherent walk (for shading:
- * the fused kernel with a warp-shared stack). Setting both is invalid. */
+ * own samples); IRGS_FLAG_WARP forces packets (for shading: the fused kernel
+ * with packets). Setting both is invalid. */
 #define IRGS_FLAG_PER_THREAD 1u
 #define IRGS_FLAG_WARP 2u
 /* Shading only (irgs_shade_mc / irgs_shade_mc_backward): the stratified
@@ -231,13 +233,14 @@ irgs_status irgs_scene_export_wide(irgs_scene scene, float* nodes, int64_t cap, 
  *                   followed by -1 if n_hits < max_hit_ids; later entries
  *                   are not written. NULL to skip. irgs_trace_backward can
  *                   take this list instead of replaying the traversal.
- * Outputs are overwritten. n_rays may be 0. With the warp-coherent walk,
- * k = 16 and at least 2^20 rays, rays still marching after each of the
- * first three k-buffer rounds are regrouped into full warps; that takes
- * 56 to 104 bytes per ray of scratch (72 at 4..10 channels), allocated and
- * freed stream-ordered (the library's scratch pool) on `stream`; if that allocation
- * fails the rays are marched without regrouping. Results are the same
- * either way.
+ * Outputs are overwritten. n_rays may be 0. With packets and at least 2^20
+ * rays, rays still marching after the first k-buffer round (32 entries,
+ * whatever k) are regrouped into full warps; that takes 56 to 104 bytes per
+ * ray of scratch (72 at 4..10 channels), allocated and freed stream-ordered
+ * (the library's scratch pool) on `stream`; if that allocation fails the
+ * rays are marched without regrouping. Packets also take one word of that
+ * scratch to look for pixel rows, and do without if there is none. Results
+ * are the same either way.
  */
 irgs_status irgs_trace_forward(irgs_scene scene, const float* ray_o, const float* ray_d,
                                int64_t n_rays, const irgs_trace_params* params,
@@ -421,9 +424,8 @@ irgs_status irgs_envmap_export(irgs_envmap envmap, float* irr, float* pref, floa
  * Pref linear between its two nearest roughness levels, all maps bilinear.
  * out_rgb [P,3]; out_vis [P] and out_ind [P,3] (means of V and of the
  * indirect term over all samples) may be NULL. By default the samples of
- * all points are regrouped by direction and origin and traced with one
- * stack per ray (scratch from the stream-ordered allocator, ~64 bytes per
- * sample in chunks of at most 2^26); IRGS_FLAG_PER_THREAD selects the fused
+ * all points are regrouped and traced as irgs_shade_mc's (scratch from the
+ * stream-ordered allocator, ~64 bytes per sample in chunks of at most 2^26); IRGS_FLAG_PER_THREAD selects the fused
  * kernel (a warp per point tracing its own samples). Both give the same
  * traces.
  */

@@ -5,8 +5,9 @@
 // reset, kernel) can be captured once into a CUDA graph and replayed with new
 // table contents. A unit of work is one block's 128 rays of a tile, so a step
 // of a few tiles still fills the GPU (a whole tile per block left a step of
-// 36 tiles on 36 of 152 SMs: two such steps took 46.5 ms of a burst's 64). The shading tiles of the step then run, one request's range
-// of G-buffer points at a time, through the wavefront shading path (secondary
+// 36 tiles on 36 of 152 SMs: two such steps took 46.5 ms of a burst's 64). The
+// shading tiles of the step then run, one request's range of G-buffer points
+// at a time, through the wavefront shading path (secondary
 // rays regrouped by direction and origin, traced in that order, estimated
 // per point), keyed by pixel index, so a pixel's estimate is the one
 // irgs_shade_mc gives for it.

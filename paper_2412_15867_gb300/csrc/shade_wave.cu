@@ -7,10 +7,9 @@
 // 30-bit key -- a 6-bit octahedral bin of the direction above the 24-bit
 // Morton code of the origin -- with a stable radix sort, and traced in that
 // order, so the rays of a warp leave neighbouring points in similar
-// directions and walk similar paths. Each lane keeps its own stack: these
-// rays are still too spread for one warp-wide walk (a shared stack visited
-// 8x the nodes), but their independent walks now diverge little (1.8x the
-// throughput of unsorted rays on the 1M-surfel scene). The per-point estimate then reads the stored
+// directions and walk similar paths. These rays are still too spread for
+// packets: each walks its own way, with a warp's 32 lanes working on it or,
+// in the largest batches, a lane. The per-point estimate then reads the stored
 // traces (L_ind, V) and applies the same per-sample arithmetic as the fused
 // kernel (shade_point_warp), with the same fixed reduction order.
 //
@@ -46,7 +45,7 @@ constexpr int kWaveSavedHits = 64;   // 12% of secondary rays blend more than 32
 constexpr int64_t kWaveUnsortedMax = int64_t(1) << 19;
 // Batches up to this size take a warp per ray, whose throughput does not depend
 // on the size; a ray per lane catches up only where the pools are refilled many
-// times: 120.5 ms against 114.5 at 41M rays, 24.7 against 27.5 at 6.4M
+// times: 120.5 ms against 105.8 at 41M rays, 24.7 against 27.5 at 6.4M
 // (relighting, the same walk).
 constexpr int64_t kWaveWarpMax = int64_t(1) << 23;
 constexpr int kWaveReplayBlocks = 152 * 4;   // blocks that share the few rays whose hit list did not fit
