@@ -322,18 +322,21 @@ __global__ void k_brdf_table(float* __restrict__ lut) {
 }
 
 // Importance-sampling tables, FP64: one warp per row for the column cdfs,
-// then one warp for the row cdf, each by a scan of 32 terms at a time onto
-// the running sum (a fixed order of additions).
-__device__ __forceinline__ double warp_scan(double v, double& run) {
+// then one warp for the row cdf, as running sums in order: each entry is the
+// one before it plus a term >= 0, rounded, so the tables never decrease and a
+// black texel has no width at all (sums associated otherwise differ in the
+// last bit there, and a sample that lands on such a bit of width has a pdf of
+// 1e-16). The lanes make 32 terms at a time; all of them carry the sum.
+// Bound by the chain of FP64 additions.
+__device__ __forceinline__ double warp_running_sum(double v, double& run) {
     const int lane = threadIdx.x & 31;
+    double mine = 0.0;
 #pragma unroll
-    for (int off = 1; off < 32; off <<= 1) {
-        const double y = __shfl_up_sync(0xffffffffu, v, off);
-        if (lane >= off) v = __dadd_rn(v, y);
+    for (int i = 0; i < 32; ++i) {
+        run = __dadd_rn(run, __shfl_sync(0xffffffffu, v, i));
+        if (lane == i) mine = run;
     }
-    v = __dadd_rn(run, v);
-    run = __shfl_sync(0xffffffffu, v, 31);
-    return v;
+    return mine;
 }
 
 __global__ void k_env_col_cdf(const float* __restrict__ env, int H, int W, double* __restrict__ col_cdf) {
@@ -352,7 +355,7 @@ __global__ void k_env_col_cdf(const float* __restrict__ env, int H, int W, doubl
                                          __dmul_rn(0.0722, (double)e[2]));
             v = __dmul_rn(lum, s);
         }
-        v = warp_scan(v, run);
+        v = warp_running_sum(v, run);
         if (c < W) cc[c + 1] = v;
     }
 }
@@ -362,7 +365,7 @@ __global__ void k_env_row_cdf(const double* __restrict__ col_cdf, int H, int W, 
     if (threadIdx.x == 0) row_cdf[0] = 0.0;
     for (int r0 = 0; r0 < H; r0 += 32) {
         const int r = r0 + threadIdx.x;
-        const double v = warp_scan(r < H ? col_cdf[(int64_t)r * (W + 1) + W] : 0.0, run);
+        const double v = warp_running_sum(r < H ? col_cdf[(int64_t)r * (W + 1) + W] : 0.0, run);
         if (r < H) row_cdf[r + 1] = v;
     }
 }
