@@ -169,19 +169,26 @@ __global__ void __launch_bounds__(256) k_bounds(const float* __restrict__ means,
 
 // Sorts with passes > 0 (then even: the result ends in keys / vals); with
 // passes = 0 only the codes are made. A block owns a contiguous piece of the
-// keys; every block sums the digit counts of the pieces before its own.
+// keys; every block sums the digit counts of the pieces before its own. A
+// barrier that gives up leaves an error bit and its flag, by which k_pack
+// knows that the order is not there.
 __global__ void __launch_bounds__(kCoopThreads, 1) k_order(
     const float* __restrict__ means, const float* __restrict__ quats, const float* __restrict__ scales,
     const float* __restrict__ opac, int64_t n, uint32_t* ctl, uint32_t* keys, int32_t* vals, uint32_t* keys_tmp,
-    int32_t* vals_tmp, uint32_t* hist, int passes) {
+    int32_t* vals_tmp, uint32_t* hist, int passes, uint32_t* status) {
     __shared__ uint32_t s_base[256], s_cnt[256];
     __shared__ uint32_t s_part[2][4][256];
     __shared__ uint16_t s_warp_cnt[kCoopThreads / 32][256];
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     uint32_t target = 0u;
     const uint32_t* bounds = ctl;
+    auto meet = [&]() {
+        const bool ok = grid_barrier(ctl + kCtlOrder, target);
+        if (!ok && tid == 0) atomicOr(status, kErrBadTree);
+        return ok;
+    };
     centre_bounds(means, quats, scales, opac, n, ctl);
-    if (!grid_barrier(ctl + kCtlOrder, target)) return;
+    if (!meet()) return;
     const int64_t piece = (n + gridDim.x - 1) / gridDim.x;
     const int64_t begin = blockIdx.x * piece, end = begin + piece < n ? begin + piece : n;
     {
@@ -215,7 +222,7 @@ __global__ void __launch_bounds__(kCoopThreads, 1) k_order(
         for (int64_t i = begin + tid; i < end; i += kCoopThreads) atomicAdd(&s_cnt[(__ldcg(kin + i) >> shift) & 255u], 1u);
         __syncthreads();
         if (tid < 256) hist[blockIdx.x * 256 + tid] = s_cnt[tid];
-        if (!grid_barrier(ctl + kCtlOrder, target)) return;
+        if (!meet()) return;
         // where this piece's keys of each digit go: all smaller digits, then the pieces before this one
         {
             const int d = tid & 255, quarter = tid >> 8;
@@ -282,7 +289,7 @@ __global__ void __launch_bounds__(kCoopThreads, 1) k_order(
             __syncthreads();
             if (tid < 256) s_base[tid] += total;
         }
-        if (!grid_barrier(ctl + kCtlOrder, target)) return;
+        if (!meet()) return;
     }
 }
 
@@ -294,7 +301,11 @@ __global__ void __launch_bounds__(kCoopThreads, 1) k_order(
 // per surfel, 149 us for 300k surfels against 35), the logarithm of the support
 // radius only where it is not capped, and the box extents' roots in FP32,
 // whose error the boxes' padding of 1e-5 covers a hundred times.
-__global__ void __launch_bounds__(256) k_pack(const int32_t* __restrict__ perm, const float* __restrict__ means,
+// With `no_order` set and nonzero, perm and keys hold no order: the surfels
+// then keep the user's, with equal keys, from which every later step builds a
+// valid (if poor) hierarchy.
+__global__ void __launch_bounds__(256) k_pack(int32_t* __restrict__ perm, uint32_t* __restrict__ keys,
+                                              const uint32_t* __restrict__ no_order, const float* __restrict__ means,
                                               const float* __restrict__ quats, const float* __restrict__ scales,
                                               const float* __restrict__ opac, int64_t n, double alpha_min,
                                               float4* __restrict__ rec, float* __restrict__ leaf_box,
@@ -302,6 +313,10 @@ __global__ void __launch_bounds__(256) k_pack(const int32_t* __restrict__ perm, 
                                               int32_t* __restrict__ inv_perm) {
     const int64_t j = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     if (j >= n) return;
+    if (no_order != nullptr && *no_order != 0u) {
+        perm[j] = (int32_t)j;
+        keys[j] = 0u;
+    }
     const int32_t i = perm[j];
     if (inv_perm != nullptr) inv_perm[i] = (int32_t)j;
     const float muf[3] = {means[3 * (int64_t)i], means[3 * (int64_t)i + 1], means[3 * (int64_t)i + 2]};
@@ -755,7 +770,10 @@ __global__ void __launch_bounds__(kCoopThreads, 1) k_ploc(PlocArgs A) {
         A.hi[0][i] = make_float4(b[3], b[4], b[5], 0.f);
     }
     if (!grid_barrier(A.ctl + kCtlPloc, target)) {
-        if (tid == 0) atomicOr(A.status, kErrBadTree);
+        if (tid == 0) {
+            atomicOr(A.status, kErrBadTree);
+            A.ctl[kCtlFallback] = 1u;
+        }
         return;
     }
     int64_t count = n, made = 0;
@@ -980,6 +998,31 @@ __device__ __forceinline__ float box_area(const float b[6]) {
     return dx * dy + dy * dz + dz * dx;
 }
 
+// Wide root of a one-surfel (or empty) scene.
+__device__ __forceinline__ void write_tiny_root(int64_t n, const float* __restrict__ leaf_box, WideNode* wide,
+                                                float4* child_box) {
+    WideNode o;
+    const float e = INFINITY;   // empty slots: lo = +inf, hi = -inf
+    float b[6] = {e, e, e, -e, -e, -e};
+    if (n == 1)
+        for (int k = 0; k < 6; ++k) b[k] = leaf_box[k];
+    o.lox = make_float4(b[0], e, e, e);
+    o.loy = make_float4(b[1], e, e, e);
+    o.loz = make_float4(b[2], e, e, e);
+    o.hix = make_float4(b[3], -e, -e, -e);
+    o.hiy = make_float4(b[4], -e, -e, -e);
+    o.hiz = make_float4(b[5], -e, -e, -e);
+    o.child = make_int4(n == 1 ? ~0 : kNoChild, kNoChild, kNoChild, kNoChild);
+    o.pad = make_int4(n == 1 ? 1 : 0, 0, 0, 0);
+    wide[0] = o;
+    child_box[0] = make_float4(b[0], b[1], b[2], __int_as_float(o.child.x));
+    child_box[1] = make_float4(b[3], b[4], b[5], 0.f);
+    for (int k = 1; k < 4; ++k) {
+        child_box[2 * k] = make_float4(e, e, e, __int_as_float(kNoChild));
+        child_box[2 * k + 1] = make_float4(-e, -e, -e, 0.f);
+    }
+}
+
 __global__ void __launch_bounds__(kCoopThreads, 1) k_wide(const Node* __restrict__ nodes, int32_t* source,
                                                           uint32_t* counters, uint32_t* ctl, int64_t max_wide,
                                                           WideNode* __restrict__ wide,
@@ -1081,7 +1124,14 @@ __global__ void __launch_bounds__(kCoopThreads, 1) k_wide(const Node* __restrict
             }
         }
         if (!grid_barrier(ctl + kCtlWide, target)) {
-            if (threadIdx.x == 0) atomicOr(status, kErrBadTree);
+            // the levels below were not made: nothing may be walked into (thread 0 of block 0 alone writes the root)
+            if (threadIdx.x == 0) {
+                atomicOr(status, kErrBadTree);
+                if (blockIdx.x == 0) {
+                    write_tiny_root(0, nullptr, wide, child_box);
+                    counters[kWideLevels] = 1u;
+                }
+            }
             return;
         }
         begin = end;
@@ -1091,28 +1141,8 @@ __global__ void __launch_bounds__(kCoopThreads, 1) k_wide(const Node* __restrict
     if (blockIdx.x == 0 && threadIdx.x == 0) counters[kWideLevels] = end;
 }
 
-// Wide root of a one-surfel (or empty) scene.
 __global__ void k_wide_tiny(int64_t n, const float* __restrict__ leaf_box, WideNode* wide, float4* child_box) {
-    WideNode o;
-    const float e = INFINITY;   // empty slots: lo = +inf, hi = -inf
-    float b[6] = {e, e, e, -e, -e, -e};
-    if (n == 1)
-        for (int k = 0; k < 6; ++k) b[k] = leaf_box[k];
-    o.lox = make_float4(b[0], e, e, e);
-    o.loy = make_float4(b[1], e, e, e);
-    o.loz = make_float4(b[2], e, e, e);
-    o.hix = make_float4(b[3], -e, -e, -e);
-    o.hiy = make_float4(b[4], -e, -e, -e);
-    o.hiz = make_float4(b[5], -e, -e, -e);
-    o.child = make_int4(n == 1 ? ~0 : kNoChild, kNoChild, kNoChild, kNoChild);
-    o.pad = make_int4(n == 1 ? 1 : 0, 0, 0, 0);
-    wide[0] = o;
-    child_box[0] = make_float4(b[0], b[1], b[2], __int_as_float(o.child.x));
-    child_box[1] = make_float4(b[3], b[4], b[5], 0.f);
-    for (int k = 1; k < 4; ++k) {
-        child_box[2 * k] = make_float4(e, e, e, __int_as_float(kNoChild));
-        child_box[2 * k + 1] = make_float4(-e, -e, -e, 0.f);
-    }
+    write_tiny_root(n, leaf_box, wide, child_box);
 }
 
 template <class T>
@@ -1220,9 +1250,9 @@ static cudaError_t enqueue_order(irgs_scene sc, const irgs_surfels* s, cudaStrea
     // beyond a few keys per thread the launches of sort_pairs cost less than a piece's serial steps
     const int passes = n <= kOrderMaxKeys ? 4 : 0;
     cudaError_t e = launch_coop<const float*, const float*, const float*, const float*, int64_t, uint32_t*, uint32_t*,
-                                int32_t*, uint32_t*, int32_t*, uint32_t*, int>(
+                                int32_t*, uint32_t*, int32_t*, uint32_t*, int, uint32_t*>(
         k_order, sc->device, n, st, s->means, s->quats, s->scales, s->opacity, n, sc->bounds, sc->keys, sc->perm,
-        sc->keys_tmp, sc->vals_tmp, sc->hist, passes);
+        sc->keys_tmp, sc->vals_tmp, sc->hist, passes, sc->status);
     if (e == cudaSuccess && passes == 0)
         e = sort_pairs(sc->keys, sc->perm, sc->keys_tmp, sc->vals_tmp, sc->hist, n, st);
     return e;
@@ -1233,7 +1263,8 @@ static cudaError_t enqueue_pack(irgs_scene sc, const irgs_surfels* s, cudaStream
     const int64_t n = sc->n;
     const int32_t F = sc->F;
     const int T = 256;
-    k_pack<<<blocks_for(n, T), T, 0, st>>>(sc->perm, s->means, s->quats, s->scales, s->opacity, n,
+    // (a refit keeps the last build's order and finds the flag zero)
+    k_pack<<<blocks_for(n, T), T, 0, st>>>(sc->perm, sc->keys, sc->bounds + kCtlOrder + 1, s->means, s->quats, s->scales, s->opacity, n,
                                            (double)sc->alpha_min, sc->rec, sc->leaf_box, sc->q_raw, sc->scale,
                                            sc->inv_perm);
     if (F > 0) k_gather_feat<<<blocks_for(n * F, T), T, 0, st>>>(sc->perm, n, F, s->features, sc->feat);
