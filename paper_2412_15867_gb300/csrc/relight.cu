@@ -40,11 +40,13 @@ constexpr int kLutN = IRGS_RELIGHT_LUT_N;
 constexpr int kLutSamples = 1024;
 constexpr int kRelightThreads = kTraceThreads;
 
-// Centre direction of texel (row, col) of an h x w equirect map.
+// Centre direction of texel (row, col) of an h x w equirect map. The azimuth over
+// pi is one quotient of whole numbers in (-1, 1): the texel's weight at the peak
+// of prefilter level 1 changes by 25 to 50 times the angle's error.
 __device__ __forceinline__ f3 texel_dir(int h, int w, int row, int col) {
     float st, ct, sp, cp;
     sincospif(((float)row + 0.5f) / (float)h, &st, &ct);
-    sincospif(((float)col + 0.5f) * 2.f / (float)w - 1.f, &sp, &cp);
+    sincospif((float)(2 * col + 1 - w) / (float)w, &sp, &cp);
     return mk3(st * cp, st * sp, ct);
 }
 
@@ -70,11 +72,22 @@ __device__ __forceinline__ float texel_solid_angle(int H, int W, int row) {
 // all of the sphere (contiguous ones face some tiles wholly and others not at
 // all); an odd number of slices walks through the columns of maps of 2^k
 // columns. An environment of 512 x 256 and the relighting of 4,096 points under
-// it take 2.98 ms (3.50 without pairs; 27 prefilter slices, as many blocks as
-// fit at once, 3.18; 127 slices 2.95, for twice the memory).
+// it took 2.98 ms (3.50 without pairs; 27 prefilter slices, as many blocks as
+// fit at once, 3.18; 127 slices 2.95, for twice the memory) before the groups below.
+//
+// Sums are made in three steps: kMapGroup texels in one accumulator, the groups
+// of a slice in another, the slices with their rounding errors carried along.
+// The errors of groups and of slices are independent, so what they leave of the
+// total falls with the square root of their number: 4e-8 rms relative at
+// 512 x 256 texels and 7e-8 at 2048 x 1024 (level 1: 7e-8 and 9e-8). A block-wide
+// tree per output left 9e-8 and 2e-7 (1.4e-7 and 1.7e-6), one accumulator per
+// slice 2e-7 and 1.2e-6 (3.5e-7 and 1e-5). The groups cost 5% of an
+// environment's time (512 x 256: 1.74 -> 1.87 ms; groups of 16 1.93, of 64
+// 1.84, but 1.2e-7 at 32 x 16 texels, where the tree had 1e-7).
 constexpr int kMapThreads = 128;
 constexpr int kMapTexels = 2;      // output texels per thread
-constexpr int kMapSlice = 512;     // least environment texels per slice
+constexpr int kMapGroup = 32;      // environment texels per accumulator
+constexpr int kMapSlice = 128;     // least environment texels per slice
 constexpr int kPrefSlices = 63;    // x 32 tiles
 constexpr int kIrrSlices = 217;    // x 8 tiles
 
@@ -121,12 +134,12 @@ struct MapTexel {
 };
 
 // The texels of slice blockIdx.y: fn(texel, whether the radiance of its chunk
-// is finite) for each. The second is a type: asked per texel and level it took
-// a quarter of the kernel's time.
+// is finite) for each, group() after every kMapGroup of them. The second is a
+// type: asked per texel and level it took a quarter of the kernel's time.
 template <bool YES>
 struct Finite {};
-template <class Fn>
-__device__ __forceinline__ void for_texels(const float* __restrict__ env, int H, int W, Fn fn) {
+template <class Fn, class Group>
+__device__ __forceinline__ void for_texels(const float* __restrict__ env, int H, int W, Fn fn, Group group) {
     __shared__ MapTexel s_tex[kMapThreads];
     const int64_t all = (int64_t)H * W;
     for (int64_t t0 = (int64_t)blockIdx.y * kMapThreads; t0 < all; t0 += (int64_t)gridDim.y * kMapThreads) {
@@ -149,10 +162,14 @@ __device__ __forceinline__ void for_texels(const float* __restrict__ env, int H,
         }
         finite = __syncthreads_and(finite);
         const int n = (int)(all - t0 < kMapThreads ? all - t0 : kMapThreads);
-        if (finite)
-            for (int i = 0; i < n; ++i) fn(s_tex[i], Finite<true>());
-        else
-            for (int i = 0; i < n; ++i) fn(s_tex[i], Finite<false>());
+        for (int g = 0; g < n; g += kMapGroup) {
+            const int e = min(g + kMapGroup, n);
+            if (finite)
+                for (int i = g; i < e; ++i) fn(s_tex[i], Finite<true>());
+            else
+                for (int i = g; i < e; ++i) fn(s_tex[i], Finite<false>());
+            group();
+        }
         __syncthreads();
     }
 }
@@ -202,12 +219,25 @@ __global__ void __launch_bounds__(kMapThreads) k_irradiance(const float* __restr
                                                             float4* __restrict__ part) {
     int id[2];
     const PairDir N = pair_dir(kIrrH, kIrrW, id);
-    float2 acc[3] = {both(0.f), both(0.f), both(0.f)};
-    for_texels(env, H, W, [&](const MapTexel& t, auto finite) {
-        const float2 cs = fma2(t.dx, N.x, fma2(t.dy, N.y, mul2(t.dz, N.z)));
-        if (!(cs.x > 0.f || cs.y > 0.f)) return;
-        add_weighted(acc, t, facing(cs, t), cs, finite);
-    });
+    float2 acc[3] = {both(0.f), both(0.f), both(0.f)}, group_acc[3] = {both(0.f), both(0.f), both(0.f)};
+    bool some = false;   // has the group a texel that an output faces?
+    for_texels(
+        env, H, W,
+        [&](const MapTexel& t, auto finite) {
+            const float2 cs = fma2(t.dx, N.x, fma2(t.dy, N.y, mul2(t.dz, N.z)));
+            if (!(cs.x > 0.f || cs.y > 0.f)) return;
+            some = true;
+            add_weighted(group_acc, t, facing(cs, t), cs, finite);
+        },
+        [&]() {
+            if (!some) return;
+            some = false;
+#pragma unroll
+            for (int c = 0; c < 3; ++c) {
+                acc[c] = add2(acc[c], group_acc[c]);
+                group_acc[c] = both(0.f);
+            }
+        });
     float4* out = part + (int64_t)blockIdx.y * (kIrrH * kIrrW);
     out[id[0]] = make_float4(acc[0].x, acc[1].x, acc[2].x, 0.f);
     out[id[1]] = make_float4(acc[0].y, acc[1].y, acc[2].y, 0.f);
@@ -223,35 +253,65 @@ __global__ void __launch_bounds__(kMapThreads) k_prefilter(const float* __restri
     constexpr int kL = kLevels - 1;
     int id[2];
     const PairDir R = pair_dir(kPrefH, kPrefW, id);
-    float2 acc[kL][4];
+    // the slice's sums lie in shared memory: in registers they would take half of the blocks
+    __shared__ float2 s_acc[kL][4][kMapThreads];
+    float2 group_acc[kL][4];
 #pragma unroll
     for (int l = 0; l < kL; ++l)
 #pragma unroll
-        for (int c = 0; c < 4; ++c) acc[l][c] = both(0.f);
-    for_texels(env, H, W, [&](const MapTexel& t, auto finite) {
-        const float2 cs = fma2(t.dx, R.x, fma2(t.dy, R.y, mul2(t.dz, R.z)));
-        if (!(cs.x > 0.f || cs.y > 0.f)) return;
-        const float2 w = facing(cs, t);
-        const float2 gx = fma2(R.x, both(-1.f), t.dx), gy = fma2(R.y, both(-1.f), t.dy), gz = fma2(R.z, both(-1.f), t.dz);
-        const float2 x2 = mul2(both(0.25f), fma2(gx, gx, fma2(gy, gy, mul2(gz, gz))));
-        const float2 nh2 = fma2(x2, both(-1.f), both(1.f));
+        for (int c = 0; c < 4; ++c) s_acc[l][c][threadIdx.x] = group_acc[l][c] = both(0.f);
+    bool some = false;
+    for_texels(
+        env, H, W,
+        [&](const MapTexel& t, auto finite) {
+            const float2 cs = fma2(t.dx, R.x, fma2(t.dy, R.y, mul2(t.dz, R.z)));
+            if (!(cs.x > 0.f || cs.y > 0.f)) return;
+            some = true;
+            const float2 w = facing(cs, t);
+            const float2 gx = fma2(R.x, both(-1.f), t.dx), gy = fma2(R.y, both(-1.f), t.dy), gz = fma2(R.z, both(-1.f), t.dz);
+            const float2 x2 = mul2(both(0.25f), fma2(gx, gx, fma2(gy, gy, mul2(gz, gz))));
+            const float2 nh2 = fma2(x2, both(-1.f), both(1.f));
 #pragma unroll
-        for (int l = 0; l < kL; ++l) {
-            const float rho = (float)(l + 1) / (float)(kLevels - 1);
-            const float2 q = fma2(nh2, both(rho * rho * rho * rho), x2);   // (n.h)^2 (a2 - 1) + 1
-            const float2 qq = mul2(q, q);
-            const float2 wgt = mul2(w, make_float2(reciprocal(qq.x), reciprocal(qq.y)));
-            add_weighted(acc[l], t, wgt, cs, finite);
-            acc[l][3] = add2(acc[l][3], wgt);
-        }
-    });
+            for (int l = 0; l < kL; ++l) {
+                const float rho = (float)(l + 1) / (float)(kLevels - 1);
+                const float2 q = fma2(nh2, both(rho * rho * rho * rho), x2);   // (n.h)^2 (a2 - 1) + 1
+                const float2 qq = mul2(q, q);
+                const float2 wgt = mul2(w, make_float2(reciprocal(qq.x), reciprocal(qq.y)));
+                add_weighted(group_acc[l], t, wgt, cs, finite);
+                group_acc[l][3] = add2(group_acc[l][3], wgt);
+            }
+        },
+        [&]() {
+            if (!some) return;
+            some = false;
+#pragma unroll
+            for (int l = 0; l < kL; ++l)
+#pragma unroll
+                for (int c = 0; c < 4; ++c) {
+                    s_acc[l][c][threadIdx.x] = add2(s_acc[l][c][threadIdx.x], group_acc[l][c]);
+                    group_acc[l][c] = both(0.f);
+                }
+        });
 #pragma unroll
     for (int l = 0; l < kL; ++l) {
         float4* out = part + ((int64_t)blockIdx.y * kL + l) * (kPrefH * kPrefW);
-        out[id[0]] = make_float4(acc[l][0].x, acc[l][1].x, acc[l][2].x, acc[l][3].x);
-        out[id[1]] = make_float4(acc[l][0].y, acc[l][1].y, acc[l][2].y, acc[l][3].y);
+        float2 acc[4];
+#pragma unroll
+        for (int c = 0; c < 4; ++c) acc[c] = s_acc[l][c][threadIdx.x];
+        out[id[0]] = make_float4(acc[0].x, acc[1].x, acc[2].x, acc[3].x);
+        out[id[1]] = make_float4(acc[0].y, acc[1].y, acc[2].y, acc[3].y);
     }
 }
+
+// s += v, its rounding error into e.
+__device__ __forceinline__ void carry_sum(float& s, float& e, float v) {
+    float t, d;
+    two_sum(s, v, t, d);
+    s = t;
+    e += d;
+}
+// The sum with what it lost; as it is where it is not finite (the errors are NaN there).
+__device__ __forceinline__ float carried(float s, float e) { return fabsf(e) < INFINITY ? s + e : s; }
 
 // The slices' partial sums in order: irradiance texels, then prefilter texels
 // of every level.
@@ -262,14 +322,15 @@ __global__ void k_map_sums(const float4* __restrict__ irr_part, const float4* __
     if (i >= kI + kP) return;
     const bool is_irr = i < kI;
     const float4* p = is_irr ? irr_part + i : pref_part + (i - kI);
-    float4 s = make_float4(0.f, 0.f, 0.f, 0.f);
+    float4 s = make_float4(0.f, 0.f, 0.f, 0.f), e = s;
     for (int k = 0; k < (is_irr ? irr_slices : pref_slices); ++k) {
         const float4 v = p[(int64_t)k * (is_irr ? kI : kP)];
-        s.x += v.x;
-        s.y += v.y;
-        s.z += v.z;
-        s.w += v.w;
+        carry_sum(s.x, e.x, v.x);
+        carry_sum(s.y, e.y, v.y);
+        carry_sum(s.z, e.z, v.z);
+        carry_sum(s.w, e.w, v.w);
     }
+    s = make_float4(carried(s.x, e.x), carried(s.y, e.y), carried(s.z, e.z), carried(s.w, e.w));
     if (is_irr) {
         irr[3 * i] = s.x * (1.f / kPi);
         irr[3 * i + 1] = s.y * (1.f / kPi);
