@@ -614,8 +614,9 @@ __global__ void k_relight_gen(EnvMaps M, const float* __restrict__ xg, int64_t p
     f3 w = mk3(0.f, 0.f, 1.f);
     float pdf = 0.f;
     const bool ok = relight_dir(M, p, (int)(i % Sn), Sn, seed, w, pdf);
-    dir[i] = make_float4(w.x, w.y, w.z, ok ? pdf : 0.f);
-    key[i] = ok ? wave_key(ld3r(xg, p), w, bounds) : kInvalidWaveKey;
+    const f3 x = ld3r(xg, p);
+    dir[i] = make_float4(w.x, w.y, w.z, ok ? (can_hit(x, w) ? pdf : -pdf) : 0.f);   // < 0: a ray that meets nothing
+    key[i] = ok ? wave_key(x, w, bounds) : kInvalidWaveKey;
     val[i] = (int32_t)i;
 }
 
@@ -664,8 +665,9 @@ __global__ void __launch_bounds__(kWarpRayThreads, kWarpRayBlocks) k_relight_tra
     const int j = blockIdx.x * kWarpRays + (threadIdx.x >> 5);
     f3 o, d;
     if (j >= rays || !job.load(j, o, d)) return;
+    const Ray ray = make_ray(o, d);
     WarpMarch w;
-    const bool ok = march_warp(S, make_ray(o, d), P, w, job.ids(j), job.max_ids, warp_ray_scratch());
+    const bool ok = march_warp(S, ray, make_ray_box(ray), P, w, job.ids(j), job.max_ids, warp_ray_scratch());
     MarchState<7> st;
 #pragma unroll
     for (int c = 0; c < 7; ++c) st.C[c] = __shfl_sync(kFullWarp, w.C, c);
@@ -695,10 +697,10 @@ __global__ void __launch_bounds__(kRelightThreads) k_relight_shade(EnvMaps M, co
     for (int s = lane; s < Sn; s += 32) {
         const int64_t i = k * Sn + s;
         const float4 d4 = __ldg(dir + i);
-        if (!(d4.w > 0.f)) continue;
+        if (d4.w == 0.f) continue;
         const float4 r0 = __ldg(res + 2 * i), r1 = __ldg(res + 2 * i + 1);
         const float C[7] = {r0.x, r0.y, r0.z, r0.w, r1.x, r1.y, r1.z};
-        relight_sample(M, F, a, mk3(d4.x, d4.y, d4.z), d4.w, C, r1.w, acc);
+        relight_sample(M, F, a, mk3(d4.x, d4.y, d4.z), fabsf(d4.w), C, r1.w, acc);
     }
     relight_write(acc, lane, p, Sn, rgb, vis, ind);
 }

@@ -53,7 +53,8 @@ constexpr int kWaveReplayBlocks = 152 * 4;   // blocks that share the few rays w
 __device__ __forceinline__ f3 ld3w(const float* p, int64_t i) { return mk3(p[3 * i], p[3 * i + 1], p[3 * i + 2]); }
 
 // One thread per sample of points [p0, p0 + rays / St): direction (w = 1 if
-// the sample is valid) and its regrouping key (invalid samples sort last).
+// the sample is valid, -1 if its ray is not finite and so meets nothing) and its
+// regrouping key (invalid samples sort last).
 // Point p draws the random numbers of point number key_base + p; a point
 // whose `valid` entry (if given) is not above 0.5 traces nothing.
 __global__ void k_wave_gen(const float* __restrict__ xg, const float* __restrict__ ng, const float* __restrict__ rg,
@@ -73,8 +74,9 @@ __global__ void k_wave_gen(const float* __restrict__ xg, const float* __restrict
     }
     const ShadeFrame F = shade_frame(ld3w(ng, p), ld3w(wog, p), rg[p]);
     const ShadeSample d = draw_sample(F, mode, key_base + (uint64_t)p, s, St, nd, seed);
-    dir[i] = make_float4(d.wi.x, d.wi.y, d.wi.z, d.valid ? 1.f : 0.f);
-    key[i] = d.valid ? wave_key(ld3w(xg, p), d.wi, bounds) : kInvalidWaveKey;
+    const f3 x = ld3w(xg, p);
+    dir[i] = make_float4(d.wi.x, d.wi.y, d.wi.z, d.valid ? (can_hit(x, d.wi) ? 1.f : -1.f) : 0.f);
+    key[i] = d.valid ? wave_key(x, d.wi, bounds) : kInvalidWaveKey;
     val[i] = (int32_t)i;
 }
 
@@ -95,8 +97,8 @@ struct WaveJob {
     __device__ __forceinline__ bool load(int j, f3& o, f3& d) const {
         const int64_t i = order[j];
         const float4 d4 = dir[i];
-        if (d4.w == 0.f) {   // every sample gets an entry, so no reader sees unwritten scratch
-            res[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (!(d4.w > 0.f)) {   // every sample gets an entry, so no reader sees unwritten scratch
+            res[i] = make_float4(0.f, 0.f, 0.f, d4.w < 0.f ? 1.f : 0.f);
             if (SAVE) nh[i] = 0;
             return false;
         }
@@ -132,8 +134,9 @@ __global__ void __launch_bounds__(kWarpRayThreads, kWarpRayBlocks) k_wave_trace_
     const int j = blockIdx.x * kWarpRays + (threadIdx.x >> 5);
     f3 o, d;
     if (j >= rays || !job.load(j, o, d)) return;
+    const Ray ray = make_ray(o, d);
     WarpMarch w;
-    const bool ok = march_warp(S, make_ray(o, d), P, w, job.ids(j), job.max_ids, warp_ray_scratch());
+    const bool ok = march_warp(S, ray, make_ray_box(ray), P, w, job.ids(j), job.max_ids, warp_ray_scratch());
     MarchState<3> st;
 #pragma unroll
     for (int c = 0; c < 3; ++c) st.C[c] = __shfl_sync(kFullWarp, w.C, c);

@@ -228,13 +228,12 @@ __device__ __forceinline__ int blend_warp(const SceneView& S, const TraceParams&
     return done;
 }
 
-// All rounds of the warp's ray.
-__device__ __forceinline__ bool march_warp(const SceneView& S, const Ray& ray, const TraceParams& P, WarpMarch& st,
-                                           int32_t* ids, int max_ids, WarpRayScratch& ws) {
+// All rounds of the warp's ray, which can_hit.
+__device__ __forceinline__ bool march_warp(const SceneView& S, const Ray& ray, const RayBox& rb, const TraceParams& P,
+                                           WarpMarch& st, int32_t* ids, int max_ids, WarpRayScratch& ws) {
     const int lane = threadIdx.x & 31;
     st.init();
     if (S.n == 0) return true;
-    const RayBox rb = make_ray_box(ray);
     uint64_t last_key = depth_key(P.t_min, 0.f);
     int32_t last_u = INT32_MAX;
     bool ok = true;
