@@ -16,10 +16,13 @@ constexpr uint32_t kErrStackOverflow = 1u;   // a ray's traversal stack overflow
 constexpr uint32_t kErrBadTree = 2u;         // the hierarchy failed a consistency bound
 constexpr uint32_t kErrBadHitList = 4u;      // a saved hit list held an index outside the scene
 
-// Traversal stack depth. Karras trees over 30-bit keys with index tie-breaks
-// are at most 30 + 31 levels deep; the stack holds deferred siblings only (64
-// of them, and room for the up to three a node adds at once).
-constexpr int kStackSize = 67;
+// Traversal stack of a ray walking on its own: siblings deferred on one path, of
+// which a node adds up to three at once; the most recent one is kept in a
+// register. Trees are at most 61 levels deep (Karras: 30 key bits and 31 of the
+// index) or 60 (clustering), and a path of that length that defers more than one
+// sibling per level all the way takes a contrived scene; beyond 67 deferred ones
+// the walk may end with kErrStackOverflow.
+constexpr int kStackSize = 70;
 
 // Child id encoding in a node: >= 0 internal node, < 0 leaf (~m, m = Morton
 // index of the surfel), kNoChild = absent.

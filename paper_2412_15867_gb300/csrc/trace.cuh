@@ -684,7 +684,7 @@ __device__ __forceinline__ void bitonic_step(uint32_t& key, int32_t& m, int step
 // staged in shared memory, where every ray tests every one; the rest waits for
 // the next batch, so that hits come nearly in order (shifts in the k-buffer are
 // most of the cost: 1.39 ms for an 800 x 800 view without the waiting ones,
-// 1.37 with). Returns 0, or 1 if the stack overflowed, or 2 if
+// 1.37 with). Returns 0, or 1 if the hierarchy is broken, or 2 if
 // the packet gave up (nothing is kept then; the caller walks per ray).
 template <class KB, bool STATS = false>
 __device__ __forceinline__ int collect_packet(const SceneView& S, const Ray& ray, const TraceParams& P,
@@ -742,7 +742,7 @@ __device__ __forceinline__ int collect_packet(const SceneView& S, const Ray& ray
                 deeper += to > td || (to == td && (lane ^ x) > lane) ? 1 : 0;
             }
             if (sp + __popc(push) > kPacketStack || visits < 0) {
-                status = 1;
+                status = visits < 0 ? 1 : 2;   // no room: the rays' own stacks hold less
                 break;
             }
             __syncwarp();   // the popped entries have been read
