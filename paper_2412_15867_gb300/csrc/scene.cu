@@ -359,8 +359,13 @@ __global__ void __launch_bounds__(256) k_pack(int32_t* __restrict__ perm, uint32
     float* B = leaf_box + 6 * j;
     for (int k = 0; k < 3; ++k) {
         const double m = ok ? (double)muf[k] : 0.0;
-        const float a = su * (float)tu[k], b = sv * (float)tv[k];
-        double e = (double)(rc * sqrtf(a * a + b * b)) * (1.0 + 1e-5) + 1e-6 * (1.0 + fabs(m));
+        const float a = su * (float)tu[k], b = sv * (float)tv[k], q = a * a + b * b;
+        double e = rc * sqrtf(q);
+        if (!(q < INFINITY)) {   // discs of 2^64 and more: the longer leg times a root of [1, 2]
+            const float leg = fmaxf(fabsf(a), fabsf(b)), r = fminf(fabsf(a), fabsf(b)) / leg;
+            e = (double)leg * (double)(rc * sqrtf(fmaf(r, r, 1.f)));
+        }
+        e = e * (1.0 + 1e-5) + 1e-6 * (1.0 + fabs(m));
         if (rc2 < 0.0) e = 0.0;   // never hit: a point box at the centre
         B[k] = __double2float_rd(m - e);
         B[3 + k] = __double2float_ru(m + e);
