@@ -992,8 +992,8 @@ __device__ __forceinline__ void node_child(const Node& nd, int s, int32_t& c, fl
 
 // K5, greedy form: wide nodes are made top-down, level by level. A wide node
 // starts from the two children of its binary node and repeatedly replaces the
-// internal child of largest box surface area by that child's two children,
-// until it has four (or only leaves). Its internal children get new wide
+// internal child of largest box surface area (one that is NaN counts as such) by
+// that child's two children, until it has four (or only leaves). Its internal children get new wide
 // indices, so a level's nodes are the range of indices the level before
 // allocated; source[w] is the binary node behind wide node w. counters: the
 // number of nodes each level allocates (zero before the launch).
@@ -1062,7 +1062,7 @@ __global__ void __launch_bounds__(kCoopThreads, 1) k_wide(const Node* __restrict
                     for (int k = 0; k < grown; ++k)
                         if (k < m && cid[k] >= 0) {
                             const float a = box_area(box[k]);
-                            if (a > ba) {
+                            if (!(a <= ba)) {
                                 ba = a;
                                 best = k;
                             }
@@ -1416,8 +1416,9 @@ irgs_status build_scene_impl(const irgs_surfels* s, float alpha_min, uint32_t bu
     A(dalloc(&sc->leaf_parent, n, B));
     A(dalloc(&sc->node_parent, nn, B));
     A(dalloc(&sc->refit_flag, nn, B));
-    // every wide node takes at least one binary internal node
-    sc->max_wide = nn + 1;
+    // Every wide node has four children, or two or three leaves: with p of the
+    // latter among W, 4 (W - p) + 2 p <= W - 1 + n, and p <= n / 2.
+    sc->max_wide = n > 1 ? (2 * n - 1) / 3 : 1;
     A(dalloc(&sc->wide, sc->max_wide, B));
     A(dalloc(&sc->child_box, 8 * sc->max_wide, B));
     A(dalloc(&sc->wide_source, sc->max_wide, B));
