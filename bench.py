@@ -173,7 +173,10 @@ class ClockSampler:
                 "samples": len(rows), "reasons": sorted(reasons)}
 
 
-def algorithmic_flops(nh, k, n_surfels, F, backward=False, saved_hits=0):
+BUFFER = 32   # hits that the kernels' k-buffer holds, whatever k a call names
+
+
+def algorithmic_flops(nh, n_surfels, F, backward=False, saved_hits=0):
     """Algorithmic FP32 flops of one launch: per composited hit one Eq. 6-7
     intersection (45, exp counted as 1) plus blending (2(F+2) + 3); per
     k-buffer round one root-to-leaf descent of ceil(log2 N) nodes with two
@@ -181,7 +184,7 @@ def algorithmic_flops(nh, k, n_surfels, F, backward=False, saved_hits=0):
     for rays whose hit list was not saved (n_hits > saved_hits)."""
     import torch
     nh = nh.to(torch.float64)
-    rounds = torch.floor(nh / k) + 1
+    rounds = torch.floor(nh / BUFFER) + 1
     per_hit = 45 + 2 * (F + 2) + 3
     depth = math.ceil(math.log2(max(n_surfels, 2)))
     if backward and saved_hits > 0:
@@ -202,9 +205,9 @@ def trace_bytes(R, N, fc, backward=False):
     return float(b)
 
 
-def per_ray_flops(nh, k, n_surfels, F, backward=False, saved_hits=0):
+def per_ray_flops(nh, n_surfels, F, backward=False, saved_hits=0):
     """Mean algorithmic flops per ray of a sample of per-ray hit counts."""
-    return algorithmic_flops(nh, k, n_surfels, F, backward=backward, saved_hits=saved_hits) / max(nh.numel(), 1)
+    return algorithmic_flops(nh, n_surfels, F, backward=backward, saved_hits=saved_hits) / max(nh.numel(), 1)
 
 
 def roof_entry(ms, rays, flops, nbytes, peak_tflops, hbm_gbs, **extra):
@@ -416,13 +419,13 @@ def run_ours(args):
     nh = out["n_hits"]
     if bwd_ms >= fwd_ms:
         kname, kms = "k_trace_backward<10>", bwd_ms
-        flops = algorithmic_flops(nh, 16, sc.n, F, backward=True, saved_hits=args.saved_hits)
+        flops = algorithmic_flops(nh, sc.n, F, backward=True, saved_hits=args.saved_hits)
         src = ["trace.cuh", "trace_warp.cuh", "trace_bwd.cuh", "trace_bwd.cu", "common.cuh", "scene.cu"]
     else:
         # the forward pass: for batches of 2^20 rays or more its compacted
         # k-buffer rounds and the compaction between them
         kname, kms = "k_trace_round<10,*>", fwd_ms
-        flops = algorithmic_flops(nh, 16, sc.n, F)
+        flops = algorithmic_flops(nh, sc.n, F)
         src = ["trace.cuh", "trace_warp.cuh", "trace_fwd.cu", "common.cuh", "scene.cu"]
     achieved = flops / (kms * 1e-3) / 1e12
     khash = _kernel_hash(src)
@@ -436,18 +439,19 @@ def run_ours(args):
     R1 = args.res * args.res
     ws = irgs.trace_stats(scene, ro[:R1], rd[:R1], p).double().mean(0).tolist()
     nh1 = float(nh[:R1].double().mean())
-    # per node visit: 4 child slab tests (6 FMA, 6 min/max, 2 three-way) ~ 20
-    # flops each; per surfel test 45; per composited hit the blend
-    work_flops_ray = ws[1] * 4 * 20 + ws[2] * 45 + nh1 * (2 * (F + 2) + 3)
+    # per node visit: 4 child tests of ~ 20 flops, made once for the 32 rays of a
+    # packet (the counter has the packet's visits for each of them); per surfel
+    # test 45; per composited hit the blend
+    work_flops_ray = ws[1] * 4 * 20 / 32 + ws[2] * 45 + nh1 * (2 * (F + 2) + 3)
     alg_flops_ray = flops / R
     work = {"sample": f"camera 0 ({R1} rays)", "rounds_per_ray": ws[0], "nodes_per_ray": ws[1],
             "candidates_per_ray": ws[2], "inserts_per_ray": ws[3], "hits_per_ray": nh1,
             "algorithmic_flops_per_ray": alg_flops_ray, "work_flops_per_ray": work_flops_ray,
             "work_over_algorithmic": work_flops_ray / alg_flops_ray,
             "work_frac": work_flops_ray * R / (kms * 1e-3) / 1e12 / peak,
-            "note": "work_frac = the counted work (4 x 20 flops per node visit, 45 per surfel test, the blend per "
-                    "hit) per second over the FP32 peak: how busy the FP32 pipe would be if every counted test "
-                    "were needed; frac / work_frac = algorithmic / counted work"}
+            "note": "counted on a march with a 16-entry k-buffer, half of the timed kernels' (more rounds, so more "
+                    "tests than theirs); work_frac = the counted work (4 x 20 flops per node visit of a packet of 32 "
+                    "rays, 45 per surfel test, the blend per hit) per second over the FP32 peak"}
     roofline = {"bound": "alu", "kernel": kname, "achieved": achieved, "peak": peak,
                 "unit": "TFLOP/s", "frac": achieved / peak, "traffic": traffic,
                 "flops_per_launch": flops, "launch_ms": kms, "peak_note": peak_note,
@@ -461,14 +465,14 @@ def run_ours(args):
     bf = trace_bytes(R, sc.n, F)
     configs["C1"] = {
         "workload": WORKLOAD,
-        "fwd": roof_entry(fwd_ms, R, algorithmic_flops(nh, 16, sc.n, F), bf, peak, hbm),
+        "fwd": roof_entry(fwd_ms, R, algorithmic_flops(nh, sc.n, F), bf, peak, hbm),
         "fwd_bwd": roof_entry(fwd_ms + bwd_ms, R,
-                              algorithmic_flops(nh, 16, sc.n, F)
-                              + algorithmic_flops(nh, 16, sc.n, F, backward=True, saved_hits=args.saved_hits),
+                              algorithmic_flops(nh, sc.n, F)
+                              + algorithmic_flops(nh, sc.n, F, backward=True, saved_hits=args.saved_hits),
                               bf + trace_bytes(R, sc.n, F, backward=True), peak, hbm),
         "step": roof_entry(ms_per_step, R,
-                           algorithmic_flops(nh, 16, sc.n, F)
-                           + algorithmic_flops(nh, 16, sc.n, F, backward=True, saved_hits=args.saved_hits),
+                           algorithmic_flops(nh, sc.n, F)
+                           + algorithmic_flops(nh, sc.n, F, backward=True, saved_hits=args.saved_hits),
                            bf + trace_bytes(R, sc.n, F, backward=True), peak, hbm,
                            note="the timed step: rebuild + forward + backward")}
 
@@ -683,9 +687,9 @@ def mc_leg(args, dev, peak, hbm, cpu=True):
     nh_rl = irgs.trace_forward(S2, xs[vr].contiguous(), drl[vr].contiguous(), pr)["n_hits"]
     torch.cuda.synchronize()
     vfrac, vfrac_rl = float(vm.float().mean()), float(vr.float().mean())
-    f_fwd = per_ray_flops(nh_sh, 16, N2, 3)
-    f_bwd = per_ray_flops(nh_sh, 16, N2, 3, backward=True, saved_hits=64)
-    f_rl = per_ray_flops(nh_rl, 16, N2, 7)
+    f_fwd = per_ray_flops(nh_sh, N2, 3)
+    f_bwd = per_ray_flops(nh_sh, N2, 3, backward=True, saved_hits=64)
+    f_rl = per_ray_flops(nh_rl, N2, 7)
     SAMPLE_FLOPS = 150          # direction, BRDF and estimator terms per sample
     env_b = 512 * 256 * 3 * 4
     scene_b = lambda fc: N2 * (64 + 4 * fc) + (N2 - 1) * 64
@@ -713,7 +717,7 @@ def mc_leg(args, dev, peak, hbm, cpu=True):
                         f"{rays / 1e6:.1f}M secondary rays, 512x256 env, k=16",
             "ms": fms, "mrays_s": rays / (fms * 1e-3) / 1e6, "points_per_s": Pn / (fms * 1e-3),
             "bwd_ms": bms, "bwd_mrays_s": rays / (bms * 1e-3) / 1e6,
-            "path": "secondary rays regrouped by direction bin and origin Morton code, one stack per ray",
+            "path": "secondary rays regrouped by direction bin and origin Morton code, a lane per ray from pools of 64",
             "fused_per_lane_ms": fused_ms,
             "relight": {"workload": f"{Pn} points x 64 environment-importance samples, 512x256 environment, "
                                     "traced albedo/roughness/normal shaded with split-sum maps",
@@ -761,8 +765,8 @@ def tiny_leg(args, dev, peak, hbm):
     f_ms = ev[0].elapsed_time(ev[1]) / reps
     fb_ms = ev[1].elapsed_time(ev[2]) / reps
     nh = out["n_hits"]
-    ff = algorithmic_flops(nh, 8, sc.n, 3)
-    fbk = algorithmic_flops(nh, 8, sc.n, 3, backward=True)
+    ff = algorithmic_flops(nh, sc.n, 3)
+    fbk = algorithmic_flops(nh, sc.n, 3, backward=True)
     res = {"workload": "1,024 surfels (centres U[-1,1]^3), one 64x64 camera = 4,096 rays, k=8, 3 channels",
            "fwd": roof_entry(f_ms, R, ff, trace_bytes(R, sc.n, 3), peak, hbm,
                              note="one launch per call; launch-bound at this size"),

@@ -69,7 +69,9 @@ typedef struct {
 
 /* Parameters of one trace (Eq. 2, 6-8 and the termination rule of Sec. 4). */
 typedef struct {
-    int32_t k;            /* k-buffer size: 1, 4, 8, 16 or 32 (8 and 16 everywhere) */
+    int32_t k;            /* k-buffer size: 1, 4, 8, 16 or 32 (8 and 16 everywhere);
+                             results do not depend on it, and it selects no code:
+                             the buffer holds 32 entries                        */
     float alpha_min;      /* hits need alpha >= alpha_min; >= the scene's value     */
     float alpha_max;      /* alpha = min(alpha_max, o exp(-rho^2/2)), <= 1          */
     float T_min;          /* stop after the hit that makes T < T_min, in [0, 1)     */
@@ -80,7 +82,8 @@ typedef struct {
     uint32_t flags;       /* IRGS_FLAG_* bits, 0 for the defaults                   */
 } irgs_trace_params;
 
-/* Traversal policy (results are identical either way, only speed differs).
+/* Traversal policy: traces are identical either way, shading estimates up to
+ * the rounding of a sample's terms; only speed differs.
  * Default for irgs_trace_forward / irgs_trace_backward: up to 2^18 rays, a
  * warp per ray; larger batches as packets -- the 32 rays of a warp walk the
  * hierarchy together where they run together (pixel rows are cut into tiles
@@ -249,11 +252,12 @@ irgs_status irgs_trace_forward(irgs_scene scene, const float* ray_o, const float
                                void* stream);
 
 /*
- * Diagnostic: the forward march of irgs_trace_forward (k = 16, feat_count
- * <= 10, same traversal policy flags) with per-ray counters instead of
- * outputs. out_stats [n_rays, 4] int32: k-buffer rounds, BVH nodes fetched
- * (in the warp-coherent walk: fetched by the warp while this ray was still
- * marching), surfel tests, k-buffer insertions.
+ * Diagnostic: a forward march (k = 16, feat_count <= 10; packets by default,
+ * IRGS_FLAG_PER_THREAD a stack per ray) with a k-buffer of 16 entries, half
+ * of irgs_trace_forward's, and per-ray counters instead of outputs.
+ * out_stats [n_rays, 4] int32: k-buffer rounds, BVH nodes fetched (by a
+ * packet: once for all its rays, while this one was still marching), surfel
+ * tests, k-buffer insertions.
  */
 irgs_status irgs_trace_stats(irgs_scene scene, const float* ray_o, const float* ray_d, int64_t n_rays,
                              const irgs_trace_params* params, int32_t* out_stats, void* stream);

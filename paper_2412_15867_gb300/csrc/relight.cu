@@ -602,8 +602,8 @@ __global__ void __launch_bounds__(kRelightThreads) k_relight(SceneView S, EnvMap
 }
 
 // Wavefront form: samples generated one thread each, regrouped by direction
-// bin and origin, traced in that order with one stack per ray, then
-// estimated per point from the stored traces with the same per-sample
+// bin and origin, traced in that order (a warp per ray, in the largest batches
+// a lane), then estimated per point from the stored traces with the same per-sample
 // arithmetic and reduction order as k_relight.
 __global__ void k_relight_gen(EnvMaps M, const float* __restrict__ xg, int64_t p0, int64_t rays, int Sn,
                               uint64_t seed, const uint32_t* __restrict__ bounds, float4* __restrict__ dir,
@@ -656,8 +656,12 @@ __global__ void __launch_bounds__(kRelightThreads, kRayBlocks) k_relight_trace(S
 }
 
 // The same with a warp per ray, for batches that do not fill the chip many
-// times over with a ray per lane: 24.7 ms against 27.5 at 6.4M rays (the lines
-// are those of shading's batches, whose rays are the same kind).
+// times over with a ray per lane (the lines are shading's, shade_wave.cu). ms
+// for scenes of 100k / 300k / 1M / 3M surfels, a warp per ray first:
+//   0.26M rays   1.45 1.47 1.58 1.76    2.42 2.50 3.11 3.77
+//   4.2M         21.4 21.7 22.4 24.1    22.7 24.1 27.4 33.7
+//   8.4M         45.1 45.9 47.3 49.9    45.9 47.9 55.7 67.8
+//   16.8M        73.5 73.8 74.6 76.8    70.9 72.1 81.3 93.9
 constexpr int64_t kRelightUnsortedMax = int64_t(1) << 19;   // smaller batches gain less from the order than its sort costs
 constexpr int64_t kRelightWarpMax = int64_t(1) << 23;
 __global__ void __launch_bounds__(kWarpRayThreads, kWarpRayBlocks) k_relight_trace_ray(SceneView S, TraceParams P, RelightJob job,

@@ -1449,8 +1449,8 @@ irgs_status update_scene_impl(irgs_scene sc, const irgs_surfels* s, cudaStream_t
 // Refit: new surfel values in the Morton order and hierarchy of the last
 // build. Records, leaf boxes and features are recomputed and gathered with
 // the kept permutation, the binary boxes are refitted bottom-up and the
-// 4-wide nodes re-emitted from them (their layout depends only on the
-// topology). Every box still bounds its subtree, so traces stay exact; only
+// 4-wide nodes made from them again (the collapse opens children by box area,
+// so their layout follows the new boxes). Every box still bounds its subtree, so traces stay exact; only
 // the quality of the tree can degrade as surfels move.
 irgs_status refit_scene_impl(irgs_scene sc, const irgs_surfels* s, cudaStream_t st) {
     const int64_t n = sc->n;

@@ -214,7 +214,7 @@ irgs_status launch_shade_mc_backward(const SceneView& sv, const int32_t* perm, c
                                      float* g_albedo, float* g_rough, float* g_env, float* g_means, float* g_quats,
                                      float* g_scales, float* g_opacity, float* g_features, cudaStream_t st);
 
-// k-buffer sizes that are compiled in
+// k-buffer sizes that callers may name (they select no code: the buffer holds kCap entries)
 inline bool k_supported(int k) { return k == 1 || k == 4 || k == 8 || k == 16 || k == 32; }
 
 }  // namespace irgs

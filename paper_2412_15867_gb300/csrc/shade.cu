@@ -9,10 +9,12 @@
 //
 // One warp shades one point: lanes take samples s = lane, lane + 32, ... and
 // the per-point sums are reduced with a fixed butterfly, so a point's result
-// depends only on (seed, point index, inputs), not on batching. The traced
-// rays of a point share their origin; by default each lane walks its own
-// stack (the directions spread over the hemisphere), IRGS_FLAG_WARP walks
-// one stack for the warp. Both give the same traces.
+// depends only on (seed, point index, inputs), not on batching. This is the
+// fused form, which a traversal flag selects (the default regroups the rays of
+// all points, shade_wave.cu): the traced rays of a point share their origin,
+// and with IRGS_FLAG_PER_THREAD each lane walks its own stack (the directions
+// spread over the hemisphere), with IRGS_FLAG_WARP those that run together
+// walk as a packet. All give the same traces.
 //
 // The gradient (k_shade_backward) holds the sample directions fixed: with
 // L = sum_p g_p . rgb_p and a sample's estimate term (w_a a_c + w_s) L_i,c,

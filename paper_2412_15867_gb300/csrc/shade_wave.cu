@@ -45,8 +45,14 @@ constexpr int kWaveSavedHits = 64;   // 12% of secondary rays blend more than 32
 constexpr int64_t kWaveUnsortedMax = int64_t(1) << 19;
 // Batches up to this size take a warp per ray, whose throughput does not depend
 // on the size; a ray per lane catches up only where the pools are refilled many
-// times: 120.5 ms against 105.8 at 41M rays, 24.7 against 27.5 at 6.4M
-// (relighting, the same walk).
+// times. ms for scenes of 100k / 300k / 1M / 3M surfels, a warp per ray first:
+//   0.26M rays   1.00 0.90 0.88 0.91    1.79 1.83 1.92 2.18
+//   4.2M         14.6 13.2 12.1 12.2    13.0 12.4 12.3 13.8
+//   8.4M         31.2 29.2 27.1 27.1    26.4 25.4 26.1 29.5
+//   16.8M        57.2 54.6 52.1 51.6    48.4 46.6 48.2 53.7
+//   41M          129.9 125.4 121.0 119.1    110.6 106.4 105.9 117.2
+// Shading breaks even at about 2^22 rays, relighting, whose rays meet twice as
+// many surfels, at 2^23 to 2^24 (relight.cu); the two share a line between.
 constexpr int64_t kWaveWarpMax = int64_t(1) << 23;
 constexpr int kWaveReplayBlocks = 152 * 4;   // blocks that share the few rays whose hit list did not fit
 

@@ -1,4 +1,5 @@
-// Forward trace kernel: one thread per ray, Trace(r_o, r_d) of IRGS Eq. 8.
+// Forward trace kernels, Trace(r_o, r_d) of IRGS Eq. 8: a warp per ray for small
+// batches, else packets of 32 rays that walk together, or a lane per ray.
 #include <cuda_runtime.h>
 
 #include "scene.h"
@@ -254,8 +255,9 @@ cudaError_t launch_f(const SceneView& S, const float* ro, const float* rd, int64
     return e;
 }
 
-// Diagnostic: the march with a k-buffer of 16 entries and per-ray counters
-// (<= 10 channels).
+// Diagnostic: the march with per-ray counters and a k-buffer of 16 entries (the
+// other calls' has kCap, so they need fewer rounds and fewer walks), <= 10
+// channels. A packet's node fetches count for each of its rays.
 template <bool PACKET>
 __global__ void __launch_bounds__(128) k_trace_stats(SceneView S, const float* __restrict__ ro,
                                                      const float* __restrict__ rd, int64_t R, TraceParams P,

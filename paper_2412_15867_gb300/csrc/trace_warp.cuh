@@ -4,8 +4,9 @@
 // each, and the longest ray of a batch ten times that). The 32 lanes test 8
 // nodes x 4 children, or 32 surfels, of the same ray at a time, and the
 // round's nearest hits are kept in order in registers, the i-th in lane i.
-// Bound by instruction issue (75% of the slots); 230 Mrays/s whatever the
-// batch's size. Half a warp per ray (two hits per lane) was 10% slower: its
+// Bound by instruction issue (75% of the slots), so the rate hardly depends on
+// the batch's size: 230 Mrays/s for camera rays, 260 for relighting's and 340
+// for shading's samples, which meet fewer surfels. Half a warp per ray (two hits per lane) was 10% slower: its
 // nodes and leaves come in smaller portions. Hits, order and blending
 // arithmetic are those of march_forward, so the results are the same.
 #pragma once
@@ -251,11 +252,18 @@ __device__ __forceinline__ bool march_warp(const SceneView& S, const Ray& ray, c
     return ok;
 }
 
-// Batches of caller's rays up to this size take a warp per ray: packets of camera rays are
-// twice as fast per ray (460 against 230 Mrays/s), but their warps are few and
-// a grazing one takes a millisecond, which a batch needs some 300k rays to
-// cover (196k camera rays of a 1M scene: 1.49 ms a warp per ray, 2.8 ms as
-// packets; 640k of a 300k scene: 2.6 and 1.39).
+// Batches of caller's rays up to this size take a warp per ray. Packets of
+// camera rays are faster per ray where a batch has many, but their warps are few
+// and the slowest of them takes a millisecond or more, longer the more surfels
+// there are, while a warp per ray takes little longer then. ms for one view, a
+// warp per ray against packets:
+//                100k surfels    300k           1M             3M
+//   256 x 256    0.29 / 0.70     0.30 / 1.17    0.33 / 2.07    0.36 / 3.25
+//   384 x 384    0.64 / 0.62     0.66 / 1.13    0.70 / 1.71    0.75 / 3.33
+//   512 x 512    1.11 / 0.67     1.14 / 1.03    1.22 / 1.72    1.30 / 3.17
+// Rays that do not run together gain at every size (2^18 random pixels of 300k
+// surfels 1.39 ms, one ray more 2.74, where they walk as lanes). The line lies
+// where views of 300k surfels break even.
 constexpr int64_t kWarpRayMax = int64_t(1) << 18;
 
 // Threads per block, and resident blocks per SM, of the kernels with a warp per
