@@ -70,10 +70,10 @@ def measured_peaks():
 # batches) scaled per ray; keyed by the hash of the sources it was measured
 # on, the hierarchy's builder included (null once they change).
 TRAFFIC = {
-    # the two rounds of one forward with hit lists: read 232.5, written 170.3 MB
-    "k_trace_round<10,*>": {"bytes_per_ray": 402.8e6 / 1.28e6, "src_hash": "fde6cd71804c"},
-    # the listed backward and the replays of long lists: read 385.7, written 28.3 MB
-    "k_trace_backward<10>": {"bytes_per_ray": 414.0e6 / 1.28e6, "src_hash": "d536dc799342"},
+    # the two rounds of one forward with hit lists: read 231.1, written 174.4 MB
+    "k_trace_round<10,*>": {"bytes_per_ray": 405.5e6 / 1.28e6, "src_hash": "28db210eb467"},
+    # the listed backward and the replays of long lists: read 399.8, written 26.9 MB
+    "k_trace_backward<10>": {"bytes_per_ray": 426.7e6 / 1.28e6, "src_hash": "d0cffa097f99"},
 }
 
 

@@ -4,8 +4,8 @@
 // each, and the longest ray of a batch ten times that). The 32 lanes test 8
 // nodes x 4 children, or 32 surfels, of the same ray at a time, and the
 // round's nearest hits are kept in order in registers, the i-th in lane i.
-// Bound by instruction issue (75% of the slots), so the rate hardly depends on
-// the batch's size: 230 Mrays/s for camera rays, 260 for relighting's and 340
+// Bound by instruction issue (80% of the slots), so the rate hardly depends on
+// the batch's size: 230 to 260 Mrays/s for camera rays, 260 for relighting's and 340
 // for shading's samples, which meet fewer surfels. Half a warp per ray (two hits per lane) was 10% slower: its
 // nodes and leaves come in smaller portions. Hits, order and blending
 // arithmetic are those of march_forward, so the results are the same.
