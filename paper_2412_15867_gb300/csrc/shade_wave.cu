@@ -100,11 +100,14 @@ struct WaveJob {
     int32_t* nh;
     int32_t* hit_ids;
     int max_ids;
+    // FINITE: rays that are not finite are dealt with here, for the kernel that must
+    // not walk them; asking costs the pools 0.4%.
+    template <bool FINITE = false>
     __device__ __forceinline__ bool load(int j, f3& o, f3& d) const {
         const int64_t i = order[j];
         const float4 d4 = dir[i];
-        if (!(d4.w > 0.f)) {   // every sample gets an entry, so no reader sees unwritten scratch
-            res[i] = make_float4(0.f, 0.f, 0.f, d4.w < 0.f ? 1.f : 0.f);
+        if (FINITE ? !(d4.w > 0.f) : d4.w == 0.f) {   // every sample gets an entry, so no reader sees unwritten scratch
+            res[i] = make_float4(0.f, 0.f, 0.f, FINITE && d4.w < 0.f ? 1.f : 0.f);
             if (SAVE) nh[i] = 0;
             return false;
         }
@@ -139,7 +142,7 @@ __global__ void __launch_bounds__(kWarpRayThreads, kWarpRayBlocks) k_wave_trace_
                                                                                 int rays) {
     const int j = blockIdx.x * kWarpRays + (threadIdx.x >> 5);
     f3 o, d;
-    if (j >= rays || !job.load(j, o, d)) return;
+    if (j >= rays || !job.template load<true>(j, o, d)) return;
     const Ray ray = make_ray(o, d);
     WarpMarch w;
     const bool ok = march_warp(S, ray, make_ray_box(ray), P, w, job.ids(j), job.max_ids, warp_ray_scratch());
