@@ -323,6 +323,7 @@ __global__ void k_map_sums(const float4* __restrict__ irr_part, const float4* __
     const bool is_irr = i < kI;
     const float4* p = is_irr ? irr_part + i : pref_part + (i - kI);
     float4 s = make_float4(0.f, 0.f, 0.f, 0.f), e = s;
+#pragma unroll 8
     for (int k = 0; k < (is_irr ? irr_slices : pref_slices); ++k) {
         const float4 v = p[(int64_t)k * (is_irr ? kI : kP)];
         carry_sum(s.x, e.x, v.x);
