@@ -66,7 +66,8 @@ __device__ __forceinline__ float texel_solid_angle(int H, int W, int row) {
 // outputs, all prefilter levels share a pair's geometry, and a warp whose
 // outputs (8 x 4 patches) all face away skips the weights.
 //
-// Bound by instruction issue: a thread's two outputs are one packed pair of
+// Bound by the FP32 pipe and the reciprocals' latency (issue active in 61% of
+// the cycles): a thread's two outputs are one packed pair of
 // FP32 lanes, which halves the arithmetic but for the reciprocals (one per output
 // and level). A slice is every so-many-th chunk of 128 texels, so that each sees
 // all of the sphere (contiguous ones face some tiles wholly and others not at
@@ -81,9 +82,9 @@ __device__ __forceinline__ float texel_solid_angle(int H, int W, int row) {
 // total falls with the square root of their number: 4e-8 rms relative at
 // 512 x 256 texels and 7e-8 at 2048 x 1024 (level 1: 7e-8 and 9e-8). A block-wide
 // tree per output left 9e-8 and 2e-7 (1.4e-7 and 1.7e-6), one accumulator per
-// slice 2e-7 and 1.2e-6 (3.5e-7 and 1e-5). The groups cost 5% of an
-// environment's time (512 x 256: 1.74 -> 1.87 ms; groups of 16 1.93, of 64
-// 1.84, but 1.2e-7 at 32 x 16 texels, where the tree had 1e-7).
+// slice 2e-7 and 1.2e-6 (3.5e-7 and 1e-5). With the tables' running sums the
+// groups take 7% of an environment's time (512 x 256: 1.74 -> 1.86 ms; groups of
+// 16 1.93, of 64 1.84, but 1.2e-7 at 32 x 16 texels, where the tree had 1e-7).
 constexpr int kMapThreads = 128;
 constexpr int kMapTexels = 2;      // output texels per thread
 constexpr int kMapGroup = 32;      // environment texels per accumulator
